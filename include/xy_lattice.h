@@ -248,21 +248,19 @@ int xy_set_coupling_schedule(xy_lattice* lat, int cfg, const int64_t* step_knots
                              const double* perp_scales, int n_knots);
 
 /* Temporal blocking of the batched stepper (the paper steps one time step
- * per pass; this is a property of the library).  Lattices with
- * 256 <= Lx <= 1024 (Lx a multiple of 128, Ly a multiple of 8) can advance two
- * BBK steps per launch: a thread block sweeps a band of H rows across the
- * lattice width, carrying the intermediate step in registers, so the state
- * crosses HBM once per two steps (8 bytes per site-update instead of 16); the
- * two bands' boundary rows of the intermediate step are computed twice.
- * States are bit-identical either way.  Two-step launches run only over
- * stretches of steps that record nothing, in batches of a multiple of four
- * steps, and only for shapes whose configurations all run the whole call.
+ * per pass; this is a property of the library).  Lattices with Lx <= 2048 that
+ * are not held whole in shared memory can advance two BBK steps per launch: a
+ * thread block sweeps a band of H rows across the lattice width, carrying the
+ * intermediate step in registers, so the state crosses HBM once per two steps
+ * (8 bytes per site-update instead of 16); the two bands' boundary rows of the
+ * intermediate step are computed twice.  States are bit-identical either way,
+ * and so are records: a step that records is the first step of its launch.  A
+ * run that ends between the two steps of a launch takes the first one only.
  *   kt = 0 (default): the autotuner times one and two steps per launch (and
- *          the band height H in {8, 16, 32, 64}) per lattice shape and keeps
- *          two only if at least 5 % faster per step;
+ *          the band height) per lattice shape and keeps the faster; small
+ *          batches, which it does not time, take two;
  *   kt = 1: one step per launch everywhere;
- *   kt = 2: two steps per launch wherever the shape allows (the tuner's
- *          fastest band height, else the largest of 32, 16, 8 dividing Ly).
+ *   kt = 2: two steps per launch wherever the shape allows.
  * XY_EINVAL for any other value. */
 int xy_set_temporal_blocking(xy_lattice* lat, int kt);
 

@@ -139,32 +139,55 @@ struct TuneCache {
 };
 TuneCache g_tune;
 
-// All strip-stepped lattices of one shape; H and the occupancy variant are
-// chosen by the autotuner.
+// All lattices of one shape stepped by the strip and band kernels.  Single steps
+// run the strip kernel where the shape allows it (strip_ok), else the band kernel;
+// pairs of steps and steps that record run the band kernel where the shape allows
+// that one (band_H > 0).  The autotuner chooses H and the occupancy variant of the
+// strip kernel, the band height, and whether steps are paired.
 struct StripGroup {
     int Lx, Ly;
     uint64_t seed;  // one noise key per group: the round keys become kernel parameters
-    int H;
-    int variant;
-    std::vector<int> cfgs;
+    bool strip_ok;
+    int H = 0;
+    int variant = 3;
+    std::vector<int> cfgs = {};
     int64_t n_lat = 0;
-    std::vector<StripTask> tasks;
+    std::vector<StripTask> tasks = {};
     StripTask* d_tasks = nullptr;
     size_t d_cap = 0;
-    int variant_rec = 0;  // occupancy variant of launches that record (0: derived from variant)
-    // two steps per launch (temporal blocking): band height chosen by the
-    // autotuner, 0 when one step per pass is faster or the shape does not fit
-    int b2_H = 0;
-    int b2_auto = 0;  // the tuner's choice (0: one step per pass)
-    int b2_var = 2;   // occupancy variant of the two-step kernel (2 or 3 blocks per SM)
-    int b2_best = 0;  // the fastest band height it timed, chosen or not
-    std::vector<BandTask> b2_tasks;
-    BandTask* d_b2_tasks = nullptr;
-    size_t d_b2_cap = 0;
+    int band_H = 0;
+    bool kt2_auto = true;  // the tuner's choice: steps in pairs
+    bool kt2 = true;       // the choice in force (xy_set_temporal_blocking)
+    std::vector<BandTask> band_tasks = {};
+    BandTask* d_band_tasks = nullptr;
+    size_t d_band_cap = 0;
+    int buf = 0;           // 0: the state is in buffers A, 1: in buffers B (within a call)
 };
 
-// Shapes the two-step band kernel takes: one warp per 128 columns, 2..8 warps.
-bool b2_shape(int Lx, int Ly) { return Lx >= 256 && Lx <= 1024 && Lx % 128 == 0 && Ly >= 8 && Ly % 8 == 0; }
+// Blocks of band tasks per lattice for bands of H rows.
+int band_blocks(int Lx, int Ly, int H)
+{
+    const int nb = (Ly + H - 1) / H, per = bands_per_block(Lx);
+    return (nb + per - 1) / per;
+}
+
+// Band heights near h: the bands of a lattice made as even as its rows allow.
+int even_band(int Ly, int h)
+{
+    const int nb = (Ly + h - 1) / h;
+    return (Ly + nb - 1) / nb;
+}
+
+// Default band height: the tallest that still gives `min_warps` warps over the
+// lattices of the shape (a warp walks its rows one after the other; taller bands
+// recompute fewer halo rows).
+int default_band_H(int Lx, int Ly, int64_t n_lat, int64_t min_warps)
+{
+    const int warps = Lx > 128 ? (Lx + 127) / 128 : kNarrowBandWarps;
+    for (int h : {64, 32, 16, 8})
+        if (n_lat * band_blocks(Lx, Ly, h) * warps >= min_warps) return even_band(Ly, h);
+    return even_band(Ly, 4);
+}
 
 bool is_device_ptr(const void* p)
 {
@@ -240,17 +263,16 @@ struct xy_lattice {
     struct Graph {
         int chunk;
         int rec;
-        uint32_t rec_mask;
-        uint32_t kt2;
-        std::vector<uint8_t> sched;  // sched_flags() at capture: the strip kernels chosen by schedule presence
+        uint64_t rec_mask;
+        std::vector<uint8_t> groups;  // group_flags() at capture
         cudaGraphExec_t exec;
         int64_t kernels;
     };
     std::vector<Graph> graphs;  // captured chunks, by chunk length and recording
     int cur_rec = 0;            // records of the current window: 0 none, 1 M, 2 M and E
     int cur_re = 0;             // its record_every
-    uint32_t cur_mask = ~0u;    // local steps of a chunk at which some strip-stepped lattice records
-    uint32_t cur_kt2 = 0u;      // strip groups that take two steps per launch in this window
+    uint64_t cur_mask = 0;      // local steps of a chunk at which some strip-stepped lattice records
+    std::vector<uint8_t> in_b;  // per configuration: its state ended the call in buffers B
     int kt_mode = 0;            // xy_set_temporal_blocking: 0 tuner, 1 one step, 2 two steps per launch
     // kernel timing (direct launches bracketed by events)
     bool timing = false;
@@ -487,26 +509,51 @@ bool any_sched(const xy_lattice* L, const std::vector<int>& cfgs)
 }
 bool group_sched(const xy_lattice* L, const StripGroup& g) { return any_sched(L, g.cfgs); }
 
-// Entry g: strip group g has a schedule (part of a captured chunk's key).
-std::vector<uint8_t> sched_flags(const xy_lattice* L)
+// Entry g: what a captured chunk fixes of strip group g besides its steps (the
+// kernels chosen by schedule presence, the pairing and the buffers it starts from).
+std::vector<uint8_t> group_flags(const xy_lattice* L)
 {
     std::vector<uint8_t> f(L->strip_groups.size());
-    for (size_t g = 0; g < f.size(); ++g) f[g] = group_sched(L, L->strip_groups[g]) ? 1 : 0;
+    for (size_t g = 0; g < f.size(); ++g) {
+        const StripGroup& sg = L->strip_groups[g];
+        f[g] = (uint8_t)((group_sched(L, sg) ? 1 : 0) | (sg.kt2 ? 2 : 0) | (sg.buf ? 4 : 0));
+    }
     return f;
 }
 
-// Whether strip group g takes the local steps [jl0, jl0 + cnt) two per launch:
-// the window allows it (cur_kt2: every configuration of the group runs the
-// whole window), none of the steps records, and the batch holds an even number
-// of pairs, so that after it the state is where single steps would leave it.
-bool kt2_batch(const xy_lattice* L, int g, int64_t jl0, int cnt)
+// The launches of a strip group over `cnt` local steps: pairs of steps where the
+// group pairs them and the second one does not record (a launch sums records of
+// its first step), single steps elsewhere.
+struct StepRun {
+    int off, n, rec;
+};
+std::vector<StepRun> step_plan(const xy_lattice* L, const StripGroup& g, int cnt)
 {
-    // (groups past the 32 bits of cur_kt2 always take one step per launch)
-    if (g >= 32 || !((L->cur_kt2 >> g) & 1u) || cnt % 4 != 0 || L->strip_groups[g].b2_H == 0) return false;
-    if (L->cur_rec)
-        for (int i = 0; i < cnt; ++i)
-            if ((L->cur_mask >> ((jl0 + i) & 31)) & 1u) return false;
-    return true;
+    std::vector<StepRun> out;
+    auto rec_at = [&](int i) { return L->cur_rec && ((L->cur_mask >> (i & 63)) & 1u) ? L->cur_rec : 0; };
+    for (int i = 0; i < cnt;) {
+        const int n = g.kt2 && g.band_H > 0 && i + 1 < cnt && !rec_at(i + 1) ? 2 : 1;
+        out.push_back(StepRun{i, n, rec_at(i)});
+        i += n;
+    }
+    return out;
+}
+
+// One launch of a strip group: lattices [lat0, lat0 + n_lat) of it.
+cudaError_t launch_group(xy_lattice* L, cudaStream_t st, StripGroup& g, int64_t lat0, int64_t n_lat, const StepRun& r,
+                         int64_t jl0, int rd_b, Buffers buf)
+{
+    ++L->launches;
+    // (when every step records nothing pairs: the strip kernel has no halo rows)
+    const bool strip = g.strip_ok && (!r.rec || L->cur_re == 1);
+    if (g.band_H > 0 && (r.n == 2 || !strip)) {
+        const int64_t per = (int64_t)g.band_tasks.size() / g.n_lat;
+        return launch_band_step(L->d_cfg, g.d_band_tasks + lat0 * per, (int)(n_lat * per), g.Lx, g.band_H, r.rec,
+                                group_sched(L, g), r.n, rd_b != 0, g.seed, jl0 + r.off, buf, L->d_call, L->pa, st);
+    }
+    const int64_t per = (int64_t)g.tasks.size() / g.n_lat;
+    return launch_strip_step(L->d_cfg, g.d_tasks + lat0 * per, (int)(n_lat * per), g.H, g.variant, r.rec,
+                             group_sched(L, g), rd_b != 0, g.seed, jl0 + r.off, buf, L->d_call, L->pa, st);
 }
 
 // Launch the batched kernels for local steps [jl0, jl0 + cnt) of the current window.
@@ -522,38 +569,46 @@ int launch_batched_steps(xy_lattice* L, cudaStream_t st, int64_t jl0, int cnt, b
         if ((rc = timed_end(end, st))) return rc;
         ++L->launches;
     }
-    for (int i = 0; i < cnt; ++i) {
-        for (auto& g : L->strip_groups) {
-            if (kt2_batch(L, (int)(&g - L->strip_groups.data()), jl0, cnt)) {
-                if (i & 1) continue;  // the launch at step i took step i + 1 too
-                if ((rc = timed_begin(L, st, XY_KCLASS_STRIP2, &end))) return rc;
-                CK(launch_band2_step(L->d_cfg, g.d_b2_tasks, (int)g.b2_tasks.size(), g.Lx, g.b2_H, g.b2_var, g.seed,
-                                     jl0 + i, buf, L->d_call, st));
-                if ((rc = timed_end(end, st))) return rc;
-                ++L->launches;
-                continue;
-            }
-            if ((rc = timed_begin(L, st, XY_KCLASS_STRIP, &end))) return rc;
-            // only the steps that record run the recording kernel
-            const int rec = (L->cur_rec && ((L->cur_mask >> ((jl0 + i) & 31)) & 1u)) ? L->cur_rec : 0;
-            const int var = rec && g.variant_rec ? g.variant_rec : g.variant;
-            CK(launch_strip_step(L->d_cfg, g.d_tasks, (int)g.tasks.size(), g.H, var, rec, group_sched(L, g),
-                                 g.seed, jl0 + i, buf, L->d_call, L->pa, st));
+    for (auto& g : L->strip_groups) {
+        int rd = g.buf;
+        for (const StepRun& r : step_plan(L, g, cnt)) {
+            if ((rc = timed_begin(L, st, r.n == 2 ? XY_KCLASS_STRIP2 : XY_KCLASS_STRIP, &end))) return rc;
+            CK(launch_group(L, st, g, 0, g.n_lat, r, jl0, rd, buf));
             if ((rc = timed_end(end, st))) return rc;
-            ++L->launches;
+            rd ^= 1;
         }
+    }
+    for (int i = 0; i < cnt; ++i)
         for (int c : L->plain_cfgs) {
             if ((rc = timed_begin(L, st, XY_KCLASS_PLAIN, &end))) return rc;
             CK(launch_plain_step(L->d_cfg, L->h_dev[c], jl0 + i, buf, L->d_call, L->pa, 1, st));
             if ((rc = timed_end(end, st))) return rc;
             ++L->launches;
         }
-    }
     if (advance) {
         CK(launch_advance(L->d_call, cnt, st));
         ++L->launches;
     }
     return XY_OK;
+}
+
+// After a chunk of `cnt` steps that began at step `pos` of the call: every group's
+// buffers advance by its launches, and a configuration whose run ended within the
+// chunk keeps the buffers that the launch of its last step wrote.
+void account_chunk(xy_lattice* L, int64_t pos, int cnt)
+{
+    for (auto& g : L->strip_groups) {
+        int rd = g.buf;
+        for (const StepRun& r : step_plan(L, g, cnt)) {
+            rd ^= 1;
+            const int64_t lo = pos + r.off, hi = lo + r.n;
+            for (int c : g.cfgs) {
+                const int64_t n = L->h_dev[c].n_call;
+                if (n > lo && n <= hi) L->in_b[c] = (uint8_t)rd;
+            }
+        }
+        g.buf = rd;
+    }
 }
 
 // Concurrent slices of a set of kernel groups.  Lattices never read each
@@ -676,36 +731,31 @@ cudaError_t launch_sliced(xy_lattice* L, const std::vector<int>& cuts, int reps,
 struct Branch {
     int kind;  // 0 resident group, 1 strip group slice, 2 plain configurations
     int group;
-    int task0, n_tasks;
-    int b2_task0 = 0, b2_n_tasks = 0;  // the same lattices' tasks of the two-step kernel
+    int64_t lat0 = 0, n_lat = 0;  // lattices of the strip group
 };
 
-// Index of the first two-step task of the lattice that strip task t starts
-// (both task lists run lattice by lattice, every lattice of a group alike).
-int b2_index_of(const StripGroup& g, int t)
+// The first lattice of each slice of group g, cut where `parts` even shares of
+// its tasks fall, followed by its number of lattices.
+std::vector<int64_t> lattice_cuts(const StripGroup& g, int parts)
 {
-    if (g.b2_H == 0 || g.tasks.empty()) return 0;
-    if (t >= (int)g.tasks.size()) return (int)g.b2_tasks.size();
-    const int per_strip = (int)(g.tasks.size() / g.n_lat);
-    return (t / per_strip) * (g.Ly / g.b2_H);
+    const std::vector<int> cuts = g.strip_ok ? cut_tasks(g.tasks, parts) : cut_tasks(g.band_tasks, parts);
+    const int64_t per = (int64_t)(g.strip_ok ? g.tasks.size() : g.band_tasks.size()) / g.n_lat;
+    std::vector<int64_t> out;
+    for (int c : cuts) out.push_back(c / per);
+    return out;
 }
 
 std::vector<Branch> chunk_branches(const xy_lattice* L)
 {
     std::vector<Branch> out;
-    for (int r = 0; r < (int)L->res_groups.size(); ++r) out.push_back({0, r, 0, 0});
+    for (int r = 0; r < (int)L->res_groups.size(); ++r) out.push_back({0, r});
     const int fixed = (int)L->res_groups.size() + (L->plain_cfgs.empty() ? 0 : 1);
-    const auto cuts = slice_groups(L->strip_groups, fixed, xy_lattice::kBranches + 1);
+    const std::vector<int> parts = slice_parts(L->strip_groups, fixed, xy_lattice::kBranches + 1);
     for (int s = 0; s < (int)L->strip_groups.size(); ++s) {
-        const StripGroup& g = L->strip_groups[s];
-        for (size_t p = 0; p + 1 < cuts[s].size(); ++p) {
-            Branch b{1, s, cuts[s][p], cuts[s][p + 1] - cuts[s][p]};
-            b.b2_task0 = b2_index_of(g, cuts[s][p]);
-            b.b2_n_tasks = b2_index_of(g, cuts[s][p + 1]) - b.b2_task0;
-            out.push_back(b);
-        }
+        const std::vector<int64_t> cuts = lattice_cuts(L->strip_groups[s], parts[s]);
+        for (size_t p = 0; p + 1 < cuts.size(); ++p) out.push_back({1, s, cuts[p], cuts[p + 1] - cuts[p]});
     }
-    if (!L->plain_cfgs.empty()) out.push_back({2, 0, 0, 0});
+    if (!L->plain_cfgs.empty()) out.push_back({2, 0});
     return out;
 }
 
@@ -720,30 +770,31 @@ cudaError_t launch_branch(xy_lattice* L, cudaStream_t st, const Branch& br, int6
         ++L->launches;
         return e;
     }
-    const bool two = br.kind == 1 && kt2_batch(L, br.group, jl0, cnt);
-    for (int i = 0; i < cnt && e == cudaSuccess; ++i) {
-        if (two) {
-            if (i & 1) continue;
-            auto& g = L->strip_groups[br.group];
-            e = launch_band2_step(L->d_cfg, g.d_b2_tasks + br.b2_task0, br.b2_n_tasks, g.Lx, g.b2_H, g.b2_var, g.seed,
-                                  jl0 + i, buf, L->d_call, st);
-            ++L->launches;
-        } else if (br.kind == 1) {
-            auto& g = L->strip_groups[br.group];
-            const int rec = (L->cur_rec && ((L->cur_mask >> ((jl0 + i) & 31)) & 1u)) ? L->cur_rec : 0;
-            const int var = rec && g.variant_rec ? g.variant_rec : g.variant;
-            e = launch_strip_step(L->d_cfg, g.d_tasks + br.task0, br.n_tasks, g.H, var, rec, group_sched(L, g), g.seed,
-                                  jl0 + i, buf, L->d_call, L->pa, st);
-            ++L->launches;
-        } else {
-            for (int c : L->plain_cfgs) {
-                if (e != cudaSuccess) break;
-                e = launch_plain_step(L->d_cfg, L->h_dev[c], jl0 + i, buf, L->d_call, L->pa, 1, st);
-                ++L->launches;
-            }
+    if (br.kind == 1) {
+        auto& g = L->strip_groups[br.group];
+        int rd = g.buf;
+        for (const StepRun& r : step_plan(L, g, cnt)) {
+            if (e != cudaSuccess) break;
+            e = launch_group(L, st, g, br.lat0, br.n_lat, r, jl0, rd, buf);
+            rd ^= 1;
         }
+        return e;
     }
+    for (int i = 0; i < cnt && e == cudaSuccess; ++i)
+        for (int c : L->plain_cfgs) {
+            if (e != cudaSuccess) break;
+            e = launch_plain_step(L->d_cfg, L->h_dev[c], jl0 + i, buf, L->d_call, L->pa, 1, st);
+            ++L->launches;
+        }
     return e;
+}
+
+constexpr size_t kMaxGraphs = 64;
+
+void drop_graphs(xy_lattice* L)
+{
+    for (auto& g : L->graphs) cudaGraphExecDestroy(g.exec);
+    L->graphs.clear();
 }
 
 // Capture `chunk` batched steps (kernels + chunk counter) into a graph, or
@@ -753,13 +804,16 @@ cudaError_t launch_branch(xy_lattice* L, cudaStream_t st, const Branch& br, int6
 // idle as its launch drains) instead of taking turns every step.
 int get_graph(xy_lattice* L, int chunk, xy_lattice::Graph** out)
 {
-    const std::vector<uint8_t> sm = sched_flags(L);
+    const std::vector<uint8_t> gf = group_flags(L);
     for (auto& g : L->graphs)
-        if (g.chunk == chunk && g.rec == L->cur_rec && g.rec_mask == L->cur_mask && g.kt2 == L->cur_kt2 &&
-            g.sched == sm) {
+        if (g.chunk == chunk && g.rec == L->cur_rec && g.rec_mask == L->cur_mask && g.groups == gf) {
             *out = &g;
             return XY_OK;
         }
+    if (L->graphs.size() >= kMaxGraphs) {  // uneven record steps make many kinds of chunk: start afresh
+        CK(cudaStreamSynchronize(L->stream));
+        drop_graphs(L);
+    }
     const std::vector<Branch> brs = chunk_branches(L);
     const int nb = (int)brs.size();
     const bool fork = nb >= 2 && nb <= xy_lattice::kBranches + 1;
@@ -800,14 +854,14 @@ int get_graph(xy_lattice* L, int chunk, xy_lattice::Graph** out)
     e = cudaGraphInstantiate(&exec, g, 0);
     cudaGraphDestroy(g);
     if (e != cudaSuccess) return fail(XY_ECUDA, "graph instantiate: %s", cudaGetErrorString(e));
-    L->graphs.push_back({chunk, L->cur_rec, L->cur_mask, L->cur_kt2, sm, exec, kernels});
+    L->graphs.push_back({chunk, L->cur_rec, L->cur_mask, gf, exec, kernels});
     *out = &L->graphs.back();
     return XY_OK;
 }
 
 
 int build_strip_tasks(xy_lattice* L, StripGroup& g);
-int build_b2_tasks(xy_lattice* L, StripGroup& g, int H);
+int build_band_tasks(xy_lattice* L, StripGroup& g, int H);
 
 // ---- autotuner: per strip shape, time strip heights x occupancy variants;
 // per resident shape, time the block sizes.  Candidates run one step from
@@ -827,6 +881,11 @@ int time_window(xy_lattice* L, int64_t n_call)
     return upload_call(L, ca);
 }
 
+// First part of every key of the tuner's cache: the GPU and the generation of
+// the kernels.  Raised when a kernel changes enough that choices timed with the
+// old one no longer hold (a cache file outlives the library that wrote it).
+constexpr int kTuneGeneration = 2;
+
 std::string gpu_name()
 {
     int dev = 0;
@@ -838,41 +897,22 @@ std::string gpu_name()
     std::string s = p.name;
     for (auto& ch : s)
         if (ch == ' ' || ch == '|') ch = '_';
-    return s;
+    return s + "/" + std::to_string(kTuneGeneration);
 }
 
-// Band height of the two-step kernel per strip group under the current mode:
-// the tuner's choice, none, or (forced) the tuner's fastest height, else the
-// largest of 32, 16, 8 dividing Ly.
-int apply_kt_mode(xy_lattice* L)
+// Whether each strip group pairs its steps under the current mode: the tuner's
+// choice, never, or wherever the shape allows.
+void apply_kt_mode(xy_lattice* L)
 {
-    for (auto& g : L->strip_groups) {
-        int h = 0;
-        if (L->kt_mode == 0) h = g.b2_auto;
-        if (L->kt_mode == 2 && b2_shape(g.Lx, g.Ly)) {
-            h = g.b2_best;
-            for (int c : {32, 16, 8})
-                if (h == 0 && g.Ly % c == 0) h = c;
-        }
-        if (h == g.b2_H) continue;
-        g.b2_H = 0;
-        if (h > 0) {
-            int rc = build_b2_tasks(L, g, h);
-            if (rc) return rc;
-            g.b2_H = h;
-        } else {
-            for (auto& gr : L->graphs) cudaGraphExecDestroy(gr.exec);
-            L->graphs.clear();
-        }
-    }
-    return XY_OK;
+    for (auto& g : L->strip_groups) g.kt2 = g.band_H > 0 && (L->kt_mode == 0 ? g.kt2_auto : L->kt_mode == 2);
 }
 
 int autotune_lattice(xy_lattice* L)
 {
     if (L->tuned) return XY_OK;
     L->tuned = true;
-    if (!L->autotune) return apply_kt_mode(L);
+    apply_kt_mode(L);
+    if (!L->autotune) return XY_OK;
     const std::string gpu = gpu_name();
     cudaEvent_t e0, e1;
     CK(cudaEventCreate(&e0));
@@ -887,9 +927,26 @@ int autotune_lattice(xy_lattice* L)
         if (rc) break;
         if ((int64_t)g.Lx * g.Ly * g.n_lat < ((int64_t)1 << 21)) continue;  // too small to matter
         const int n_parts = parts[&g - L->strip_groups.data()];
-        char key[256];
-        snprintf(key, sizeof key, "%s|strip-sliced|%d|%d|%lld", gpu.c_str(), g.Lx, g.Ly, (long long)g.n_lat);
-        int bh = 0, bv = 0;
+        // milliseconds of one launch per slice: the best of 5 timings, each over
+        // enough launches to span about half a millisecond (single launches of a
+        // small batch differ by less than their timing noise)
+        auto time_it = [&](const std::vector<int>& cuts, auto&& run, float& out) -> int {
+            int reps = 3;
+            out = 1e30f;
+            for (int round = 0; round < 5; ++round) {
+                CK(launch_sliced(L, cuts, 1, run));
+                CK(cudaEventRecord(e0, L->stream));
+                CK(launch_sliced(L, cuts, reps, run));
+                CK(cudaEventRecord(e1, L->stream));
+                CK(cudaEventSynchronize(e1));
+                float ms = 0.f;
+                CK(cudaEventElapsedTime(&ms, e0, e1));
+                L->launches += (int64_t)(1 + reps) * ((int)cuts.size() - 1);
+                out = std::min(out, ms / reps);
+                if (round == 0 && ms < 0.5f) reps = std::min(64, (int)(0.5f / std::max(ms / reps, 1e-3f)) + 1);
+            }
+            return XY_OK;
+        };
         // a cached choice is used only if it satisfies the same constraints
         // as the candidates below (the cache is a plain text file)
         auto strip_ok = [&](int H, int v) {
@@ -897,47 +954,31 @@ int autotune_lattice(xy_lattice* L)
             return H >= 1 && H <= 64 && v >= 2 && v <= 4 && g.Ly % (H * groups) == 0 &&
                    (strip_units_per_lattice(g.Lx, g.Ly, H) + 7) / 8 <= L->pa.max_units;
         };
-        if (g_tune.get(key, &bh, &bv) && !strip_ok(bh, bv)) bh = bv = 0;
-        if (bh == 0) {
-            // per candidate: the best of 5 timings, each over enough launches
-            // to span about half a millisecond (single launches of a small
-            // batch differ by less than their timing noise)
+        char key[256];
+        snprintf(key, sizeof key, "%s|strip-sliced|%d|%d|%lld", gpu.c_str(), g.Lx, g.Ly, (long long)g.n_lat);
+        int bh = 0, bv = 0;
+        if (g.strip_ok && g_tune.get(key, &bh, &bv) && !strip_ok(bh, bv)) bh = bv = 0;
+        if (g.strip_ok && bh == 0) {
             float best = 1e30f;
             for (int H : {4, 8, 16, 32, 64}) {
-                const int groups = g.Lx >= 128 ? 1 : 32 / (g.Lx / 4);
-                if (g.Ly % (H * groups) != 0) continue;
-                // one record partial per block of 8 units
-                if ((strip_units_per_lattice(g.Lx, g.Ly, H) + 7) / 8 > L->pa.max_units) continue;
+                if (!strip_ok(H, 2)) continue;
                 g.H = H;
                 if ((rc = build_strip_tasks(L, g))) break;
                 const std::vector<int> cuts = cut_tasks(g.tasks, n_parts);
-                float t_best[3] = {1e30f, 1e30f, 1e30f};
-                int reps = 3;
-                for (int round = 0; round < 5; ++round)
-                    for (int vi = 0; vi < 3; ++vi) {
-                        const int v = 2 + vi;
-                        auto run = [&](cudaStream_t st, int t0, int cnt) {
-                            return launch_strip_step(L->d_cfg, g.d_tasks + t0, cnt, H, v, 0, group_sched(L, g), g.seed,
-                                                     0, buf, L->d_call, L->pa, st);
-                        };
-                        CK(launch_sliced(L, cuts, 1, run));
-                        CK(cudaEventRecord(e0, L->stream));
-                        CK(launch_sliced(L, cuts, reps, run));
-                        CK(cudaEventRecord(e1, L->stream));
-                        CK(cudaEventSynchronize(e1));
-                        float ms = 0.f;
-                        CK(cudaEventElapsedTime(&ms, e0, e1));
-                        L->launches += (int64_t)(1 + reps) * ((int)cuts.size() - 1);
-                        t_best[vi] = std::min(t_best[vi], ms / reps);
-                        if (round == 0 && vi == 0 && ms < 0.5f)
-                            reps = std::min(64, (int)(0.5f / std::max(ms / reps, 1e-3f)) + 1);
-                    }
-                for (int vi = 0; vi < 3; ++vi)
-                    if (t_best[vi] < best) {
-                        best = t_best[vi];
+                for (int v : {2, 3, 4}) {
+                    float t = 1e30f;
+                    rc = time_it(cuts, [&](cudaStream_t st, int t0, int cnt) {
+                        return launch_strip_step(L->d_cfg, g.d_tasks + t0, cnt, H, v, 0, group_sched(L, g), false, g.seed, 0,
+                                                 buf, L->d_call, L->pa, st);
+                    }, t);
+                    if (rc) break;
+                    if (t < best) {
+                        best = t;
                         bh = H;
-                        bv = 2 + vi;
+                        bv = v;
                     }
+                }
+                if (rc) break;
             }
             if (rc) break;
             if (bh > 0) g_tune.put(key, bh, bv);
@@ -946,135 +987,44 @@ int autotune_lattice(xy_lattice* L)
             g.H = bh;
             g.variant = bv;
             if ((rc = build_strip_tasks(L, g))) break;
-            // launches that record M (every step of the adjoint's recompute)
-            // carry more live registers: their own variant at this H, among
-            // those that do not spill
-            char keyr[256];
-            snprintf(keyr, sizeof keyr, "%s|striprec-sliced|%d|%d|%lld|%d", gpu.c_str(), g.Lx, g.Ly,
-                     (long long)g.n_lat, bh);
-            int rv = 0, unused = 0;
-            if (g_tune.get(keyr, &rv, &unused) && (rv < 2 || rv > 4)) rv = 0;
-            if (rv == 0) {
-                double2* scratch = nullptr;
-                CK(cudaMalloc(&scratch, sizeof(double2) * (size_t)L->B));
-                CallArgs ca{};
-                ca.fixed_parity = 1;
-                ca.record_every = 1;
-                ca.rec_dev = scratch;
-                ca.rec_stride = 1;
-                ca.m_only = 1;
-                if ((rc = upload_call(L, ca))) {
-                    cudaFree(scratch);
-                    break;
-                }
-                const std::vector<int> cuts = cut_tasks(g.tasks, n_parts);
-                float t_best[2] = {1e30f, 1e30f};
-                int reps = 3;
-                for (int round = 0; round < 5 && rc == XY_OK; ++round)
-                    for (int vi = 0; vi < 2; ++vi) {
-                        const int v = 2 + vi;
-                        auto run = [&](cudaStream_t st, int t0, int cnt) {
-                            return launch_strip_step(L->d_cfg, g.d_tasks + t0, cnt, bh, v, 1, group_sched(L, g),
-                                                     g.seed, 0, buf, L->d_call, L->pa, st);
-                        };
-                        cudaError_t e = launch_sliced(L, cuts, 1, run);
-                        if (e == cudaSuccess) e = cudaEventRecord(e0, L->stream);
-                        if (e == cudaSuccess) e = launch_sliced(L, cuts, reps, run);
-                        if (e == cudaSuccess) e = cudaEventRecord(e1, L->stream);
-                        if (e == cudaSuccess) e = cudaEventSynchronize(e1);
-                        float ms = 0.f;
-                        if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, e0, e1);
-                        if (e != cudaSuccess) {
-                            cudaGetLastError();
-                            rc = fail(XY_ECUDA, "autotune (recording launches): %s", cudaGetErrorString(e));
-                            break;
-                        }
-                        L->launches += (int64_t)(1 + reps) * ((int)cuts.size() - 1);
-                        t_best[vi] = std::min(t_best[vi], ms / reps);
-                        if (round == 0 && vi == 0 && ms < 0.5f)
-                            reps = std::min(64, (int)(0.5f / std::max(ms / reps, 1e-3f)) + 1);
-                    }
-                cudaStreamSynchronize(L->stream);
-                cudaFree(scratch);
-                if (rc) break;
-                rv = t_best[1] < t_best[0] ? 3 : 2;
-                g_tune.put(keyr, rv, 0);
-                CallArgs ca0{};
-                ca0.fixed_parity = 1;
-                if ((rc = upload_call(L, ca0))) break;
-            }
-            g.variant_rec = rv;
         }
-        // temporal blocking: two steps per launch on bands of H2 rows, timed
-        // against one step per pass as chosen above, sliced alike; kept only
-        // when at least 5 % faster per step
-        if (rc == XY_OK && bh > 0 && b2_shape(g.Lx, g.Ly)) {
-            char key2[256];
-            snprintf(key2, sizeof key2, "%s|band2-sliced|%d|%d|%lld", gpu.c_str(), g.Lx, g.Ly, (long long)g.n_lat);
-            int h2 = -1, unused = 0;
-            if (g_tune.get(key2, &h2, &unused) && !(h2 == 0 || (h2 >= 8 && h2 <= 64 && g.Ly % h2 == 0))) h2 = -1;
-            if (h2 < 0) {
-                const std::vector<int> cuts1 = cut_tasks(g.tasks, n_parts);
-                auto time_it = [&](const std::vector<int>& cuts, auto&& run, float& out) -> int {
-                    int reps = 3;
-                    out = 1e30f;
-                    for (int round = 0; round < 5; ++round) {
-                        CK(launch_sliced(L, cuts, 1, run));
-                        CK(cudaEventRecord(e0, L->stream));
-                        CK(launch_sliced(L, cuts, reps, run));
-                        CK(cudaEventRecord(e1, L->stream));
-                        CK(cudaEventSynchronize(e1));
-                        float ms = 0.f;
-                        CK(cudaEventElapsedTime(&ms, e0, e1));
-                        L->launches += (int64_t)(1 + reps) * ((int)cuts.size() - 1);
-                        out = std::min(out, ms / reps);
-                        if (round == 0 && ms < 0.5f) reps = std::min(64, (int)(0.5f / std::max(ms / reps, 1e-3f)) + 1);
-                    }
-                    return XY_OK;
-                };
-                float t1 = 1e30f;
-                rc = time_it(cuts1, [&](cudaStream_t st, int t0, int cnt) {
-                    return launch_strip_step(L->d_cfg, g.d_tasks + t0, cnt, g.H, g.variant, 0, group_sched(L, g),
+        if (g.band_H == 0) continue;
+        // temporal blocking: pairs of steps on bands of h rows, timed against
+        // single steps as chosen above, sliced alike
+        char key2[256];
+        snprintf(key2, sizeof key2, "%s|band-sliced|%d|%d|%lld", gpu.c_str(), g.Lx, g.Ly, (long long)g.n_lat);
+        int h2 = 0, pair = 0;
+        if (g_tune.get(key2, &h2, &pair) && !(h2 >= 4 && h2 <= 64 && (pair == 0 || pair == 1))) h2 = 0;
+        if (h2 == 0) {
+            float t1 = 1e30f, best2 = 1e30f;
+            if (g.strip_ok)
+                rc = time_it(cut_tasks(g.tasks, n_parts), [&](cudaStream_t st, int t0, int cnt) {
+                    return launch_strip_step(L->d_cfg, g.d_tasks + t0, cnt, g.H, g.variant, 0, group_sched(L, g), false,
                                              g.seed, 0, buf, L->d_call, L->pa, st);
                 }, t1);
-                float best2 = 1e30f;
-                int bestH = 0, bestV = 2;
-                for (int H2 : {8, 16, 32, 64}) {
-                    if (rc || g.Ly % H2 != 0) continue;
-                    if ((rc = build_b2_tasks(L, g, H2))) break;
-                    g.b2_H = H2;
-                    std::vector<int> cuts2;
-                    for (int c1 : cuts1) cuts2.push_back(b2_index_of(g, c1));
-                    for (int v2 : {2, 3}) {
-                        float t2 = 1e30f;
-                        rc = time_it(cuts2, [&](cudaStream_t st, int t0, int cnt) {
-                            return launch_band2_step(L->d_cfg, g.d_b2_tasks + t0, cnt, g.Lx, H2, v2, g.seed, 0, buf,
-                                                     L->d_call, st);
-                        }, t2);
-                        if (rc) break;
-                        if (t2 / 2 < best2) {
-                            best2 = t2 / 2;
-                            bestH = H2;
-                            bestV = v2;
-                        }
-                    }
-                }
-                g.b2_H = 0;
+            for (int h : {4, 8, 16, 32, 64}) {
+                if (rc || (h > 4 && h > g.Ly)) continue;
+                const int H = even_band(g.Ly, h);
+                if ((rc = build_band_tasks(L, g, H))) break;
+                float t2 = 1e30f;
+                rc = time_it(cut_tasks(g.band_tasks, n_parts), [&](cudaStream_t st, int t0, int cnt) {
+                    return launch_band_step(L->d_cfg, g.d_band_tasks + t0, cnt, g.Lx, H, 0, group_sched(L, g), 2, false,
+                                            g.seed, 0, buf, L->d_call, L->pa, st);
+                }, t2);
                 if (rc) break;
-                // a margin: isolated sliced timings overstate the two-step
-                // kernel's gain inside a mixed batch (512^2 lattices of the
-                // static-criticality batch: 2 % faster alone, 0.4 % slower in the batch)
-                h2 = best2 < 0.95f * t1 ? bestH : 0;
-                unused = bestH * 8 + bestV;  // height and variant of the fastest two-step candidate
-                g_tune.put(key2, h2, unused);
+                if (t2 < best2) {
+                    best2 = t2;
+                    h2 = h;
+                }
             }
-            g.b2_auto = h2;
-            const int hb = unused / 8, vb = unused % 8;
-            g.b2_best = (hb >= 8 && hb <= 64 && g.Ly % hb == 0) ? hb : 0;
-            g.b2_var = (vb == 3) ? 3 : 2;
+            if (rc) break;
+            pair = best2 / 2 < t1 ? 1 : 0;
+            g_tune.put(key2, h2, pair);
         }
+        g.kt2_auto = pair != 0;
+        if ((rc = build_band_tasks(L, g, even_band(g.Ly, h2)))) break;
     }
-    if (rc == XY_OK) rc = apply_kt_mode(L);
+    if (rc == XY_OK) apply_kt_mode(L);
     // resident shapes: block size x cluster size (1 = one block per lattice;
     // more blocks per lattice spread a small batch over more SMs)
     for (auto& g : L->res_groups) {
@@ -1132,8 +1082,7 @@ int autotune_lattice(xy_lattice* L)
             g.threads = bt;
             g.csize = bc;
             CK(prepare_resident(g.Lx, g.Ly, bt, bc, nullptr));
-            for (auto& gr : L->graphs) cudaGraphExecDestroy(gr.exec);
-            L->graphs.clear();
+            drop_graphs(L);
         } else {
             CK(prepare_resident(g.Lx, g.Ly, g.threads, g.csize, nullptr));
         }
@@ -1145,21 +1094,14 @@ int autotune_lattice(xy_lattice* L)
     return rc;
 }
 
+constexpr int kChunk = 64;             // steps of a captured chunk at most (the bits of cur_mask)
+constexpr int kResidentSteps = 1 << 14;  // steps of one resident launch at most
+
 // Advance every configuration by its n_call of the current window (already
 // uploaded), recording into rec_dev with stride rec_stride.
 int run_window(xy_lattice* L, int64_t n_max)
 {
     if (n_max <= 0) return XY_OK;
-    // two steps per launch for the strip groups the tuner gave a band height,
-    // when every configuration of the group runs the whole window (a pair
-    // never straddles the last step of one of them)
-    L->cur_kt2 = 0u;
-    for (int gi = 0; gi < (int)L->strip_groups.size() && gi < 32; ++gi) {
-        const StripGroup& g = L->strip_groups[gi];
-        bool all = g.b2_H > 0;
-        for (int c : g.cfgs) all = all && L->h_dev[c].n_call == n_max;
-        if (all) L->cur_kt2 |= 1u << gi;
-    }
     if (L->path == XY_PATH_PLAIN) {
         for (int64_t j = 0; j < n_max; ++j)
             for (int c = 0; c < L->n_cfg; ++c) {
@@ -1173,97 +1115,84 @@ int run_window(xy_lattice* L, int64_t n_max)
             }
         return XY_OK;
     }
-    // Records further apart than a chunk: the stretches between recording
-    // steps run as non-recording graph chunks, and each step at which some
-    // strip configuration records runs alone with the recording kernel.
-    if (L->cur_rec && L->cur_re > 32) {
-        std::vector<int64_t> rec_steps;
-        for (const auto& g : L->strip_groups)
-            for (int c : g.cfgs) {
-                const DevCfg& d = L->h_dev[c];
-                const int64_t re = L->cur_re;
-                for (int64_t j = ((re - d.k_start % re) % re); j < std::min(n_max, d.n_call); j += re)
-                    rec_steps.push_back(j);
-            }
-        std::sort(rec_steps.begin(), rec_steps.end());
-        rec_steps.erase(std::unique(rec_steps.begin(), rec_steps.end()), rec_steps.end());
-        auto stretch = [&](int64_t cnt) -> int {
-            L->cur_mask = 0u;
-            const int ch = (int)std::min<int64_t>(32, cnt);
-            const int64_t nf = (L->timing || ch < 2) ? 0 : cnt / ch;
-            if (nf > 0) {
-                xy_lattice::Graph* g = nullptr;
-                int rc = get_graph(L, ch, &g);
-                if (rc) return rc;
-                for (int64_t i = 0; i < nf; ++i) {
-                    CK(cudaGraphLaunch(g->exec, L->stream));
-                    L->launches += g->kernels;
-                }
-            }
-            for (int64_t done = nf * ch; done < cnt;) {
-                const int k = (int)std::min<int64_t>(ch, cnt - done);
-                int rc = launch_batched_steps(L, L->stream, 0, k, true);
-                if (rc) return rc;
-                done += k;
-            }
-            return XY_OK;
-        };
-        int64_t pos = 0;
-        for (int64_t r : rec_steps) {
-            int rc = r > pos ? stretch(r - pos) : XY_OK;
+    // A chunk of steps is captured once as a graph and replayed; steps between
+    // two records that the chunks do not fill evenly are cut into equal chunks,
+    // so that a window takes few kinds of them.
+    for (auto& g : L->strip_groups) g.buf = 0;
+    L->in_b.assign((size_t)L->n_cfg, 0);
+    if (L->strip_groups.empty() && L->plain_cfgs.empty() && !L->res_groups.empty()) {
+        // resident lattices alone: one launch runs thousands of steps (the bound
+        // keeps a launch to some tens of milliseconds)
+        for (int64_t pos = 0; pos < n_max;) {
+            const int cnt = (int)std::min<int64_t>(kResidentSteps, n_max - pos);
+            int rc = launch_batched_steps(L, L->stream, pos, cnt, false);
             if (rc) return rc;
-            L->cur_mask = 1u;  // local step 0 of this one-step launch records
-            if ((rc = launch_batched_steps(L, L->stream, 0, 1, true))) return rc;
-            pos = r + 1;
+            pos += cnt;
         }
-        return pos < n_max ? stretch(n_max - pos) : XY_OK;
+        return XY_OK;
     }
-    // graph replays of 32-step chunks (or one chunk of the whole window when
-    // it is shorter), then direct launches for the remainder.  When the
-    // window records every re <= 32 steps, the chunk is a multiple of re, so
-    // the local steps that record are the same in every chunk and only they
-    // run the recording strip kernel (cur_mask); otherwise every step may.
-    int chunk = (int)std::min<int64_t>(32, n_max);
-    L->cur_mask = ~0u;
-    if (L->cur_rec && L->cur_re > 0 && L->cur_re <= 32) {
-        chunk = (int)std::min<int64_t>((32 / L->cur_re) * L->cur_re, n_max);
-        uint32_t mask = 0;
+    // the steps at which some strip-stepped configuration records
+    const int64_t re = L->cur_rec ? L->cur_re : 0;
+    std::vector<int64_t> phase;  // the distinct first record steps, and where each ends
+    std::vector<int64_t> last;
+    if (re > 0)
         for (const auto& g : L->strip_groups)
             for (int c : g.cfgs) {
                 const DevCfg& d = L->h_dev[c];
-                for (int jl = 0; jl < chunk; ++jl)
-                    if ((d.k_start + jl) % L->cur_re == 0) mask |= 1u << jl;
+                const int64_t ph = (re - d.k_start % re) % re;
+                size_t q = 0;
+                while (q < phase.size() && phase[q] != ph) ++q;
+                if (q == phase.size()) {
+                    phase.push_back(ph);
+                    last.push_back(0);
+                }
+                last[q] = std::max(last[q], d.n_call);
             }
+    auto next_record = [&](int64_t from) {  // the first record step >= from (n_max: none)
+        int64_t best = n_max;
+        for (size_t q = 0; q < phase.size(); ++q) {
+            const int64_t r = from <= phase[q] ? phase[q] : phase[q] + (from - phase[q] + re - 1) / re * re;
+            if (r < last[q]) best = std::min(best, r);
+        }
+        return best;
+    };
+    int64_t pos = 0;
+    while (pos < n_max) {
+        int64_t cnt;
+        if (re > 0 && re <= kChunk) {
+            cnt = std::min<int64_t>(kChunk / re * re, n_max - pos);
+        } else {
+            const int64_t span = next_record(pos + 1) - pos;  // up to the next record
+            const int64_t parts = (span + kChunk - 1) / kChunk;
+            cnt = std::min(span, ((span + parts - 1) / parts + 1) / 2 * 2);
+        }
+        uint64_t mask = 0;
+        for (int64_t r = re > 0 ? next_record(pos) : n_max; r < pos + cnt; r = next_record(r + 1)) mask |= 1ull << (r - pos);
         L->cur_mask = mask;
-    }
-    const int64_t n_full = (L->timing || chunk < 2) ? 0 : n_max / chunk;
-    const int rem = (int)(n_max - n_full * chunk);
-    if (n_full > 0) {
-        xy_lattice::Graph* g = nullptr;
-        int rc = get_graph(L, chunk, &g);
-        if (rc) return rc;
-        for (int64_t i = 0; i < n_full; ++i) {
+        if (cnt >= 2 && !L->timing) {
+            xy_lattice::Graph* g = nullptr;
+            int rc = get_graph(L, (int)cnt, &g);
+            if (rc) return rc;
             CK(cudaGraphLaunch(g->exec, L->stream));
             L->launches += g->kernels;
+        } else {
+            int rc = launch_batched_steps(L, L->stream, 0, (int)cnt, pos + cnt < n_max);
+            if (rc) return rc;
         }
-    }
-    for (int64_t done = 0; done < rem;) {
-        // direct launches: at most one chunk per resident launch
-        const int cnt = (int)std::min<int64_t>(chunk, rem - done);
-        const bool more = done + cnt < rem;
-        int rc = launch_batched_steps(L, L->stream, 0, cnt, more);
-        if (rc) return rc;
-        done += cnt;
+        account_chunk(L, pos, (int)cnt);
+        pos += cnt;
     }
     return XY_OK;
 }
 
-// After a window: configurations that took an odd number of steps hold their
-// state in buffer B; copy it back so that the caller's buffers are current.
+// After a window: configurations whose state ended in buffers B (an odd number
+// of steps, or of launches for strip groups) are copied back so that the
+// caller's buffers are current.
 int fixup_parity(xy_lattice* L)
 {
     for (int c = 0; c < L->n_cfg; ++c) {
-        if ((L->h_dev[c].n_call & 1) == 0) continue;
+        const bool strip = L->path == XY_PATH_BATCHED && L->cfg[c].kind == 1;
+        if (strip ? (L->h_dev[c].n_call == 0 || !L->in_b[c]) : (L->h_dev[c].n_call & 1) == 0) continue;
         const DevCfg& d = L->h_dev[c];
         const size_t bytes = sizeof(float) * (size_t)d.N * d.n_rep;
         CK(cudaMemcpyAsync(L->thA + d.offset, L->thB + d.offset, bytes, cudaMemcpyDeviceToDevice, L->stream));
@@ -1329,30 +1258,29 @@ int build_strip_tasks(xy_lattice* L, StripGroup& g)
         g.d_cap = g.tasks.size();
     }
     CK(cudaMemcpy(g.d_tasks, g.tasks.data(), sizeof(StripTask) * g.tasks.size(), cudaMemcpyHostToDevice));
-    for (auto& gr : L->graphs) cudaGraphExecDestroy(gr.exec);
-    L->graphs.clear();
+    drop_graphs(L);
     return XY_OK;
 }
 
-// Tasks of the two-step band kernel: one block per band of H rows of every
-// lattice of the group, lattice by lattice like the strip tasks.
-int build_b2_tasks(xy_lattice* L, StripGroup& g, int H)
+// Tasks of the band kernel for bands of H rows (from now on the group's height),
+// lattice by lattice like the strip tasks.
+int build_band_tasks(xy_lattice* L, StripGroup& g, int H)
 {
-    g.b2_tasks.clear();
-    const int nb = g.Ly / H;
+    g.band_tasks.clear();
+    g.band_H = H;
+    const int nb = (g.Ly + H - 1) / H, per = bands_per_block(g.Lx);
     for (int c : g.cfgs)
         for (int r = 0; r < L->cfg[c].desc.n_replicas; ++r)
-            for (int b = 0; b < nb; ++b) g.b2_tasks.push_back(BandTask{c, r, b, nb});
-    if (g.b2_tasks.size() > g.d_b2_cap) {
-        cudaFree(g.d_b2_tasks);
-        g.d_b2_tasks = nullptr;
-        g.d_b2_cap = 0;
-        CK(cudaMalloc(&g.d_b2_tasks, sizeof(BandTask) * g.b2_tasks.size()));
-        g.d_b2_cap = g.b2_tasks.size();
+            for (int b = 0; b < nb; b += per) g.band_tasks.push_back(BandTask{c, r, b, nb});
+    if (g.band_tasks.size() > g.d_band_cap) {
+        cudaFree(g.d_band_tasks);
+        g.d_band_tasks = nullptr;
+        g.d_band_cap = 0;
+        CK(cudaMalloc(&g.d_band_tasks, sizeof(BandTask) * g.band_tasks.size()));
+        g.d_band_cap = g.band_tasks.size();
     }
-    CK(cudaMemcpy(g.d_b2_tasks, g.b2_tasks.data(), sizeof(BandTask) * g.b2_tasks.size(), cudaMemcpyHostToDevice));
-    for (auto& gr : L->graphs) cudaGraphExecDestroy(gr.exec);
-    L->graphs.clear();
+    CK(cudaMemcpy(g.d_band_tasks, g.band_tasks.data(), sizeof(BandTask) * g.band_tasks.size(), cudaMemcpyHostToDevice));
+    drop_graphs(L);
     return XY_OK;
 }
 
@@ -1384,10 +1312,12 @@ int classify(xy_lattice* L)
         const int H = choose_strip_H(Lx, Ly, same, (int64_t)sms * 16);
         if (rt > 0) {
             h.kind = 0;
-        } else if (H > 0) {
+        } else if (H > 0 || band_shape(Lx, Ly)) {
             h.kind = 1;
             h.H = H;
-            max_units = std::max(max_units, strip_units_per_lattice(Lx, Ly, std::min(H, min_strip_H(Lx, Ly))));
+            if (H > 0)
+                max_units = std::max(max_units, strip_units_per_lattice(Lx, Ly, std::min(H, min_strip_H(Lx, Ly))));
+            if (band_shape(Lx, Ly)) max_units = std::max(max_units, band_blocks(Lx, Ly, even_band(Ly, 4)));
         } else {
             h.kind = 2;
         }
@@ -1412,8 +1342,9 @@ int classify(xy_lattice* L)
             for (auto& gg : L->strip_groups)
                 if (gg.Lx == Lx && gg.Ly == Ly && gg.seed == h.desc.seed) g = &gg;
             if (!g) {
-                L->strip_groups.push_back(StripGroup{Lx, Ly, h.desc.seed, h.H, 3, {}, 0, {}, nullptr, 0});
+                L->strip_groups.push_back(StripGroup{Lx, Ly, h.desc.seed, h.H > 0});
                 g = &L->strip_groups.back();
+                g->H = h.H;
             }
             g->cfgs.push_back(c);
             g->n_lat += h.desc.n_replicas;
@@ -1427,9 +1358,12 @@ int classify(xy_lattice* L)
         CK(prepare_resident(g.Lx, g.Ly, g.threads, g.csize, nullptr));
     }
     for (auto& g : L->strip_groups) {
-        int rc = build_strip_tasks(L, g);
+        int rc = g.strip_ok ? build_strip_tasks(L, g) : XY_OK;
+        if (rc == XY_OK && band_shape(g.Lx, g.Ly))
+            rc = build_band_tasks(L, g, default_band_H(g.Lx, g.Ly, g.n_lat, (int64_t)sms * 16));
         if (rc) return rc;
     }
+    apply_kt_mode(L);
     return XY_OK;
 }
 
@@ -1444,7 +1378,7 @@ void free_lattice(xy_lattice* L)
     for (auto& g : L->res_groups) cudaFree(g.d_tasks);
     for (auto& g : L->strip_groups) {
         cudaFree(g.d_tasks);
-        cudaFree(g.d_b2_tasks);
+        cudaFree(g.d_band_tasks);
     }
     cudaFree(L->thB);
     cudaFree(L->omB);
@@ -1695,7 +1629,8 @@ int xy_set_temporal_blocking(xy_lattice* L, int kt)
     if (!L) return fail(XY_EINVAL, "NULL lattice");
     if (kt < 0 || kt > 2) return fail(XY_EINVAL, "temporal blocking must be 0 (tuner), 1 or 2 steps per launch");
     L->kt_mode = kt;
-    return L->tuned ? apply_kt_mode(L) : XY_OK;
+    apply_kt_mode(L);
+    return XY_OK;
 }
 
 int xy_set_adjoint_mode(xy_lattice* L, int mode)
@@ -2459,11 +2394,8 @@ int xy_adjoint_step_n(xy_lattice* L, int64_t n, int K, double wE, double wM, dou
                                              buf, L->d_call, L->stream));
                     ++L->launches;
                 }
-                for (auto& g : L->strip_groups) {
-                    CKA(launch_strip_step(L->d_cfg, g.d_tasks, (int)g.tasks.size(), g.H, g.variant, 0,
-                                          group_sched(L, g), g.seed, i, buf, L->d_call, L->pa, L->stream));
-                    ++L->launches;
-                }
+                for (auto& g : L->strip_groups)
+                    CKA(launch_group(L, L->stream, g, 0, g.n_lat, StepRun{0, 1, 0}, i, 0, buf));
                 for (int c : L->plain_cfgs) {
                     CKA(launch_plain_step(L->d_cfg, L->h_dev[c], i, buf, L->d_call, L->pa, 1, L->stream));
                     ++L->launches;

@@ -14,6 +14,37 @@
 namespace xy {
 
 // -------------------------------------------------------------------------
+// The four sites of a quad as two pairs (0, 1), (2, 3).  sm_103a issues one
+// FP32 instruction for a pair (fma.rn.f32x2 and its add and mul), each half
+// rounded like the scalar instruction, so a pair costs one issue slot and the
+// bits are those of the scalar code.  The steppers are bound by the issue rate
+// (82 instructions per site-update in the one-step strip kernel, 74 in the
+// two-step band kernel, at 67-71 % of the issue slots), and a third of their
+// instructions were FP32 adds and multiplies of whole quads.
+// -------------------------------------------------------------------------
+struct P4 {
+    float2 a, b;
+};
+__device__ __forceinline__ float2 splat2(float v) { return make_float2(v, v); }
+__device__ __forceinline__ P4 p4(const float4& t) { return P4{make_float2(t.x, t.y), make_float2(t.z, t.w)}; }
+__device__ __forceinline__ float4 f4(const P4& t) { return make_float4(t.a.x, t.a.y, t.b.x, t.b.y); }
+__device__ __forceinline__ P4 add4(const P4& x, const P4& y) { return P4{__fadd2_rn(x.a, y.a), __fadd2_rn(x.b, y.b)}; }
+__device__ __forceinline__ P4 mul4(const P4& x, const P4& y) { return P4{__fmul2_rn(x.a, y.a), __fmul2_rn(x.b, y.b)}; }
+__device__ __forceinline__ P4 mul4(float k, const P4& y) { return P4{__fmul2_rn(splat2(k), y.a), __fmul2_rn(splat2(k), y.b)}; }
+__device__ __forceinline__ P4 fma4(const P4& x, const P4& y, const P4& z)
+{
+    return P4{__ffma2_rn(x.a, y.a, z.a), __ffma2_rn(x.b, y.b, z.b)};
+}
+__device__ __forceinline__ P4 fma4(float k, const P4& y, const P4& z)
+{
+    return P4{__ffma2_rn(splat2(k), y.a, z.a), __ffma2_rn(splat2(k), y.b, z.b)};
+}
+__device__ __forceinline__ float p4get(const P4& v, int i)
+{
+    return i == 0 ? v.a.x : (i == 1 ? v.a.y : (i == 2 ? v.b.x : v.b.y));
+}
+
+// -------------------------------------------------------------------------
 // Counter-based noise: Philox4x32-10 (Salmon, Moraes, Dror, Shaw, SC'11).
 // Counter = (quad, (config << 16) | replica, step lo32, (tag << 24) | step hi24),
 // key = 64-bit seed.  One call gives the four Gaussians of four consecutive
@@ -57,42 +88,48 @@ __device__ __forceinline__ uint4 noise_counter(uint32_t quad, uint32_t cfg_rep, 
 }
 
 // Uniform (m + 1/2) 2^-23 in (0,1) from the top 23 bits of a word, exactly:
-// the float 1 + m 2^-23 minus (1 - 2^-24) is exact by Sterbenz' lemma.
-__device__ __forceinline__ float uniform01(uint32_t x)
+// the float 1 + m 2^-23 minus (1 - 2^-24) is exact by Sterbenz' lemma.  The
+// bits of 1 + m 2^-23, 0x3F800000 | (x >> 9), are one funnel shift of 0x7F:x.
+__device__ __forceinline__ float uniform01_plus(uint32_t x) { return __uint_as_float(__funnelshift_r(x, 0x7Fu, 9)); }
+__device__ __forceinline__ float uniform01(uint32_t x) { return __fadd_rn(uniform01_plus(x), -0.99999994f); }
+
+// Hardware log2 and reciprocal square root without the code that scales
+// subnormal operands: the operands below are never subnormal (a uniform is at
+// least 2^-24, and -2 ln u at least 1.2e-7), and for normal ones the results
+// are those of __log2f and rsqrtf.
+__device__ __forceinline__ float log2_normal(float x)
 {
-    return __fadd_rn(__uint_as_float(0x3F800000u | (x >> 9)), -0.99999994f);
+    float r;
+    asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+__device__ __forceinline__ float rsqrt_normal(float x)
+{
+    float r;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
 }
 
 // Box-Muller (Box & Muller 1958) of two uniform pairs, scaled by the noise
 // amplitude c: returns c*g0..c*g3 with g0 = r cos(2 pi u1), g1 = r sin(2 pi u1),
 // g2 = r' cos(2 pi u3), g3 = r' sin(2 pi u3), r = sqrt(-2 ln u0),
 // r' = sqrt(-2 ln u2).  The angle is shifted by -pi into the accurate range of
-// the hardware sine, and the sign flip is folded into the radius.
+// the hardware sine, and the sign flip is folded into the radius.  The two
+// Box-Muller pairs run as one packed pair.
 __device__ __forceinline__ float4 gauss4_scaled(uint4 w, float c)
 {
     const float kTwoPi = 6.28318530717958648f;
     const float kPi = 3.14159265358979324f;
     const float kM2Ln2 = -1.38629436111989061f;  // -2 ln 2
-    float4 out;
-    {
-        const float u0 = uniform01(w.x), u1 = uniform01(w.y);
-        const float t = __fmul_rn(kM2Ln2, __log2f(u0));   // -2 ln u0 > 0
-        const float r = __fmul_rn(__fmul_rn(t, rsqrtf(t)), -c);
-        float s, co;
-        __sincosf(fmaf(kTwoPi, u1, -kPi), &s, &co);
-        out.x = __fmul_rn(r, co);
-        out.y = __fmul_rn(r, s);
-    }
-    {
-        const float u2 = uniform01(w.z), u3 = uniform01(w.w);
-        const float t = __fmul_rn(kM2Ln2, __log2f(u2));
-        const float r = __fmul_rn(__fmul_rn(t, rsqrtf(t)), -c);
-        float s, co;
-        __sincosf(fmaf(kTwoPi, u3, -kPi), &s, &co);
-        out.z = __fmul_rn(r, co);
-        out.w = __fmul_rn(r, s);
-    }
-    return out;
+    const float2 ur = __fadd2_rn(make_float2(uniform01_plus(w.x), uniform01_plus(w.z)), splat2(-0.99999994f));
+    const float2 ua = __fadd2_rn(make_float2(uniform01_plus(w.y), uniform01_plus(w.w)), splat2(-0.99999994f));
+    const float2 t = __fmul2_rn(splat2(kM2Ln2), make_float2(log2_normal(ur.x), log2_normal(ur.y)));  // -2 ln u > 0
+    const float2 r = __fmul2_rn(__fmul2_rn(t, make_float2(rsqrt_normal(t.x), rsqrt_normal(t.y))), splat2(-c));
+    const float2 ang = __ffma2_rn(splat2(kTwoPi), ua, splat2(-kPi));
+    float s0, c0, s1, c1;
+    __sincosf(ang.x, &s0, &c0);
+    __sincosf(ang.y, &s1, &c1);
+    return make_float4(__fmul_rn(r.x, c0), __fmul_rn(r.x, s0), __fmul_rn(r.y, c1), __fmul_rn(r.y, s1));
 }
 
 // -------------------------------------------------------------------------
@@ -119,6 +156,19 @@ __device__ __forceinline__ float wrap_angle(float t)
     const float kHalfPi = 1.57079632679489662f;
     if (__builtin_expect(fabsf(t) < kHalfPi, 1)) return t;
     return wrap_angle_reduce(t);
+}
+
+// The same for the four angles of a quad: one test and one branch for all of
+// them (a branch per angle took three instructions each).
+__device__ __forceinline__ P4 wrap_angle4(P4 t)
+{
+    const float kHalfPi = 1.57079632679489662f;
+    const float m = fmaxf(fmaxf(fabsf(t.a.x), fabsf(t.a.y)), fmaxf(fabsf(t.b.x), fabsf(t.b.y)));
+    if (__builtin_expect(!(m < kHalfPi), 0)) {
+        t.a = make_float2(wrap_angle(t.a.x), wrap_angle(t.a.y));
+        t.b = make_float2(wrap_angle(t.b.x), wrap_angle(t.b.y));
+    }
+    return t;
 }
 
 // -------------------------------------------------------------------------
@@ -268,6 +318,48 @@ __device__ __forceinline__ SiteOut site_update(const StepConst& K, float theta, 
     o.v = fmaf(K.oma, o.omega, g);
     o.theta = wrap_angle(fmaf(K.dt, o.v, theta));
     return o;
+}
+
+// The four sites of a quad at once: (s, c) = (sin q t, cos q t) of the quad,
+// of its x neighbours (sL, cL left of site 0; sR, cR right of site 3) and of
+// the quads above and below (P, N), v and the noise cn.  The same roundings as
+// site_force and site_update.
+struct QuadOut {
+    P4 theta, v, omega;
+};
+__device__ __forceinline__ QuadOut quad_update(const StepConst& K, const P4& th, const P4& v, const P4& cn, const P4& s,
+                                               const P4& c, float sL, float cL, float sR, float cR, const P4& Ps,
+                                               const P4& Pc, const P4& Ns, const P4& Nc)
+{
+    // minus the sums of the neighbours' sines (scalar adds negate their operands
+    // for free; a packed add would need a packed negation), the cosines' sums
+    const P4 sx{make_float2(__fadd_rn(-sL, -s.a.y), __fadd_rn(-s.a.x, -s.b.x)),
+                make_float2(__fadd_rn(-s.a.y, -s.b.y), __fadd_rn(-s.b.x, -sR))};
+    const P4 sy{make_float2(__fadd_rn(-Ps.a.x, -Ns.a.x), __fadd_rn(-Ps.a.y, -Ns.a.y)),
+                make_float2(__fadd_rn(-Ps.b.x, -Ns.b.x), __fadd_rn(-Ps.b.y, -Ns.b.y))};
+    const P4 cx{make_float2(__fadd_rn(cL, c.a.y), __fadd_rn(c.a.x, c.b.x)),
+                make_float2(__fadd_rn(c.a.y, c.b.y), __fadd_rn(c.b.x, cR))};
+    const P4 cy = add4(Pc, Nc);
+    const P4 ax = fma4(s, cx, mul4(c, sx)), ay = fma4(s, cy, mul4(c, sy));
+    const P4 pt = mul4(K.p, th);
+    const P4 sp{make_float2(__sinf(pt.a.x), __sinf(pt.a.y)), make_float2(__sinf(pt.b.x), __sinf(pt.b.y))};
+    const P4 F = fma4(K.nqJx, ax, fma4(K.nqJy, ay, mul4(K.hp, sp)));
+    const P4 g = fma4(K.hdt, F, cn);
+    QuadOut o;
+    o.omega = mul4(K.inv1pa, add4(v, g));
+    o.v = fma4(K.oma, o.omega, g);
+    o.theta = wrap_angle4(fma4(K.dt, o.v, th));
+    return o;
+}
+
+// (sin q t, cos q t) of a quad
+__device__ __forceinline__ void quad_sc(float q, const P4& th, P4& s, P4& c)
+{
+    const P4 a = mul4(q, th);
+    __sincosf(a.a.x, &s.a.x, &c.a.x);
+    __sincosf(a.a.y, &s.a.y, &c.a.y);
+    __sincosf(a.b.x, &s.b.x, &c.b.x);
+    __sincosf(a.b.y, &s.b.y, &c.b.y);
 }
 
 // Energy of one site with its forward bonds (x+1, y+1), per Eq. (XY-Hamilton-Kinetic),

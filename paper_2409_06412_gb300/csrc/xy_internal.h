@@ -71,7 +71,7 @@ struct CallArgs {
     double2* rec_dev;   // [B][R] (M, E)
     int64_t k_shift;    // added to the step index (segment recompute of the adjoint)
     int record_every;   // 0: no observables
-    int fixed_parity;   // 1: always read buffers A and write buffers B
+    int fixed_parity;   // 1: always read buffers A and write buffers B (plain and resident kernels)
     int err;            // device error flag
     int m_only;         // 1: records carry M only (E left 0)
 };
@@ -138,16 +138,22 @@ cudaError_t launch_plain_step(const DevCfg* d_cfg, const DevCfg& h_cfg, int64_t 
                               const CallArgs* ca, Partials pa, int write_state, cudaStream_t st);
 // rec: 0 = no records in this launch, 1 = records of M only, 2 = M and E;
 // sched: some configuration of the tasks has a field or coupling schedule
-// (false selects kernels that read the configurations' constants only)
+// (false selects kernels that read the configurations' constants only);
+// rd_b: the state is read from buffers B and written to A (else A to B)
 cudaError_t launch_strip_step(const DevCfg* d_cfg, const StripTask* tasks, int n_tasks, int H, int variant,
-                              int rec, bool sched, uint64_t seed, int64_t j_local, Buffers buf, const CallArgs* ca,
-                              Partials pa, cudaStream_t st);
-// two steps per launch (k -> k + 2) on bands of H rows across the lattice
-// width (256 <= Lx <= 1024); the launch at j_local takes steps j and j + 1 of
-// the call; a batch of launches must hold an even number of such pairs
+                              int rec, bool sched, bool rd_b, uint64_t seed, int64_t j_local, Buffers buf,
+                              const CallArgs* ca, Partials pa, cudaStream_t st);
+// one or two steps per launch on bands of H rows across the lattice width (Lx <=
+// 2048); the launch at j_local takes step j (and j + 1) of the call, reading
+// buffers B when rd_b is set and writing the others; rec and sched as above
 struct BandTask;
-cudaError_t launch_band2_step(const DevCfg* d_cfg, const BandTask* tasks, int n_tasks, int Lx, int H, int variant,
-                              uint64_t seed, int64_t j_local, Buffers buf, const CallArgs* ca, cudaStream_t st);
+constexpr int kBandWarps = 16;       // warps of a wide band's block at most
+constexpr int kNarrowBandWarps = 4;  // warps of a block of narrow bands (Lx <= 128)
+bool band_shape(int Lx, int Ly);
+int bands_per_block(int Lx);
+cudaError_t launch_band_step(const DevCfg* d_cfg, const BandTask* tasks, int n_tasks, int Lx, int H, int rec, bool sched,
+                             int n_steps, bool rd_b, uint64_t seed, int64_t j_local, Buffers buf, const CallArgs* ca,
+                             Partials pa, cudaStream_t st);
 // every task of one launch uses the noise key `seed`
 cudaError_t launch_resident_step(const DevCfg* d_cfg, const ResidentTask* tasks, int n_tasks, int Lx, int Ly,
                                  int threads, int csize, uint64_t seed, int64_t j_local, int n_steps, Buffers buf,

@@ -365,18 +365,12 @@ namespace {
 // One row of a strip as seen by one lane: the raw angles of its quad and of
 // its edge column, and their (sin q t, cos q t).
 struct RowBuf {
-    float4 th;
+    P4 th;
     float te;
-    float s[4], c[4];
+    P4 s, c;
 };
 
-__device__ __forceinline__ void rowbuf_sc(float q, RowBuf& r)
-{
-    sc_of(q, r.th.x, r.s[0], r.c[0]);
-    sc_of(q, r.th.y, r.s[1], r.c[1]);
-    sc_of(q, r.th.z, r.s[2], r.c[2]);
-    sc_of(q, r.th.w, r.s[3], r.c[3]);
-}
+__device__ __forceinline__ void rowbuf_sc(float q, RowBuf& r) { quad_sc(q, r.th, r.s, r.c); }
 
 // Everything one lane needs to update its quad in every row of its unit.
 struct StripCtx {
@@ -421,10 +415,10 @@ __device__ __forceinline__ void strip_rows(StripCtx& X, const DevCfg& cf, const 
     int ynn = yn + 1;
     if (ynn >= X.Ly) ynn -= X.Ly;
     RowBuf P, C, N;
-    P.th = ld4(X.thS + yp * Lx + X.x);
-    C.th = ld4(X.thS + (int64_t)ybeg * Lx + X.x);
+    P.th = p4(ld4(X.thS + yp * Lx + X.x));
+    C.th = p4(ld4(X.thS + (int64_t)ybeg * Lx + X.x));
     C.te = X.thS[(int64_t)ybeg * Lx + X.xe];
-    N.th = ld4(X.thS + yn * Lx + X.x);
+    N.th = p4(ld4(X.thS + yn * Lx + X.x));
     N.te = X.thS[yn * Lx + X.xe];
     rowbuf_sc(X.K.q, P);
     rowbuf_sc(X.K.q, C);
@@ -458,10 +452,10 @@ __device__ __forceinline__ void strip_rows(StripCtx& X, const DevCfg& cf, const 
         const float4 v = stg.v[s_use][ln];
         s_use = s_use + 1 == kStages ? 0 : s_use + 1;
         rowbuf_sc(X.K.q, N);
-        float sL = __shfl_sync(kFull, C.s[3], X.srcL);
-        float cL = __shfl_sync(kFull, C.c[3], X.srcL);
-        float sR = __shfl_sync(kFull, C.s[0], X.srcR);
-        float cR = __shfl_sync(kFull, C.c[0], X.srcR);
+        float sL = __shfl_sync(kFull, C.s.b.y, X.srcL);
+        float cL = __shfl_sync(kFull, C.c.b.y, X.srcL);
+        float sR = __shfl_sync(kFull, C.s.a.x, X.srcR);
+        float cR = __shfl_sync(kFull, C.c.a.x, X.srcR);
         if (X.multi) {
             // the strip's edge column (lane 0: x0 - 1, lane 31: x0 + 128)
             float se, ce;
@@ -470,39 +464,31 @@ __device__ __forceinline__ void strip_rows(StripCtx& X, const DevCfg& cf, const 
             if (X.lg == 31) { sR = se; cR = ce; }
         }
         const float4 cn = gauss4_scaled(philox4x32_10_rk(noise_counter(quad, X.cfgrep, X.k, 0u), keys), X.K.c);
-        float to[4], vo[4];
+        const QuadOut o = quad_update(X.K, C.th, p4(v), p4(cn), C.s, C.c, sL, cL, sR, cR, P.s, P.c, N.s, N.c);
+        if (REC == 2) {
 #pragma unroll
-        for (int s = 0; s < 4; ++s) {
-            const float sl = s == 0 ? sL : C.s[s - 1];
-            const float cl = s == 0 ? cL : C.c[s - 1];
-            const float sr = s == 3 ? sR : C.s[s + 1];
-            const float cr = s == 3 ? cR : C.c[s + 1];
-            const float sx = __fadd_rn(sl, sr), cx = __fadd_rn(cl, cr);
-            const float sy = __fadd_rn(P.s[s], N.s[s]), cy = __fadd_rn(P.c[s], N.c[s]);
-            const float th = f4get(C.th, s);
-            const float F = site_force(X.K, C.s[s], C.c[s], sx, cx, sy, cy, sinp_of(X.K.p, th));
-            const SiteOut so = site_update(X.K, th, f4get(v, s), F, f4get(cn, s));
-            to[s] = so.theta;
-            vo[s] = so.v;
-            if (REC == 2) {
-                const float bx = fmaf(C.c[s], cr, __fmul_rn(C.s[s], sr));
-                const float by = fmaf(C.c[s], N.c[s], __fmul_rn(C.s[s], N.s[s]));
-                X.pe = __fadd_rn(X.pe, site_energy_rel(so.omega, bx, by, cosp_of(X.K.p, th), X.Jx, X.Jy, X.hF,
-                                                       X.eref));
+            for (int s = 0; s < 4; ++s) {
+                const float cs = p4get(C.s, s), cc = p4get(C.c, s);
+                const float sr = s == 3 ? sR : p4get(C.s, s + 1);
+                const float cr = s == 3 ? cR : p4get(C.c, s + 1);
+                const float bx = fmaf(cc, cr, __fmul_rn(cs, sr));
+                const float by = fmaf(cc, p4get(N.c, s), __fmul_rn(cs, p4get(N.s, s)));
+                X.pe = __fadd_rn(X.pe, site_energy_rel(p4get(o.omega, s), bx, by, cosp_of(X.K.p, p4get(C.th, s)), X.Jx,
+                                                       X.Jy, X.hF, X.eref));
             }
         }
         if (REC) {
             // order parameter of the row: sites x + 0, x + 2 have the parity of
             // y (x is a multiple of 4), sites x + 1, x + 3 the other one
-            const float ev = __fadd_rn(C.s[0], C.s[2]), od = __fadd_rn(C.s[1], C.s[3]);
+            const float ev = __fadd_rn(C.s.a.x, C.s.b.x), od = __fadd_rn(C.s.a.y, C.s.b.y);
             const float m = !X.stag ? __fadd_rn(ev, od) : ((y & 1) ? __fadd_rn(od, -ev) : __fadd_rn(ev, -od));
             X.pm = __fadd_rn(X.pm, m);
         }
-        st4_stream(p_to + X.x, make_float4(to[0], to[1], to[2], to[3]));
-        st4_stream(p_vo + X.x, make_float4(vo[0], vo[1], vo[2], vo[3]));
+        st4_stream(p_to + X.x, f4(o.theta));
+        st4_stream(p_vo + X.x, f4(o.v));
         P = C;
         C = N;
-        N.th = th_nn;
+        N.th = p4(th_nn);
         N.te = te_nn;
         p_to += Lx;
         p_vo += Lx;
@@ -519,7 +505,7 @@ __device__ __forceinline__ void strip_rows(StripCtx& X, const DevCfg& cf, const 
 // kernel carries none of the knot searches (1.7 % of the batch's step time).
 template <int MINB, int REC, bool SCHED>
 __global__ void __launch_bounds__(256, MINB) strip_step_kernel(const DevCfg* cfgs, const StripTask* tasks, int H,
-                                                               int64_t j_local, Buffers buf, const CallArgs* cap,
+                                                               int rd_b, int64_t j_local, Buffers buf, const CallArgs* cap,
                                                                Partials pa, PhiloxKeys keys)
 {
     const CallArgs ca = *cap;
@@ -536,12 +522,11 @@ __global__ void __launch_bounds__(256, MINB) strip_step_kernel(const DevCfg* cfg
     X.K = SCHED ? step_const_k(cf, X.k, noise_amp(cf, X.k)) : step_const(cf, noise_amp(cf, X.k));
     X.Lx = cf.Lx;
     X.Ly = cf.Ly;
-    const bool odd = !ca.fixed_parity && (j & 1) != 0;
     const int64_t lat_off = cf.offset + (int64_t)task.rep * cf.N;
-    X.thS = (odd ? buf.thB : buf.thA) + lat_off;
-    X.omS = (odd ? buf.omB : buf.omA) + lat_off;
-    X.thD = (odd ? buf.thA : buf.thB) + lat_off;
-    X.omD = (odd ? buf.omA : buf.omB) + lat_off;
+    X.thS = (rd_b ? buf.thB : buf.thA) + lat_off;
+    X.omS = (rd_b ? buf.omB : buf.omA) + lat_off;
+    X.thD = (rd_b ? buf.thA : buf.thB) + lat_off;
+    X.omD = (rd_b ? buf.omA : buf.omB) + lat_off;
 
     const int G = X.Lx >= 128 ? 32 : (X.Lx >> 2);  // lanes per row
     const int groups = 32 / G;
@@ -609,12 +594,12 @@ int strip_units_per_lattice(int Lx, int Ly, int H)
 // variant = resident blocks per SM the registers are capped for (2, 3 or 4).
 // Every task of one launch uses the noise key `seed`.
 cudaError_t launch_strip_step(const DevCfg* d_cfg, const StripTask* tasks, int n_tasks, int H, int variant,
-                              int rec, bool sched, uint64_t seed, int64_t j_local, Buffers buf, const CallArgs* ca,
-                              Partials pa, cudaStream_t st)
+                              int rec, bool sched, bool rd_b, uint64_t seed, int64_t j_local, Buffers buf,
+                              const CallArgs* ca, Partials pa, cudaStream_t st)
 {
     if (n_tasks == 0) return cudaSuccess;
     const PhiloxKeys keys = philox_round_keys(seed);
-    using Kern = void (*)(const DevCfg*, const StripTask*, int, int64_t, Buffers, const CallArgs*, Partials,
+    using Kern = void (*)(const DevCfg*, const StripTask*, int, int, int64_t, Buffers, const CallArgs*, Partials,
                           PhiloxKeys);
     // Launches that record run at most 3 blocks per SM: capped at 64
     // registers the recording code spills inside the row loop.
@@ -632,231 +617,337 @@ cudaError_t launch_strip_step(const DevCfg* d_cfg, const StripTask* tasks, int n
     };
     const int vi = variant >= 4 ? 2 : (variant == 3 ? 1 : 0);
     const Kern kern = table[sched ? 1 : 0][vi][rec < 0 ? 0 : (rec > 2 ? 2 : rec)];
-    kern<<<(unsigned)n_tasks, 256, 0, st>>>(d_cfg, tasks, H, j_local, buf, ca, pa, keys);
+    kern<<<(unsigned)n_tasks, 256, 0, st>>>(d_cfg, tasks, H, rd_b ? 1 : 0, j_local, buf, ca, pa, keys);
     return cudaGetLastError();
 }
 
 
 // ===========================================================================
-// Two steps per pass (temporal blocking over K_t = 2 steps)
+// Band stepper: two steps per pass (temporal blocking over K_t = 2 steps), or one
 // ===========================================================================
-// A block owns a band of H rows across the whole lattice width (Lx / 128
-// warps side by side, 256 <= Lx <= 1024) and sweeps it once for two steps:
-// iteration i loads row y = y0 - 2 + i of theta_k (and v_k of row y - 1),
-// advances row a = y - 1 to step k + 1 (level 1, rows y0 - 1 .. y0 + H) and
-// row b = y - 2 to step k + 2 (level 2, rows y0 .. y0 + H - 1), which is the
-// only row written back: 8 bytes per site-update instead of 16.  The two
-// extra level-1 rows are recomputed by the neighbouring bands too (2 / H
-// more level-1 work).  Columns next to a warp's strip come from the
+// A band is H rows across the whole lattice width.  It is swept once for two
+// steps: iteration i loads row y = y0 - 2 + i of theta_k (and v_k of row
+// y - 1), advances row a = y - 1 to step k + 1 (level 1, rows y0 - 1 .. y0 + H)
+// and row b = y - 2 to step k + 2 (level 2, rows y0 .. y0 + H - 1), which is the
+// only row written back: 8 bytes per site-update instead of 16.  The two extra
+// level-1 rows are recomputed by the neighbouring bands too (2 / H more level-1
+// work).  The per-site arithmetic is that of every other stepper, so states are
+// bit-identical to two single steps.  A launch of one step (or the last step of
+// a configuration whose run ends after it) writes level 1 instead.
+//
+// WIDE (Lx > 128): a block is one band, its ceil(Lx / 128) warps side by side
+// with the row's quads dealt out evenly (any Lx that is a multiple of 4: no warp
+// gets fewer than half its lanes); columns next to a warp's strip come from the
 // neighbouring warp through shared memory (one barrier per row, the lattice's
-// periodic wrap inside the block); the per-site arithmetic is that of every
-// other stepper, so states are bit-identical to two single steps.
+// periodic wrap inside the block).  Narrow lattices: a warp holds
+// floor(32 / (Lx / 4)) bands, one per lane group, and warps are independent.
+//
+// What bounds it: the issue rate.  Per site-update the step needs about 50
+// instructions (10 of Philox, 5 on the special-function unit), and the pass moves
+// 8 bytes, so at the chip's issue rate HBM is at 70 %.  So: rows rotate through
+// three register sets (the loop is unrolled by three, no copies), the noise of
+// both levels is formed at the top of the iteration (two independent Philox
+// chains to interleave, ahead of the wrap branches that split the rest), and the
+// first iterations, which have no level 1 or 2 row yet, are peeled.
 namespace {
 
-constexpr int kB2Stages = 4;
-struct B2Stage {
-    float4 th[kB2Stages][32];  // theta_k of the row loaded by an iteration
-    float4 v[kB2Stages][32];   // v_k of the row above it
+constexpr int kBStages = 3;
+struct BStage {
+    float4 th[kBStages][32];  // theta_k of the row loaded by an iteration
+    float4 v[kBStages][32];   // v_k of the row above it
 };
 struct R0 {  // a level-0 row: theta_k and its (sin q t, cos q t)
-    float4 th;
-    float s[4], c[4];
+    P4 th;
+    P4 s, c;
 };
 struct R1 {  // a level-1 row: theta_{k+1}, v_{k+1} and (sin q t, cos q t)
-    float4 th, v;
-    float s[4], c[4];
+    P4 th, v;
+    P4 s, c;
 };
-
-__device__ __forceinline__ void sc_row(float q, const float4& t, float* s, float* c)
-{
-    sc_of(q, t.x, s[0], c[0]);
-    sc_of(q, t.y, s[1], c[1]);
-    sc_of(q, t.z, s[2], c[2]);
-    sc_of(q, t.w, s[3], c[3]);
-}
-
-// One row of one level: the update of the center row C from its rows above
-// (P) and below (N); sL.. are the x neighbours of the row's first and last
-// site of this lane (shuffles, or the neighbouring warp's edge for lanes 0, 31).
-__device__ __forceinline__ void b2_update(const StepConst& K, const float* Ps, const float* Pc, const float4& th,
-                                          const float* Cs, const float* Cc, const float* Ns, const float* Nc,
-                                          const float4& v, float sL, float cL, float sR, float cR, const float4& cn,
-                                          float4& th_out, float4& v_out)
-{
-    float to[4], vo[4];
-#pragma unroll
-    for (int s = 0; s < 4; ++s) {
-        const float sl = s == 0 ? sL : Cs[s - 1];
-        const float cl = s == 0 ? cL : Cc[s - 1];
-        const float sr = s == 3 ? sR : Cs[s + 1];
-        const float cr = s == 3 ? cR : Cc[s + 1];
-        const float sx = __fadd_rn(sl, sr), cx = __fadd_rn(cl, cr);
-        const float sy = __fadd_rn(Ps[s], Ns[s]), cy = __fadd_rn(Pc[s], Nc[s]);
-        const float t = f4get(th, s);
-        const float F = site_force(K, Cs[s], Cc[s], sx, cx, sy, cy, sinp_of(K.p, t));
-        const SiteOut so = site_update(K, t, f4get(v, s), F, f4get(cn, s));
-        to[s] = so.theta;
-        vo[s] = so.v;
-    }
-    th_out = make_float4(to[0], to[1], to[2], to[3]);
-    v_out = make_float4(vo[0], vo[1], vo[2], vo[3]);
-}
 
 }  // namespace
 
-template <int MINB>
-__global__ void __launch_bounds__(256, MINB) band2_step_kernel(const DevCfg* cfgs, const BandTask* tasks, int H,
-                                                               int64_t j_local, Buffers buf, const CallArgs* cap,
-                                                               PhiloxKeys keys)
+// REC: 0 = the launch records nothing, 1 = M, 2 = M and E of step k (summed over
+// the band's own rows of level 1); SCHED: some configuration of the launch has a
+// field or coupling schedule.  n_steps: 1 or 2.  rd_b: the state is in buffers B.
+// Threads are capped so that every block size keeps 16 warps per SM (128
+// registers).
+template <bool WIDE, int REC, bool SCHED>
+__global__ void __launch_bounds__(512, 1) band_step_kernel(const DevCfg* cfgs, const BandTask* tasks, int H, int n_steps,
+                                                           int rd_b, int64_t j_local, Buffers buf, const CallArgs* cap,
+                                                           Partials pa, PhiloxKeys keys)
 {
-    extern __shared__ B2Stage s_b2stage[];  // one per warp
-    __shared__ float2 s_edge[2][2][8][2];  // [slot][level][warp][first, last site]: (sin q t, cos q t)
-    const CallArgs ca = *cap;
+    extern __shared__ BStage s_bstage[];            // one per warp
+    __shared__ float2 s_edge[2][2][kBandWarps][2];  // [slot][level][warp][first, last site]: (sin q t, cos q t)
     const int lane = threadIdx.x & 31, warp = (int)(threadIdx.x >> 5), nw = (int)(blockDim.x >> 5);
     const BandTask task = tasks[blockIdx.x];
     const DevCfg& cf = cfgs[task.cfg];
-    const int64_t j = ca.j_base + j_local;
+    const int64_t j = cap->j_base + j_local;
     if (j >= cf.n_call) return;
-    if (j + 1 >= cf.n_call) {  // the host never pairs a last single step; say so if it ever did
-        if (threadIdx.x == 0) atomicExch(&((CallArgs*)cap)->err, XY_EINVAL);
-        return;
-    }
-    const int64_t k = cf.k_start + j + ca.k_shift;
-    const StepConst K1 = step_const_k(cf, k, noise_amp(cf, k));
-    const float c2 = noise_amp(cf, k + 1);
-    const StepConst K2c = step_const_k(cf, k + 1, c2);  // the field and couplings of step k + 1
+    const bool two = n_steps == 2 && j + 1 < cf.n_call;
+    const int64_t k = cf.k_start + j + cap->k_shift;
+    const float c1 = noise_amp(cf, k), c2 = noise_amp(cf, k + 1);
+    const StepConst K1 = SCHED ? step_const_k(cf, k, c1) : step_const(cf, c1);
+    const StepConst K2 = SCHED ? step_const_k(cf, k + 1, c2) : K1;  // (the noise takes c2 itself)
     const int Lx = cf.Lx, Ly = cf.Ly;
+    const int Q = Lx >> 2;
+    // the lane's quad column, and its group of lanes spanning a row (narrow) or
+    // the warp's share of the row (wide)
+    int x, lg, last, srcL, srcR, band, own;
+    if (WIDE) {
+        const int base = Q / nw, extra = Q - base * nw;
+        const int n_lanes = base + (warp < extra ? 1 : 0);
+        lg = lane;
+        last = n_lanes - 1;
+        x = lane < n_lanes ? 4 * (warp * base + min(warp, extra) + lane) : 0;
+        srcL = (lane + 31) & 31;
+        srcR = (lane + 1) & 31;
+        band = task.band0;
+        own = lane < n_lanes ? H : 0;
+    } else {
+        const int groups = 32 / Q;
+        const int grp = min(lane / Q, groups - 1);
+        lg = lane - grp * Q;  // >= Q in the lanes left over
+        last = -1;
+        x = lg < Q ? 4 * lg : 0;
+        srcL = grp * Q + (lg == 0 ? Q - 1 : lg - 1);
+        srcR = grp * Q + (lg + 1 >= Q ? 0 : lg + 1);
+        band = task.band0 + warp * groups + grp;
+        own = lg < Q && band < task.n_bands ? H : 0;
+        if (lg >= Q) srcL = srcR = lane;
+        band = min(band, task.n_bands - 1);
+    }
+    const int y0 = band * H;
+    own = min(own, Ly - y0);  // rows this lane writes (none in the lanes that idle)
     const int64_t lat_off = cf.offset + (int64_t)task.rep * cf.N;
-    // a batch of steps holds an even number of pairs: pair p = j_local / 2 of it
-    // reads the buffer the single-step convention gives for step j, flipped when
-    // p is odd, and writes the other
-    const bool rd_b = ca.fixed_parity ? false : (((j & 1) != 0) != (((j_local >> 1) & 1) != 0));
-    const float* thS = (rd_b ? buf.thB : buf.thA) + lat_off;
-    const float* omS = (rd_b ? buf.omB : buf.omA) + lat_off;
-    float* thD = (rd_b ? buf.thA : buf.thB) + lat_off;
-    float* omD = (rd_b ? buf.omA : buf.omB) + lat_off;
-    const int x = warp * 128 + 4 * lane;
-    const int y0 = task.band0 * H;
-    const int wl = warp == 0 ? nw - 1 : warp - 1, wr = warp + 1 == nw ? 0 : warp + 1;
-    const int srcL = (lane + 31) & 31, srcR = (lane + 1) & 31;
+    const float* thS = (rd_b ? buf.thB : buf.thA) + lat_off + x;
+    const float* omS = (rd_b ? buf.omB : buf.omA) + lat_off + x;
+    float* thD = (rd_b ? buf.thA : buf.thB) + lat_off + x;
+    float* omD = (rd_b ? buf.omA : buf.omB) + lat_off + x;
     const uint32_t cfgrep = ((uint32_t)cf.noise_cfg << 16) | (uint32_t)(cf.rep0 + task.rep);
-    B2Stage& stg = s_b2stage[warp];
+    BStage& stg = s_bstage[warp];
     const int n_it = H + 4;
-    // prefetch: iteration ii loads theta_k of row y0 - 2 + ii and (ii >= 2) v_k of row y0 - 3 + ii
-    auto issue = [&](int ii) {
+    const int N = Lx * Ly;
+    // row offsets: o_ld of the row loaded next, o_v of the row whose v is loaded
+    // next, o_a of the level-1 row (all wrap at the lattice's end), o_b of the
+    // level-2 row (a row of the band: never wraps)
+    int o_ld = (y0 + 2 * Ly - 2) % Ly * Lx;
+    int o_v = o_ld, o_a = 0, o_b = y0 * Lx;
+    auto next_row = [&](int o) { return o + Lx == N ? 0 : o + Lx; };
+    // prefetch of iteration ii into slot ii % kBStages: theta_k of row y0 - 2 + ii
+    // and (ii >= 2) v_k of row y0 - 3 + ii; an empty group past the last row
+    // keeps the group count uniform
+    auto issue = [&](int ii, int slot) {
         if (ii < n_it) {
-            const int sl = ii % kB2Stages;
-            cp_async16(&stg.th[sl][lane], thS + (int64_t)wrapi(y0 - 2 + ii, Ly) * Lx + x);
-            if (ii >= 2) cp_async16(&stg.v[sl][lane], omS + (int64_t)wrapi(y0 - 3 + ii, Ly) * Lx + x);
+            cp_async16(&stg.th[slot][lane], thS + o_ld);
+            if (ii >= 2) cp_async16(&stg.v[slot][lane], omS + o_v);
+            o_v = o_ld;
+            o_ld = next_row(o_ld);
         }
         cp_async_commit();
     };
-    for (int ii = 0; ii < kB2Stages - 1; ++ii) issue(ii);
-    // neighbours in x of a row of this lane: shuffles inside the warp, the
-    // neighbouring warps' edge sites (published the iteration before) for lanes 0 and 31
-    auto x_nbrs = [&](const float* Cs, const float* Cc, int slot, int lev, float& sL, float& cL, float& sR, float& cR) {
-        sL = __shfl_sync(kFull, Cs[3], srcL);
-        cL = __shfl_sync(kFull, Cc[3], srcL);
-        sR = __shfl_sync(kFull, Cs[0], srcR);
-        cR = __shfl_sync(kFull, Cc[0], srcR);
-        // every lane reads the two edge words (a broadcast) and lanes 0 and 31
-        // select them: no divergent branch in the row loop
-        const float2 el = s_edge[slot][lev][wl][1], er = s_edge[slot][lev][wr][0];
-        sL = lane == 0 ? el.x : sL;
-        cL = lane == 0 ? el.y : cL;
-        sR = lane == 31 ? er.x : sR;
-        cR = lane == 31 ? er.y : cR;
+    issue(0, 0);
+    issue(1, 1);
+    // x neighbours of a row of this lane: shuffles inside the warp; at the ends of
+    // a wide strip the neighbouring warps' edge sites (published the iteration
+    // before), which every lane reads and the end lanes select: no branch
+    const bool at_l = WIDE && lg == 0, at_r = WIDE && lg == last;
+    const int wl = warp == 0 ? nw - 1 : warp - 1, wr = warp + 1 == nw ? 0 : warp + 1;
+    const float2* e_rd = &s_edge[0][0][at_l ? wl : wr][at_l ? 1 : 0];
+    float2* e_wr = &s_edge[0][0][warp][at_l ? 0 : 1];
+    constexpr int kLevel = kBandWarps * 2, kSlot = 2 * kLevel;  // strides of s_edge
+    auto x_nbrs = [&](const P4& Cs, const P4& Cc, int slot, int lev, float& sL, float& cL, float& sR, float& cR) {
+        sL = __shfl_sync(kFull, Cs.b.y, srcL);
+        cL = __shfl_sync(kFull, Cc.b.y, srcL);
+        sR = __shfl_sync(kFull, Cs.a.x, srcR);
+        cR = __shfl_sync(kFull, Cc.a.x, srcR);
+        if (WIDE) {
+            const float2 e = e_rd[slot * kSlot + lev * kLevel];
+            sL = at_l ? e.x : sL;
+            cL = at_l ? e.y : cL;
+            sR = at_r ? e.x : sR;
+            cR = at_r ? e.y : cR;
+        }
     };
-    auto publish = [&](const float* Cs, const float* Cc, int slot, int lev) {
-        if (lane == 0) s_edge[slot][lev][warp][0] = make_float2(Cs[0], Cc[0]);
-        if (lane == 31) s_edge[slot][lev][warp][1] = make_float2(Cs[3], Cc[3]);
+    auto publish = [&](const P4& Cs, const P4& Cc, int slot, int lev) {
+        if (WIDE && (at_l || at_r))
+            e_wr[slot * kSlot + lev * kLevel] = make_float2(at_l ? Cs.a.x : Cs.b.y, at_l ? Cc.a.x : Cc.b.y);
     };
-    R0 a0, b0, c0;
-    R1 a1, b1, c1;
+    float pm = 0.f, pe = 0.f;
+    const float2 Jk = SCHED ? couplings_at(cf, k) : make_float2(cf.Jx, cf.Jy);
+    const float hk = SCHED ? field_h(cf, k) : cf.h;
+    const float e_ref = cf.e_ref;
+    const bool stag = cf.stag != 0;
+    R0 r0[3];
+    R1 r1[3];
     // iteration i: P0, C0, N0 = level-0 rows y - 2, y - 1, y; P1, C1, N1 =
-    // level-1 rows b - 1, b, a (N1 computed here)
-    auto body = [&](int i, R0& P0, R0& C0, R0& N0, R1& P1, R1& C1, R1& N1) {
-        issue(i + kB2Stages - 1);
-        cp_async_wait<kB2Stages - 1>();  // this lane's copies of iteration i have landed
-        const int sl = i % kB2Stages;
-        const int slot = i & 1, prev = slot ^ 1;
-        N0.th = stg.th[sl][lane];
-        sc_row(K1.q, N0.th, N0.s, N0.c);
-        publish(N0.s, N0.c, slot, 0);
-        if (i >= 2) {  // level 1 on row a = y - 1
-            const int a = wrapi(y0 - 3 + i, Ly);
-            const float4 va = stg.v[sl][lane];
+    // level-1 rows b - 1, b, a (N1 computed here); levels: how many there are yet
+    auto body = [&](auto levels, int i, int slot, R0& P0, R0& C0, R0& N0, R1& P1, R1& C1, R1& N1) {
+        constexpr int LV = decltype(levels)::value;
+        issue(i + kBStages - 1, slot == 0 ? kBStages - 1 : slot - 1);
+        cp_async_wait<kBStages - 1>();  // this lane's copies of iteration i have landed
+        const int cur = i & 1, prev = cur ^ 1;
+        N0.th = p4(stg.th[slot][lane]);
+        float4 cn1, cn2;
+        if (LV >= 1) cn1 = gauss4_scaled(philox4x32_10_rk(noise_counter((uint32_t)(o_a + x) >> 2, cfgrep, k, 0u), keys), c1);
+        if (LV >= 2)
+            cn2 = gauss4_scaled(philox4x32_10_rk(noise_counter((uint32_t)(o_b + x) >> 2, cfgrep, k + 1, 0u), keys), c2);
+        quad_sc(K1.q, N0.th, N0.s, N0.c);
+        publish(N0.s, N0.c, cur, 0);
+        if (LV >= 1) {  // level 1 on row a = y - 1
+            const P4 va = p4(stg.v[slot][lane]);
             float sL, cL, sR, cR;
             x_nbrs(C0.s, C0.c, prev, 0, sL, cL, sR, cR);
-            const uint32_t quad = (uint32_t)(((int64_t)a * Lx + x) >> 2);
-            const float4 cn = gauss4_scaled(philox4x32_10_rk(noise_counter(quad, cfgrep, k, 0u), keys), K1.c);
-            b2_update(K1, P0.s, P0.c, C0.th, C0.s, C0.c, N0.s, N0.c, va, sL, cL, sR, cR, cn, N1.th, N1.v);
-            sc_row(K1.q, N1.th, N1.s, N1.c);
-            publish(N1.s, N1.c, slot, 1);
+            const QuadOut o = quad_update(K1, C0.th, va, p4(cn1), C0.s, C0.c, sL, cL, sR, cR, P0.s, P0.c, N0.s, N0.c);
+            N1.th = o.theta;
+            N1.v = o.v;
+            const int ra = i - 3;  // row of the band
+            if (REC > 0 && ra >= 0 && ra < own) {
+                const int odd = stag ? (x + y0 + ra) & 1 : 0;
+                const float ev = __fadd_rn(C0.s.a.x, C0.s.b.x), od = __fadd_rn(C0.s.a.y, C0.s.b.y);
+                pm = __fadd_rn(pm, !stag ? __fadd_rn(ev, od) : (odd ? __fadd_rn(od, -ev) : __fadd_rn(ev, -od)));
+                if (REC == 2) {
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                        const float s = p4get(C0.s, q), c = p4get(C0.c, q);
+                        const float sr = q == 3 ? sR : p4get(C0.s, q + 1), cr = q == 3 ? cR : p4get(C0.c, q + 1);
+                        const float bx = fmaf(c, cr, __fmul_rn(s, sr));
+                        const float by = fmaf(c, p4get(N0.c, q), __fmul_rn(s, p4get(N0.s, q)));
+                        pe = __fadd_rn(pe, site_energy_rel(p4get(o.omega, q), bx, by, cosp_of(K1.p, p4get(C0.th, q)),
+                                                           Jk.x, Jk.y, hk, e_ref));
+                    }
+                }
+            }
+            if (two) {
+                quad_sc(K1.q, N1.th, N1.s, N1.c);
+                publish(N1.s, N1.c, cur, 1);
+            } else if (ra >= 0 && ra < own) {
+                st4_stream(thD + o_a, f4(N1.th));
+                st4_stream(omD + o_a, f4(N1.v));
+            }
+            o_a = next_row(o_a);
         }
-        if (i >= 4) {  // level 2 on row b = y - 2
-            const int b = wrapi(y0 - 4 + i, Ly);
+        if (LV >= 2 && two) {  // level 2 on row b = y - 2
             float sL, cL, sR, cR;
             x_nbrs(C1.s, C1.c, prev, 1, sL, cL, sR, cR);
-            const uint32_t quad = (uint32_t)(((int64_t)b * Lx + x) >> 2);
-            const StepConst K2 = K2c;
-            const float4 cn = gauss4_scaled(philox4x32_10_rk(noise_counter(quad, cfgrep, k + 1, 0u), keys), c2);
-            float4 to, vo;
-            b2_update(K2, P1.s, P1.c, C1.th, C1.s, C1.c, N1.s, N1.c, C1.v, sL, cL, sR, cR, cn, to, vo);
-            st4_stream(thD + (int64_t)b * Lx + x, to);
-            st4_stream(omD + (int64_t)b * Lx + x, vo);
+            const QuadOut o = quad_update(K2, C1.th, C1.v, p4(cn2), C1.s, C1.c, sL, cL, sR, cR, P1.s, P1.c, N1.s, N1.c);
+            if (i - 4 < own) {
+                st4_stream(thD + o_b, f4(o.theta));
+                st4_stream(omD + o_b, f4(o.v));
+            }
+            o_b += Lx;
         }
-        __syncthreads();  // edges of this iteration visible; the slot read here free for the next
+        if (WIDE) __syncthreads();  // edges of this iteration visible; the slot read here free for the next
     };
-    for (int i = 0; i < n_it; i += 3) {
-        body(i, a0, b0, c0, a1, b1, c1);
-        if (i + 1 < n_it) body(i + 1, b0, c0, a0, b1, c1, a1);
-        if (i + 2 < n_it) body(i + 2, c0, a0, b0, c1, a1, b1);
+    using L0 = std::integral_constant<int, 0>;
+    using L1 = std::integral_constant<int, 1>;
+    using L2 = std::integral_constant<int, 2>;
+    o_a = (y0 + Ly - 1) % Ly * Lx;
+    body(L0{}, 0, 0, r0[1], r0[2], r0[0], r1[1], r1[2], r1[0]);
+    body(L0{}, 1, 1, r0[2], r0[0], r0[1], r1[2], r1[0], r1[1]);
+    body(L1{}, 2, 2, r0[0], r0[1], r0[2], r1[0], r1[1], r1[2]);
+    body(L1{}, 3, 0, r0[1], r0[2], r0[0], r1[1], r1[2], r1[0]);
+    for (int i = 4; i < n_it; i += 3) {
+        body(L2{}, i, 1, r0[2], r0[0], r0[1], r1[2], r1[0], r1[1]);
+        if (i + 1 < n_it) body(L2{}, i + 1, 2, r0[0], r0[1], r0[2], r1[0], r1[1], r1[2]);
+        if (i + 2 < n_it) body(L2{}, i + 2, 0, r0[1], r0[2], r0[0], r1[1], r1[2], r1[0]);
     }
     cp_async_wait<0>();
+    if (REC > 0) {
+        // one partial per block: warp sums, then the block's warps in order
+        __shared__ double2 s_part[kBandWarps];
+        const double wm = warp_sumf(pm), we = warp_sumf(pe);
+        if (lane == 0) s_part[warp] = make_double2(wm, we);
+        __syncthreads();
+        if (warp == 0) {
+            double bm = 0.0, be = 0.0;
+            for (int w = 0; w < nw; ++w) {
+                bm += s_part[w].x;
+                be += s_part[w].y;
+            }
+            const CallArgs ca = *cap;
+            if (ca.record_every <= 0 || k % ca.record_every != 0) return;  // uniform
+            const int per_block = WIDE ? 1 : nw * (32 / Q);
+            const int64_t b = cf.b_first + task.rep;
+            const int64_t r = (k - cf.rec_first) / ca.record_every;
+            commit_partial(pa, b, task.band0 / per_block, (task.n_bands + per_block - 1) / per_block, bm, be,
+                           ca.rec_dev + b * ca.rec_stride + r, cf.N, REC == 2 ? (double)cf.e_ref : 0.0);
+        }
+    }
 }
 
-// Bands of the two-step kernel: H (dividing Ly) is the tuner's to choose;
-// threads = Lx / 4, one warp per 128 columns.
-cudaError_t launch_band2_step(const DevCfg* d_cfg, const BandTask* tasks, int n_tasks, int Lx, int H, int variant,
-                              uint64_t seed, int64_t j_local, Buffers buf, const CallArgs* ca, cudaStream_t st)
+// Shapes of the band kernel: rows of up to 16 warps (Lx <= 2048), any Lx that is
+// a multiple of 4 and any Ly.
+bool band_shape(int Lx, int Ly) { return Lx >= 4 && Lx <= 128 * kBandWarps && Lx % 4 == 0 && Ly >= 1; }
+// Bands of one lattice that a block takes, and the block's threads.
+int bands_per_block(int Lx) { return Lx > 128 ? 1 : kNarrowBandWarps * (32 / (Lx / 4)); }
+
+// One step (n_steps = 1) or two of every task, H rows per band; the launch at
+// j_local takes step j (and j + 1) of the call.
+cudaError_t launch_band_step(const DevCfg* d_cfg, const BandTask* tasks, int n_tasks, int Lx, int H, int rec, bool sched,
+                             int n_steps, bool rd_b, uint64_t seed, int64_t j_local, Buffers buf, const CallArgs* ca,
+                             Partials pa, cudaStream_t st)
 {
     if (n_tasks == 0) return cudaSuccess;
-    if (Lx < 256 || Lx > 1024 || Lx % 128 != 0) return cudaErrorInvalidValue;
-    // variant = resident 256-thread blocks per SM the registers are capped for:
-    // 2 (no spills) or 3 (a few spilled words, more warps to hide latency)
-    using Kern = void (*)(const DevCfg*, const BandTask*, int, int64_t, Buffers, const CallArgs*, PhiloxKeys);
-    const Kern kern = variant >= 3 ? band2_step_kernel<3> : band2_step_kernel<2>;
-    const size_t smem = sizeof(B2Stage) * (size_t)(Lx / 128);
-    kern<<<(unsigned)n_tasks, Lx / 4, smem, st>>>(d_cfg, tasks, H, j_local, buf, ca, philox_round_keys(seed));
+    if (!band_shape(Lx, 1) || H < 1) return cudaErrorInvalidValue;
+    using Kern = void (*)(const DevCfg*, const BandTask*, int, int, int, int64_t, Buffers, const CallArgs*, Partials,
+                          PhiloxKeys);
+    static const Kern table[2][2][3] = {
+        {{band_step_kernel<false, 0, false>, band_step_kernel<false, 1, false>, band_step_kernel<false, 2, false>},
+         {band_step_kernel<false, 0, true>, band_step_kernel<false, 1, true>, band_step_kernel<false, 2, true>}},
+        {{band_step_kernel<true, 0, false>, band_step_kernel<true, 1, false>, band_step_kernel<true, 2, false>},
+         {band_step_kernel<true, 0, true>, band_step_kernel<true, 1, true>, band_step_kernel<true, 2, true>}},
+    };
+    const Kern kern = table[Lx > 128 ? 1 : 0][sched ? 1 : 0][rec < 0 ? 0 : (rec > 2 ? 2 : rec)];
+    const int warps = Lx > 128 ? (Lx + 127) / 128 : kNarrowBandWarps;
+    const size_t smem = sizeof(BStage) * (size_t)warps;
+    if (smem > 46 * 1024) {  // 16 warps: with the static part above the default limit
+        const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+    }
+    kern<<<(unsigned)n_tasks, 32 * warps, smem, st>>>(d_cfg, tasks, H, n_steps, rd_b ? 1 : 0,
+                                                                               j_local, buf, ca, pa,
+                                                                               philox_round_keys(seed));
     return cudaGetLastError();
 }
 
 namespace {
 struct SC4 {
-    float s[4], c[4];
+    P4 s, c;
 };
 
-__device__ __forceinline__ void sc4_from_theta(const float4& t, float q, SC4& r)
-{
-    sc_of(q, t.x, r.s[0], r.c[0]);
-    sc_of(q, t.y, r.s[1], r.c[1]);
-    sc_of(q, t.z, r.s[2], r.c[2]);
-    sc_of(q, t.w, r.s[3], r.c[3]);
-}
+__device__ __forceinline__ void sc4_from_theta(const float4& t, float q, SC4& r) { quad_sc(q, p4(t), r.s, r.c); }
 
+// An exported row holds, quad by quad, four sines and then four cosines.
 __device__ __forceinline__ void sc4_load(const float2* p, SC4& r)
 {
-    const float4 a = *reinterpret_cast<const float4*>(p);
-    const float4 b = *reinterpret_cast<const float4*>(p + 2);
-    r.s[0] = a.x; r.c[0] = a.y; r.s[1] = a.z; r.c[1] = a.w;
-    r.s[2] = b.x; r.c[2] = b.y; r.s[3] = b.z; r.c[3] = b.w;
+    r.s = p4(*reinterpret_cast<const float4*>(p));
+    r.c = p4(*reinterpret_cast<const float4*>(p + 2));
 }
 
 __device__ __forceinline__ void sc4_store(float2* p, const SC4& r)
 {
-    *reinterpret_cast<float4*>(p) = make_float4(r.s[0], r.c[0], r.s[1], r.c[1]);
-    *reinterpret_cast<float4*>(p + 2) = make_float4(r.s[2], r.c[2], r.s[3], r.c[3]);
+    *reinterpret_cast<float4*>(p) = f4(r.s);
+    *reinterpret_cast<float4*>(p + 2) = f4(r.c);
+}
+
+// A quad's terms of M and E in site order; odd: site 0 carries the minus sign
+// of the staggered order parameter.
+__device__ __forceinline__ void quad_observe(const DevCfg& cf, float2 Jk, float hk, float p, bool odd, bool stag,
+                                             bool want_e, const P4& th, const P4& omega, const SC4& cur, float sR,
+                                             float cR, const SC4& nxt, float& pm, float& pe)
+{
+#pragma unroll
+    for (int s = 0; s < 4; ++s) {
+        const float sigma = (stag && (odd != ((s & 1) != 0))) ? -1.f : 1.f;
+        pm = fmaf(sigma, p4get(cur.s, s), pm);
+        if (want_e) {
+            const float sr = s == 3 ? sR : p4get(cur.s, s + 1);
+            const float cr = s == 3 ? cR : p4get(cur.c, s + 1);
+            pe = __fadd_rn(pe, site_energy(cf, Jk, hk, p4get(omega, s), p4get(cur.s, s), p4get(cur.c, s), sr, cr,
+                                           p4get(nxt.s, s), p4get(nxt.c, s), cosp_of(p, p4get(th, s))));
+        }
+    }
 }
 }  // namespace
 
@@ -1028,33 +1119,16 @@ __global__ void __launch_bounds__(MAXT, 1) resident_step_kernel(const DevCfg* cf
             // compiler with this step's update
             float4 cn_next = cn1;
             if (j + 1 < j1) cn_next = noise1(k + 1);
-            const float sL = __shfl_sync(kFull, cur.s[3], srcL), cL = __shfl_sync(kFull, cur.c[3], srcL);
-            const float sR = __shfl_sync(kFull, cur.s[0], srcR), cR = __shfl_sync(kFull, cur.c[0], srcR);
-            float to[4], vo[4];
+            const float sL = __shfl_sync(kFull, cur.s.b.y, srcL), cL = __shfl_sync(kFull, cur.c.b.y, srcL);
+            const float sR = __shfl_sync(kFull, cur.s.a.x, srcR), cR = __shfl_sync(kFull, cur.c.a.x, srcR);
             float pm = 0.f, pe = 0.f;
-#pragma unroll
-            for (int s = 0; s < 4; ++s) {
-                const float sl = s == 0 ? sL : cur.s[s - 1];
-                const float cl_ = s == 0 ? cL : cur.c[s - 1];
-                const float sr = s == 3 ? sR : cur.s[s + 1];
-                const float cr = s == 3 ? cR : cur.c[s + 1];
-                const float sx = __fadd_rn(sl, sr), cx = __fadd_rn(cl_, cr);
-                const float sy = __fadd_rn(prev.s[s], nxt.s[s]), cy = __fadd_rn(prev.c[s], nxt.c[s]);
-                const float th = f4get(th4, s);
-                const float F = site_force(K, cur.s[s], cur.c[s], sx, cx, sy, cy, sinp_of(K.p, th));
-                const SiteOut so = site_update(K, th, f4get(v4, s), F, f4get(cn1, s));
-                to[s] = so.theta;
-                vo[s] = so.v;
-                if (rec) {
-                    const float sigma = (stag && ((x + s + gy) & 1)) ? -1.f : 1.f;
-                    pm = fmaf(sigma, cur.s[s], pm);
-                    if (!ca.m_only)
-                        pe = __fadd_rn(pe, site_energy(cf, FS ? couplings_at(cf, k) : J0, FS ? field_h(cf, k) : h0, so.omega, cur.s[s], cur.c[s], sr, cr,
-                                                       nxt.s[s], nxt.c[s], cosp_of(K.p, th)));
-                }
-            }
-            th4 = make_float4(to[0], to[1], to[2], to[3]);
-            v4 = make_float4(vo[0], vo[1], vo[2], vo[3]);
+            const QuadOut o = quad_update(K, p4(th4), p4(v4), p4(cn1), cur.s, cur.c, sL, cL, sR, cR, prev.s, prev.c,
+                                          nxt.s, nxt.c);
+            if (rec)
+                quad_observe(cf, FS ? couplings_at(cf, k) : J0, FS ? field_h(cf, k) : h0, K.p, stag && ((x + gy) & 1), stag,
+                             !ca.m_only, p4(th4), o.omega, cur, sR, cR, nxt, pm, pe);
+            th4 = f4(o.theta);
+            v4 = f4(o.v);
             cn1 = cn_next;
             if (rec) {
                 double* red = s_red + 64 * par;
@@ -1127,37 +1201,21 @@ __global__ void __launch_bounds__(MAXT, 1) resident_step_kernel(const DevCfg* cf
                 else sc4_from_theta(ld4(s_th + (y + 1) * Lx + x), K.q, nxt);
                 const float4 th4 = ld4(s_th + y * Lx + x);
                 const float4 v4 = ld4(s_om + y * Lx + x);
-                const float sL = __shfl_sync(kFull, cur.s[3], srcL), cL = __shfl_sync(kFull, cur.c[3], srcL);
-                const float sR = __shfl_sync(kFull, cur.s[0], srcR), cR = __shfl_sync(kFull, cur.c[0], srcR);
+                const float sL = __shfl_sync(kFull, cur.s.b.y, srcL), cL = __shfl_sync(kFull, cur.c.b.y, srcL);
+                const float sR = __shfl_sync(kFull, cur.s.a.x, srcR), cR = __shfl_sync(kFull, cur.c.a.x, srcR);
                 float4 cn = cn1;
                 if (!R1) {
                     const uint32_t quad = (uint32_t)(((y_base + y) * Lx + x) >> 2);
                     cn = gauss4_scaled(philox4x32_10_rk(noise_counter(quad, cfgrep, k, 0u), keys), K.c);
                 }
-                float to[4], vo[4];
-    #pragma unroll
-                for (int s = 0; s < 4; ++s) {
-                    const float sl = s == 0 ? sL : cur.s[s - 1];
-                    const float cl_ = s == 0 ? cL : cur.c[s - 1];
-                    const float sr = s == 3 ? sR : cur.s[s + 1];
-                    const float cr = s == 3 ? cR : cur.c[s + 1];
-                    const float sx = __fadd_rn(sl, sr), cx = __fadd_rn(cl_, cr);
-                    const float sy = __fadd_rn(prev.s[s], nxt.s[s]), cy = __fadd_rn(prev.c[s], nxt.c[s]);
-                    const float th = f4get(th4, s);
-                    const float F = site_force(K, cur.s[s], cur.c[s], sx, cx, sy, cy, sinp_of(K.p, th));
-                    const SiteOut so = site_update(K, th, f4get(v4, s), F, f4get(cn, s));
-                    to[s] = so.theta;
-                    vo[s] = so.v;
-                    if (rec) {
-                        const float sigma = (stag && ((x + s + y_base + y) & 1)) ? -1.f : 1.f;
-                        pm = fmaf(sigma, cur.s[s], pm);
-                        if (!ca.m_only)
-                            pe = __fadd_rn(pe, site_energy(cf, FS ? couplings_at(cf, k) : J0, FS ? field_h(cf, k) : h0, so.omega, cur.s[s], cur.c[s], sr, cr,
-                                                           nxt.s[s], nxt.c[s], cosp_of(K.p, th)));
-                    }
-                }
-                st4(s_th + y * Lx + x, make_float4(to[0], to[1], to[2], to[3]));
-                st4(s_om + y * Lx + x, make_float4(vo[0], vo[1], vo[2], vo[3]));
+                const QuadOut o = quad_update(K, p4(th4), p4(v4), p4(cn), cur.s, cur.c, sL, cL, sR, cR, prev.s, prev.c,
+                                              nxt.s, nxt.c);
+                if (rec)
+                    quad_observe(cf, FS ? couplings_at(cf, k) : J0, FS ? field_h(cf, k) : h0, K.p,
+                                 stag && ((x + y_base + y) & 1), stag, !ca.m_only, p4(th4), o.omega, cur, sR, cR, nxt, pm,
+                                 pe);
+                st4(s_th + y * Lx + x, f4(o.theta));
+                st4(s_om + y * Lx + x, f4(o.v));
                 prev = cur;
                 cur = nxt;
             }
