@@ -313,6 +313,7 @@ int upload_call(xy_lattice* L, const CallArgs& ca)
     L->call_next = (L->call_next + 1) % xy_lattice::kRing;
     CK(cudaEventSynchronize(L->call_ev[slot]));
     L->h_call[slot] = ca;
+    L->h_call[slot].err = L->d_err;
     CK(cudaMemcpyAsync(L->d_call, &L->h_call[slot], sizeof(CallArgs), cudaMemcpyHostToDevice, L->stream));
     CK(cudaEventRecord(L->call_ev[slot], L->stream));
     return XY_OK;
@@ -994,7 +995,7 @@ int autotune_lattice(xy_lattice* L)
         char key2[256];
         snprintf(key2, sizeof key2, "%s|band-sliced|%d|%d|%lld", gpu.c_str(), g.Lx, g.Ly, (long long)g.n_lat);
         int h2 = 0, pair = 0;
-        if (g_tune.get(key2, &h2, &pair) && !(h2 >= 4 && h2 <= 64 && (pair == 0 || pair == 1))) h2 = 0;
+        if (g_tune.get(key2, &h2, &pair) && !(h2 >= 4 && h2 <= 128 && (pair == 0 || pair == 1))) h2 = 0;
         if (h2 == 0) {
             float t1 = 1e30f, best2 = 1e30f;
             if (g.strip_ok)
@@ -1002,7 +1003,7 @@ int autotune_lattice(xy_lattice* L)
                     return launch_strip_step(L->d_cfg, g.d_tasks + t0, cnt, g.H, g.variant, 0, group_sched(L, g), false,
                                              g.seed, 0, buf, L->d_call, L->pa, st);
                 }, t1);
-            for (int h : {4, 8, 16, 32, 64}) {
+            for (int h : {4, 8, 16, 32, 64, 128}) {
                 if (rc || (h > 4 && h > g.Ly)) continue;
                 const int H = even_band(g.Ly, h);
                 if ((rc = build_band_tasks(L, g, H))) break;

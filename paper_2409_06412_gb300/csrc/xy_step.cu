@@ -642,20 +642,53 @@ cudaError_t launch_strip_step(const DevCfg* d_cfg, const StripTask* tasks, int n
 // periodic wrap inside the block).  Narrow lattices: a warp holds
 // floor(32 / (Lx / 4)) bands, one per lane group, and warps are independent.
 //
-// What bounds it: the issue rate.  Per site-update the step needs about 50
-// instructions (10 of Philox, 5 on the special-function unit), and the pass moves
-// 8 bytes, so at the chip's issue rate HBM is at 70 %.  So: rows rotate through
-// three register sets (the loop is unrolled by three, no copies), the noise of
-// both levels is formed at the top of the iteration (two independent Philox
-// chains to interleave, ahead of the wrap branches that split the rest), and the
-// first iterations, which have no level 1 or 2 row yet, are peeled.
+// What bounds it: the issue slots that dependent instructions leave empty.  A
+// site-update takes about 49 instructions (10 of Philox, 5 on the special-function
+// unit), 57 % of the issue slots at 16 warps per SM (128 registers; 20 warps at
+// 96 registers gained 2 %, less than what they spilled), and 8 bytes, 60 % of the
+// copy bandwidth.  So: rows rotate through three register sets (the loop is
+// unrolled by three, no copies), each of the two updates has the other one's
+// noise to interleave with, neighbours come from shared memory, and the first
+// iterations, which have no level 1 or 2 row yet, are peeled.  Measured on
+// 3.4e7 sites at 2070 MHz, one step per launch (strip kernel) against two:
+// 256 x 256 4.02e11 -> 5.1e11 site-updates/s, 1024 x 1024 4.13e11 -> 4.8e11,
+// 2048 x 2048 4.13e11 -> 4.8e11.
 namespace {
 
 constexpr int kBStages = 3;
 struct BStage {
     float4 th[kBStages][32];  // theta_k of the row loaded by an iteration
     float4 v[kBStages][32];   // v_k of the row above it
+    // ends of the quads of a row, for the lanes beside: (sin q t, cos q t) of the
+    // first and of the last site, by iteration % 3 and level
+    float4 e0[3][32], e1[3][32];
 };
+// A barrier of the block's warps with arrival and wait apart.  The wait is
+// bounded: every warp arrives once per phase whatever its data, so the bound is
+// reached only if the launch itself is broken; the caller then says so and goes
+// on with what the edge slots hold.
+__device__ __forceinline__ void mbar_init(uint64_t* bar, int count)
+{
+    asm volatile("mbarrier.init.shared.b64 [%0], %1;" ::"r"((unsigned)__cvta_generic_to_shared(bar)), "r"(count) : "memory");
+}
+__device__ __forceinline__ void mbar_arrive(uint64_t* bar)
+{
+    asm volatile("{\n .reg .b64 t;\n mbarrier.arrive.shared.b64 t, [%0];\n}" ::"r"((unsigned)__cvta_generic_to_shared(bar))
+                 : "memory");
+}
+__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity)
+{
+    for (int it = 0; it < (1 << 16); ++it) {
+        uint32_t done;
+        asm volatile("{\n .reg .pred p;\n mbarrier.try_wait.parity.shared.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}"
+                     : "=r"(done)
+                     : "r"((unsigned)__cvta_generic_to_shared(bar)), "r"(parity)
+                     : "memory");
+        if (done) return true;
+    }
+    return false;
+}
+
 struct R0 {  // a level-0 row: theta_k and its (sin q t, cos q t)
     P4 th;
     P4 s, c;
@@ -672,19 +705,24 @@ struct R1 {  // a level-1 row: theta_{k+1}, v_{k+1} and (sin q t, cos q t)
 // field or coupling schedule.  n_steps: 1 or 2.  rd_b: the state is in buffers B.
 // Threads are capped so that every block size keeps 16 warps per SM (128
 // registers).
-template <bool WIDE, int REC, bool SCHED>
+// APART: a wide band's warps arrive and wait apart.
+template <bool WIDE, bool APART, int REC, bool SCHED>
 __global__ void __launch_bounds__(512, 1) band_step_kernel(const DevCfg* cfgs, const BandTask* tasks, int H, int n_steps,
                                                            int rd_b, int64_t j_local, Buffers buf, const CallArgs* cap,
                                                            Partials pa, PhiloxKeys keys)
 {
-    extern __shared__ BStage s_bstage[];            // one per warp
-    __shared__ float2 s_edge[2][2][kBandWarps][2];  // [slot][level][warp][first, last site]: (sin q t, cos q t)
+    extern __shared__ BStage s_bstage[];  // one per warp
+    __shared__ uint64_t s_bar;            // phase i: every warp has published its quads' ends of iteration i
     const int lane = threadIdx.x & 31, warp = (int)(threadIdx.x >> 5), nw = (int)(blockDim.x >> 5);
     const BandTask task = tasks[blockIdx.x];
     const DevCfg& cf = cfgs[task.cfg];
     const int64_t j = cap->j_base + j_local;
     if (j >= cf.n_call) return;
     const bool two = n_steps == 2 && j + 1 < cf.n_call;
+    if (APART) {
+        if (threadIdx.x == 0) mbar_init(&s_bar, nw);
+        __syncthreads();
+    }
     const int64_t k = cf.k_start + j + cap->k_shift;
     const float c1 = noise_amp(cf, k), c2 = noise_amp(cf, k + 1);
     const StepConst K1 = SCHED ? step_const_k(cf, k, c1) : step_const(cf, c1);
@@ -693,28 +731,32 @@ __global__ void __launch_bounds__(512, 1) band_step_kernel(const DevCfg* cfgs, c
     const int Q = Lx >> 2;
     // the lane's quad column, and its group of lanes spanning a row (narrow) or
     // the warp's share of the row (wide)
-    int x, lg, last, srcL, srcR, band, own;
+    int x, wL = warp, lL, wR = warp, lR, band, own;  // (wL, lL), (wR, lR): warp and lane of the quads beside
     if (WIDE) {
         const int base = Q / nw, extra = Q - base * nw;
         const int n_lanes = base + (warp < extra ? 1 : 0);
-        lg = lane;
-        last = n_lanes - 1;
         x = lane < n_lanes ? 4 * (warp * base + min(warp, extra) + lane) : 0;
-        srcL = (lane + 31) & 31;
-        srcR = (lane + 1) & 31;
+        lL = lane - 1;
+        lR = lane + 1;
+        if (lane == 0) {
+            wL = warp == 0 ? nw - 1 : warp - 1;
+            lL = base - (wL < extra ? 0 : 1);
+        }
+        if (lane >= n_lanes - 1) {
+            wR = warp + 1 == nw ? 0 : warp + 1;
+            lR = 0;
+        }
         band = task.band0;
         own = lane < n_lanes ? H : 0;
     } else {
         const int groups = 32 / Q;
         const int grp = min(lane / Q, groups - 1);
-        lg = lane - grp * Q;  // >= Q in the lanes left over
-        last = -1;
+        const int lg = lane - grp * Q;  // >= Q in the lanes left over
         x = lg < Q ? 4 * lg : 0;
-        srcL = grp * Q + (lg == 0 ? Q - 1 : lg - 1);
-        srcR = grp * Q + (lg + 1 >= Q ? 0 : lg + 1);
+        lL = grp * Q + (lg == 0 ? Q - 1 : lg - 1);
+        lR = grp * Q + (lg + 1 >= Q ? 0 : lg + 1);
         band = task.band0 + warp * groups + grp;
         own = lg < Q && band < task.n_bands ? H : 0;
-        if (lg >= Q) srcL = srcR = lane;
         band = min(band, task.n_bands - 1);
     }
     const int y0 = band * H;
@@ -748,31 +790,45 @@ __global__ void __launch_bounds__(512, 1) band_step_kernel(const DevCfg* cfgs, c
     };
     issue(0, 0);
     issue(1, 1);
-    // x neighbours of a row of this lane: shuffles inside the warp; at the ends of
-    // a wide strip the neighbouring warps' edge sites (published the iteration
-    // before), which every lane reads and the end lanes select: no branch
-    const bool at_l = WIDE && lg == 0, at_r = WIDE && lg == last;
-    const int wl = warp == 0 ? nw - 1 : warp - 1, wr = warp + 1 == nw ? 0 : warp + 1;
-    const float2* e_rd = &s_edge[0][0][at_l ? wl : wr][at_l ? 1 : 0];
-    float2* e_wr = &s_edge[0][0][warp][at_l ? 0 : 1];
-    constexpr int kLevel = kBandWarps * 2, kSlot = 2 * kLevel;  // strides of s_edge
-    auto x_nbrs = [&](const P4& Cs, const P4& Cc, int slot, int lev, float& sL, float& cL, float& sR, float& cR) {
-        sL = __shfl_sync(kFull, Cs.b.y, srcL);
-        cL = __shfl_sync(kFull, Cc.b.y, srcL);
-        sR = __shfl_sync(kFull, Cs.a.x, srcR);
-        cR = __shfl_sync(kFull, Cc.a.x, srcR);
-        if (WIDE) {
-            const float2 e = e_rd[slot * kSlot + lev * kLevel];
-            sL = at_l ? e.x : sL;
-            cL = at_l ? e.y : cL;
-            sR = at_r ? e.x : sR;
-            cR = at_r ? e.y : cR;
-        }
+    // The ends of the quads beside come from shared memory, inside the warp as
+    // across warps: one store and two loads per level, published an iteration
+    // before they are read (four shuffles, and selecting the neighbouring warp's
+    // value in the end lanes, took twelve instructions).
+    const float4* e_l = &s_bstage[wL].e0[0][lL];
+    const float4* e_r = &s_bstage[wR].e0[0][lR];
+    auto x_nbrs = [&](int slot, int lev, float& sL, float& cL, float& sR, float& cR) {
+        const float2 l = *(reinterpret_cast<const float2*>(e_l + (3 * lev + slot) * 32) + 1);
+        const float2 r = *reinterpret_cast<const float2*>(e_r + (3 * lev + slot) * 32);
+        sL = l.x;
+        cL = l.y;
+        sR = r.x;
+        cR = r.y;
     };
     auto publish = [&](const P4& Cs, const P4& Cc, int slot, int lev) {
-        if (WIDE && (at_l || at_r))
-            e_wr[slot * kSlot + lev * kLevel] = make_float2(at_l ? Cs.a.x : Cs.b.y, at_l ? Cc.a.x : Cc.b.y);
+        (lev ? stg.e1 : stg.e0)[slot][lane] = make_float4(Cs.a.x, Cc.a.x, Cs.b.y, Cc.b.y);
     };
+    // The ends of iteration i are published in slot i % 3 before its barrier (a
+    // narrow band's warp: before its __syncwarp) and read after it, in iteration
+    // i + 1.  Blocks of up to 8 warps meet at a block barrier there.  In wider ones
+    // the warps would wait for the slowest of all every row (256 x 256 5.1e11
+    // site-updates/s with two warps, 2048 x 2048 4.3e11 with sixteen), so arrival
+    // and wait are apart: phase i completes when every warp has published
+    // iteration i, and a warp may run up to most of a row ahead (2048 x 2048
+    // 4.8e11; 1024 x 1024 the same either way; two warps 4.8e11, the wait being
+    // dearer than a barrier).  Slot i % 3 is written again in iteration i + 3: its
+    // level 0 after the wait for phase i + 1, which every warp reaches after
+    // reading level 0 of slot i, its level 1 after the wait for phase i + 2, which
+    // is after reading level 1 of slot i.
+    auto edges_published = [&]() {
+        __syncwarp();
+        if (APART && lane == 0) mbar_arrive(&s_bar);
+    };
+    auto edges_ready = [&](int phase) {
+        if (!WIDE) return;
+        if (!APART) __syncthreads();
+        else if (!mbar_wait(&s_bar, (uint32_t)(phase & 1)) && lane == 0) atomicExch(cap->err, XY_ETIMEOUT);
+    };
+    const int own2 = two ? own : 0;  // rows of level 2 that this lane writes
     float pm = 0.f, pe = 0.f;
     const float2 Jk = SCHED ? couplings_at(cf, k) : make_float2(cf.Jx, cf.Jy);
     const float hk = SCHED ? field_h(cf, k) : cf.h;
@@ -780,25 +836,33 @@ __global__ void __launch_bounds__(512, 1) band_step_kernel(const DevCfg* cfgs, c
     const bool stag = cf.stag != 0;
     R0 r0[3];
     R1 r1[3];
+    // noise of the quad of a row at offset o
+    auto noise = [&](int o, int64_t kk, float c) {
+        return p4(gauss4_scaled(philox4x32_10_rk(noise_counter((uint32_t)(o + x) >> 2, cfgrep, kk, 0u), keys), c));
+    };
+    o_a = (y0 + Ly - 1) % Ly * Lx;
+    P4 cn1 = noise(o_a, k, c1), cn2;
     // iteration i: P0, C0, N0 = level-0 rows y - 2, y - 1, y; P1, C1, N1 =
-    // level-1 rows b - 1, b, a (N1 computed here); levels: how many there are yet
+    // level-1 rows b - 1, b, a (N1 computed here); levels: how many there are yet.
+    // The wait and the two wrap tests cut the iteration into blocks of straight
+    // code; each of the two updates, a chain of dependent instructions, gets the
+    // noise that the other one needs next to fill it.
     auto body = [&](auto levels, int i, int slot, R0& P0, R0& C0, R0& N0, R1& P1, R1& C1, R1& N1) {
         constexpr int LV = decltype(levels)::value;
         issue(i + kBStages - 1, slot == 0 ? kBStages - 1 : slot - 1);
         cp_async_wait<kBStages - 1>();  // this lane's copies of iteration i have landed
-        const int cur = i & 1, prev = cur ^ 1;
+        const int prev = slot == 0 ? 2 : slot - 1;
         N0.th = p4(stg.th[slot][lane]);
-        float4 cn1, cn2;
-        if (LV >= 1) cn1 = gauss4_scaled(philox4x32_10_rk(noise_counter((uint32_t)(o_a + x) >> 2, cfgrep, k, 0u), keys), c1);
-        if (LV >= 2)
-            cn2 = gauss4_scaled(philox4x32_10_rk(noise_counter((uint32_t)(o_b + x) >> 2, cfgrep, k + 1, 0u), keys), c2);
         quad_sc(K1.q, N0.th, N0.s, N0.c);
-        publish(N0.s, N0.c, cur, 0);
+        publish(N0.s, N0.c, slot, 0);
+        if (i > 0) edges_ready(i - 1);
+        if (LV == 0) edges_published();
         if (LV >= 1) {  // level 1 on row a = y - 1
             const P4 va = p4(stg.v[slot][lane]);
             float sL, cL, sR, cR;
-            x_nbrs(C0.s, C0.c, prev, 0, sL, cL, sR, cR);
-            const QuadOut o = quad_update(K1, C0.th, va, p4(cn1), C0.s, C0.c, sL, cL, sR, cR, P0.s, P0.c, N0.s, N0.c);
+            x_nbrs(prev, 0, sL, cL, sR, cR);
+            if (LV >= 2) cn2 = noise(o_b, k + 1, c2);
+            const QuadOut o = quad_update(K1, C0.th, va, cn1, C0.s, C0.c, sL, cL, sR, cR, P0.s, P0.c, N0.s, N0.c);
             N1.th = o.theta;
             N1.v = o.v;
             const int ra = i - 3;  // row of the band
@@ -818,31 +882,30 @@ __global__ void __launch_bounds__(512, 1) band_step_kernel(const DevCfg* cfgs, c
                     }
                 }
             }
-            if (two) {
-                quad_sc(K1.q, N1.th, N1.s, N1.c);
-                publish(N1.s, N1.c, cur, 1);
-            } else if (ra >= 0 && ra < own) {
+            quad_sc(K1.q, N1.th, N1.s, N1.c);
+            publish(N1.s, N1.c, slot, 1);
+            edges_published();
+            if (!two && ra >= 0 && ra < own) {
                 st4_stream(thD + o_a, f4(N1.th));
                 st4_stream(omD + o_a, f4(N1.v));
             }
             o_a = next_row(o_a);
+            cn1 = noise(o_a, k, c1);
         }
-        if (LV >= 2 && two) {  // level 2 on row b = y - 2
+        if (LV >= 2) {  // level 2 on row b = y - 2 (dropped by a launch of one step)
             float sL, cL, sR, cR;
-            x_nbrs(C1.s, C1.c, prev, 1, sL, cL, sR, cR);
-            const QuadOut o = quad_update(K2, C1.th, C1.v, p4(cn2), C1.s, C1.c, sL, cL, sR, cR, P1.s, P1.c, N1.s, N1.c);
-            if (i - 4 < own) {
+            x_nbrs(prev, 1, sL, cL, sR, cR);
+            const QuadOut o = quad_update(K2, C1.th, C1.v, cn2, C1.s, C1.c, sL, cL, sR, cR, P1.s, P1.c, N1.s, N1.c);
+            if (i - 4 < own2) {
                 st4_stream(thD + o_b, f4(o.theta));
                 st4_stream(omD + o_b, f4(o.v));
             }
             o_b += Lx;
         }
-        if (WIDE) __syncthreads();  // edges of this iteration visible; the slot read here free for the next
     };
     using L0 = std::integral_constant<int, 0>;
     using L1 = std::integral_constant<int, 1>;
     using L2 = std::integral_constant<int, 2>;
-    o_a = (y0 + Ly - 1) % Ly * Lx;
     body(L0{}, 0, 0, r0[1], r0[2], r0[0], r1[1], r1[2], r1[0]);
     body(L0{}, 1, 1, r0[2], r0[0], r0[1], r1[2], r1[0], r1[1]);
     body(L1{}, 2, 2, r0[0], r0[1], r0[2], r1[0], r1[1], r1[2]);
@@ -892,16 +955,17 @@ cudaError_t launch_band_step(const DevCfg* d_cfg, const BandTask* tasks, int n_t
     if (!band_shape(Lx, 1) || H < 1) return cudaErrorInvalidValue;
     using Kern = void (*)(const DevCfg*, const BandTask*, int, int, int, int64_t, Buffers, const CallArgs*, Partials,
                           PhiloxKeys);
-    static const Kern table[2][2][3] = {
-        {{band_step_kernel<false, 0, false>, band_step_kernel<false, 1, false>, band_step_kernel<false, 2, false>},
-         {band_step_kernel<false, 0, true>, band_step_kernel<false, 1, true>, band_step_kernel<false, 2, true>}},
-        {{band_step_kernel<true, 0, false>, band_step_kernel<true, 1, false>, band_step_kernel<true, 2, false>},
-         {band_step_kernel<true, 0, true>, band_step_kernel<true, 1, true>, band_step_kernel<true, 2, true>}},
+#define BAND_ROW(W, A, S) {band_step_kernel<W, A, 0, S>, band_step_kernel<W, A, 1, S>, band_step_kernel<W, A, 2, S>}
+    static const Kern table[3][2][3] = {
+        {BAND_ROW(false, false, false), BAND_ROW(false, false, true)},
+        {BAND_ROW(true, false, false), BAND_ROW(true, false, true)},
+        {BAND_ROW(true, true, false), BAND_ROW(true, true, true)},
     };
-    const Kern kern = table[Lx > 128 ? 1 : 0][sched ? 1 : 0][rec < 0 ? 0 : (rec > 2 ? 2 : rec)];
+#undef BAND_ROW
+    const Kern kern = table[Lx <= 128 ? 0 : (Lx <= 1024 ? 1 : 2)][sched ? 1 : 0][rec < 0 ? 0 : (rec > 2 ? 2 : rec)];
     const int warps = Lx > 128 ? (Lx + 127) / 128 : kNarrowBandWarps;
     const size_t smem = sizeof(BStage) * (size_t)warps;
-    if (smem > 46 * 1024) {  // 16 warps: with the static part above the default limit
+    if (smem > 46 * 1024) {  // 8 warps or more: with the static part above the default limit
         const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
     }
