@@ -285,20 +285,42 @@ struct xy_lattice {
     void* ccl_buf = nullptr;
     int64_t ccl_bytes = 0;
     int64_t ccl_clean = 0;
-    // working memory of the adjoint, kept between calls (each slot grown on
-    // demand, all freed with the object): checkpoints, segment states,
-    // adjoint states, records, gradient partials, partials of M, band tasks
+    // working memory kept between calls (each slot grown on demand, all freed
+    // with the object), of the adjoint: checkpoints, segment states, adjoint
+    // states, records, gradient partials, partials of M, band tasks; of the
+    // structure factors: the table of lattices (written once), partial sums
     struct DevSlot {
         void* p = nullptr;
         size_t cap = 0;
     };
-    enum { kAdjCk, kAdjSbuf, kAdjSeg, kAdjB, kAdjFb, kAdjRec, kAdjGacc, kAdjMpart, kAdjTasks, kAdjSlots };
-    DevSlot adj_slot[kAdjSlots];
+    enum { kAdjCk, kAdjSbuf, kAdjSeg, kAdjB, kAdjFb, kAdjRec, kAdjGacc, kAdjMpart, kAdjTasks, kSfLats, kSfPart, kSlots };
+    DevSlot slot[kSlots];
 };
 
 namespace {
 
 Buffers state_buffers(const xy_lattice* L) { return Buffers{L->thA, L->omA, L->thB, L->omB}; }
+
+// At least `bytes` of slot i of the object's working memory (reallocated
+// only when it must grow; cudaFree waits for the device, so no launch still
+// uses the old block).
+cudaError_t reserve_slot(xy_lattice* L, int i, size_t bytes, void** out)
+{
+    xy_lattice::DevSlot& sl = L->slot[i];
+    if (bytes > sl.cap) {
+        cudaFree(sl.p);
+        sl.p = nullptr;
+        sl.cap = 0;
+        const cudaError_t e = cudaMalloc(&sl.p, bytes);
+        if (e != cudaSuccess) {
+            sl.p = nullptr;
+            return e;
+        }
+        sl.cap = bytes;
+    }
+    *out = sl.p;
+    return cudaSuccess;
+}
 
 int upload_cfg(xy_lattice* L)
 {
@@ -1393,7 +1415,7 @@ void free_lattice(xy_lattice* L)
     cudaFree(L->d_moments);
     cudaFree(L->rec_buf);
     cudaFree(L->ccl_buf);
-    for (auto& sl : L->adj_slot) cudaFree(sl.p);
+    for (auto& sl : L->slot) cudaFree(sl.p);
     cudaFree(L->d_err);
     if (L->cap_stream) cudaStreamDestroy(L->cap_stream);
     for (int i = 0; i < xy_lattice::kBranches; ++i) {
@@ -1860,17 +1882,39 @@ int xy_structure_factor(xy_lattice* L, int b_first, int b_count, int K, double r
         return fail(XY_EINVAL, "lattice range out of bounds");
     if (K < 1) return fail(XY_EINVAL, "K must be >= 1");
     if (!std::isfinite(rotor)) return fail(XY_EINVAL, "rotor multiplicity must be finite");
-    std::vector<int64_t> off((size_t)b_count);
-    std::vector<int> lx((size_t)b_count), ly((size_t)b_count);
+    int max_x = 0, max_y = 0;
     for (int c = 0; c < L->n_cfg; ++c) {
         const DevCfg& d = L->h_dev[c];
         const int lo = std::max(b_first, d.b_first), hi = std::min(b_first + b_count, d.b_first + d.n_rep);
-        for (int b = lo; b < hi; ++b) {
-            if (K > std::min(d.Lx, d.Ly)) return fail(XY_EINVAL, "K = %d exceeds min(Lx, Ly) of lattice %d", K, b);
-            if (d.Lx > 8192 || d.Ly > 8192) return fail(XY_EINVAL, "structure factors need Lx, Ly <= 8192");
-            off[(size_t)(b - b_first)] = d.offset + (int64_t)(b - d.b_first) * d.N;
-            lx[(size_t)(b - b_first)] = d.Lx;
-            ly[(size_t)(b - b_first)] = d.Ly;
+        if (lo >= hi) continue;
+        if (K > std::min(d.Lx, d.Ly)) return fail(XY_EINVAL, "K = %d exceeds min(Lx, Ly) of lattice %d", K, lo);
+        if (d.Lx > 8192 || d.Ly > 8192) return fail(XY_EINVAL, "structure factors need Lx, Ly <= 8192");
+        max_x = std::max(max_x, d.Lx);
+        max_y = std::max(max_y, d.Ly);
+    }
+    // the table of all lattices and the partial sums stay on the object (grown on
+    // demand; cudaFree waits for the device, so no launch still uses the old block)
+    void *lats = nullptr, *scratch = nullptr;
+    if (!L->slot[xy_lattice::kSfLats].p) {
+        std::vector<SfLattice> h;
+        h.reserve((size_t)L->B);
+        for (const DevCfg& d : L->h_dev)
+            for (int r = 0; r < d.n_rep; ++r) h.push_back(SfLattice{d.offset + r * d.N, d.Lx, d.Ly});
+        cudaError_t e0 = reserve_slot(L, xy_lattice::kSfLats, sizeof(SfLattice) * h.size(), &lats);
+        if (e0 == cudaSuccess) e0 = cudaMemcpy(lats, h.data(), sizeof(SfLattice) * h.size(), cudaMemcpyHostToDevice);
+        if (e0 != cudaSuccess) {
+            cudaGetLastError();
+            cudaFree(L->slot[xy_lattice::kSfLats].p);
+            L->slot[xy_lattice::kSfLats] = {};
+            return fail(XY_ENOMEM, "structure factor tables: %s", cudaGetErrorString(e0));
+        }
+    }
+    lats = L->slot[xy_lattice::kSfLats].p;
+    {
+        const cudaError_t e0 = reserve_slot(L, xy_lattice::kSfPart, sf_scratch_bytes(b_count, max_x, max_y, K), &scratch);
+        if (e0 != cudaSuccess) {
+            cudaGetLastError();
+            return fail(XY_ENOMEM, "structure factor partial sums: %s", cudaGetErrorString(e0));
         }
     }
     const bool dev = is_device_ptr(S_par) && is_device_ptr(S_perp);
@@ -1885,8 +1929,8 @@ int xy_structure_factor(xy_lattice* L, int b_first, int b_count, int K, double r
         dq = dp + (size_t)b_count * K;
     }
     int launches = 0;
-    cudaError_t e = launch_structure_factor(L->thA, off.data(), lx.data(), ly.data(), b_count, K, (float)rotor, dp, dq,
-                                            &launches, L->stream);
+    cudaError_t e = launch_structure_factor(L->thA, static_cast<const SfLattice*>(lats) + b_first, b_count, max_x, max_y, K,
+                                            (float)rotor, scratch, dp, dq, &launches, L->stream);
     L->launches += launches;
     if (e == cudaSuccess && !dev) {
         e = cudaMemcpyAsync(S_par, dp, bytes, cudaMemcpyDeviceToHost, L->stream);
@@ -1899,27 +1943,6 @@ int xy_structure_factor(xy_lattice* L, int b_first, int b_count, int K, double r
         return fail(XY_ECUDA, "structure factor: %s", cudaGetErrorString(e));
     }
     return XY_OK;
-}
-
-// At least `bytes` of slot i of the adjoint's working memory (reallocated
-// only when it must grow; cudaFree waits for the device, so no launch still
-// uses the old block).
-cudaError_t adj_reserve(xy_lattice* L, int i, size_t bytes, void** out)
-{
-    xy_lattice::DevSlot& sl = L->adj_slot[i];
-    if (bytes > sl.cap) {
-        cudaFree(sl.p);
-        sl.p = nullptr;
-        sl.cap = 0;
-        const cudaError_t e = cudaMalloc(&sl.p, bytes);
-        if (e != cudaSuccess) {
-            sl.p = nullptr;
-            return e;
-        }
-        sl.cap = bytes;
-    }
-    *out = sl.p;
-    return cudaSuccess;
 }
 
 int xy_adjoint_step_n(xy_lattice* L, int64_t n, int K, double wE, double wM, double* objective, double* grads)
@@ -2024,7 +2047,7 @@ int xy_adjoint_step_n(xy_lattice* L, int64_t n, int K, double wE, double wM, dou
     // the buffers are slots of the object's working memory, kept for the next call
     auto reserve = [&](int i, size_t bytes, auto** out) {
         void* p = nullptr;
-        const cudaError_t e1 = adj_reserve(L, i, bytes, &p);
+        const cudaError_t e1 = reserve_slot(L, i, bytes, &p);
         *out = static_cast<std::remove_reference_t<decltype(**out)>*>(p);
         return e1;
     };

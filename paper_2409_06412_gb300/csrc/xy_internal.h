@@ -283,10 +283,16 @@ cudaError_t launch_segment_m(const DevCfg* d_cfg, int n_cfg, int64_t B, const fl
 // Autocorrelation time of recorded series (xy_tau.cu); out: device, 4 * n_series doubles
 cudaError_t launch_autocorr(const double2* rec, int64_t n_series, int64_t R, int component, int transform,
                             int64_t skip, int n, double c_win, int half_window, double* out, cudaStream_t st);
-// Structure factors (xy_sf.cu) of n_lat lattices starting at theta +
-// offsets[b], shapes Lx[b] x Ly[b]; S_par, S_perp: device, n_lat * K doubles
-cudaError_t launch_structure_factor(const float* theta, const int64_t* offsets, const int* Lx, const int* Ly,
-                                    int n_lat, int K, float r, double* S_par, double* S_perp, int* n_launches,
+// Structure factors (xy_sf.cu) of n_lat lattices (device table `lats`, sides at
+// most max_x, max_y); scratch: sf_scratch_bytes() bytes; S_par, S_perp: device,
+// n_lat * K doubles
+struct SfLattice {
+    int64_t offset;  // first site of the lattice in the state buffer
+    int Lx, Ly;
+};
+size_t sf_scratch_bytes(int n_lat, int max_x, int max_y, int K);
+cudaError_t launch_structure_factor(const float* theta, const SfLattice* lats, int n_lat, int max_x, int max_y, int K,
+                                    float r, void* scratch, double* S_par, double* S_perp, int* n_launches,
                                     cudaStream_t st);
 cudaError_t launch_adjoint_band(const DevCfg* d_cfg, const BandTask* tasks, int n_tasks, int Lx, int H, uint64_t seed,
                                 BandArgs R, cudaStream_t st);
