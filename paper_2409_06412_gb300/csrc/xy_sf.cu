@@ -318,10 +318,11 @@ cudaError_t launch_structure_factor(const float* theta, const SfLattice* lats, i
     const size_t smem_x = max_x * sizeof(float2);
     const size_t smem_y = std::max(max_y * sizeof(float2), (size_t)4 * 2 * kKC * 32 * sizeof(float2));
     cudaError_t e = cudaSuccess;
-    if (smem_x > 48 * 1024)
-        e = cudaFuncSetAttribute(sf_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_x);
-    if (e == cudaSuccess && smem_y > 48 * 1024)
-        e = cudaFuncSetAttribute(sf_cols_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_y);
+    constexpr int smem_max = 8192 * (int)sizeof(float2);  // (the limit belongs to the kernel: always the largest)
+    if (smem_x > 46 * 1024)
+        e = cudaFuncSetAttribute(sf_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max);
+    if (e == cudaSuccess && smem_y > 46 * 1024)
+        e = cudaFuncSetAttribute(sf_cols_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max);
     if (e != cudaSuccess) return e;
     sf_rows_kernel<<<dim3((unsigned)n_lat, (unsigned)n_rc, (unsigned)n_kc), 256, smem_x, st>>>(theta, lats, r, p_rows, n_rc);
     sf_cols_kernel<<<dim3((unsigned)n_lat, (unsigned)n_cc, (unsigned)n_kc), 256, smem_y, st>>>(theta, lats, r, p_cols, n_cc);

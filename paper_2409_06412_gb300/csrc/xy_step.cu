@@ -966,7 +966,9 @@ cudaError_t launch_band_step(const DevCfg* d_cfg, const BandTask* tasks, int n_t
     const int warps = Lx > 128 ? (Lx + 127) / 128 : kNarrowBandWarps;
     const size_t smem = sizeof(BStage) * (size_t)warps;
     if (smem > 46 * 1024) {  // 8 warps or more: with the static part above the default limit
-        const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        // (the limit belongs to the kernel, which other shapes share: always the largest)
+        const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                   (int)sizeof(BStage) * kBandWarps);
         if (e != cudaSuccess) return e;
     }
     kern<<<(unsigned)n_tasks, 32 * warps, smem, st>>>(d_cfg, tasks, H, n_steps, rd_b ? 1 : 0,
