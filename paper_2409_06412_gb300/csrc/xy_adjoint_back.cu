@@ -26,6 +26,8 @@
 // when it reads that adjoint: every launch writes per-block partial sums of
 // M_k into a two-slot ring, and the next one sums them in a fixed order,
 // records M_k and applies the deferred term.
+#include <type_traits>
+
 #include "xy_device.cuh"
 
 namespace xy {
@@ -34,30 +36,15 @@ namespace {
 
 constexpr unsigned kFullB = 0xFFFFFFFFu;
 constexpr int kMaxBackWarps = 16;  // Lx <= 2048
+constexpr int kStages = 3;
 
 __device__ __forceinline__ int wrapb(int v, int n) { return v < 0 ? v + n : (v >= n ? v - n : v); }
 
-__device__ __forceinline__ void sc_b(float q, float th, float& s, float& c) { __sincosf(__fmul_rn(q, th), &s, &c); }
-
-struct SCb {
-    float s[4], c[4];
-};
-
-__device__ __forceinline__ void scb4(float q, const float4& t, SCb& r)
-{
-    sc_b(q, t.x, r.s[0], r.c[0]);
-    sc_b(q, t.y, r.s[1], r.c[1]);
-    sc_b(q, t.z, r.s[2], r.c[2]);
-    sc_b(q, t.w, r.s[3], r.c[3]);
-}
+__device__ __forceinline__ P4 sub4(const P4& x, const P4& y) { return fma4(-1.0f, y, x); }
 
 // theta_k = wrap(theta_{k+1} - dt v_{k+1}): the drift of step k undone, with
 // one explicit rounding so that every block recovering a row gets its bits
-__device__ __forceinline__ float4 undrift(const float4& t1, const float4& v1, float dt)
-{
-    return make_float4(wrap_angle(fmaf(-dt, v1.x, t1.x)), wrap_angle(fmaf(-dt, v1.y, t1.y)),
-                       wrap_angle(fmaf(-dt, v1.z, t1.z)), wrap_angle(fmaf(-dt, v1.w, t1.w)));
-}
+__device__ __forceinline__ P4 undrift(const P4& t1, const P4& v1, float dt) { return wrap_angle4(fma4(-dt, v1, t1)); }
 
 __device__ __forceinline__ float warp_sumf_b(float v)
 {
@@ -66,6 +53,21 @@ __device__ __forceinline__ float warp_sumf_b(float v)
     return v;
 }
 
+// Shared memory of one warp: the rows in flight (by iteration % 3), and the ends
+// of its lanes' quads for the lanes beside (by iteration % 3).
+struct BackWarp {
+    float4 th[kStages][32], v[kStages][32], tb[kStages][32], vb[kStages][32];
+    float4 sc[3][32];           // (sin q t, cos q t) of the first and of the last site
+    float4 fb[3][32], bx[3][32];  // F-bar, and the bond cosines to the column x + 1
+    float4 th0[2][32];          // theta_k, for the lane's own next iteration (by iteration % 2)
+    float4 tbp[2][32];          // adjoint of theta without the Hessian stencil, likewise
+};
+
+// (sin q t, cos q t) of a row of theta_k
+struct RowK {
+    P4 s, c;
+};
+
 }  // namespace
 
 // WIDE: Lx > 128 (a block spans one band of Lx / 128 strips); OBS: k > k0;
@@ -73,71 +75,76 @@ __device__ __forceinline__ float warp_sumf_b(float v)
 // launch but the first, which reads the final state itself); SCHED: some
 // configuration of the launch has a field or coupling schedule (without one
 // the step's constants are the configuration's own and no knot is searched).  At 128
-// registers an SM partition holds four warps (16 per SM), enough for bands
-// of 16 rows on 64 lattices of 256 x 256 to run in one wave.
+// registers an SM partition holds four warps (16 per SM).
+//
+// What bounds it: the issue slots that dependent instructions leave empty; a row
+// moves 32 bytes per site, which the launch needs a third of its time for.  So the
+// four sites of a lane go as packed pairs, the sums for the gradient too; the
+// stencil of phase B is formed from fluxes, each bond's term once (up and down, a
+// row's flux is kept for the next one); quads' ends cross lanes and warps through
+// shared memory, where a row's results wait for the next one too (eight pointers
+// and twelve more values in registers spilled); and the noise of the next row is
+// formed beside phase B, whose chain is short of independent work.  Unrolled by
+// three, without copies of the window, the loop outgrew the instruction cache and
+// gained nothing.  64 lattices of 256 x 256, 8-row bands, four slices at once: 200 ->
+// 136 instructions per site, 35.8 -> 28.1 us per step (half of the issue slots).
 template <bool WIDE, bool OBS, bool BACK, bool SCHED>
 __global__ void __launch_bounds__(512, 1) adjoint_back_kernel(const DevCfg* cfgs, const BandTask* tasks, int H,
                                                               BackArgs R, PhiloxKeys keys)
 {
-    // per warp, two stages of [theta_in(t+1), v_in, tb(t), vb(t)] for its 32 lanes
-    extern __shared__ float4 s_stage[];
-    // edge slots of the wide bands, four rows deep: a slot last read in phase B
-    // of row t + 1 is rewritten for row t + 4, in the phase A of a warp that has
-    // passed the barrier of row t + 2, after every warp's phase B of row t + 1
-    __shared__ float2 s_sc[4][kMaxBackWarps][2];
-    __shared__ float s_fb[4][kMaxBackWarps][2];
-    __shared__ float s_bx[4][kMaxBackWarps];  // bond cosine of a strip's last site to the next strip
+    extern __shared__ BackWarp s_warps[];
     __shared__ double s_red[kGacc + 1][kMaxBackWarps];
     __shared__ float s_wm1;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, n_warps = blockDim.x >> 5;
     const BandTask task = tasks[blockIdx.x];
     const DevCfg& cf = cfgs[task.cfg];
     const int Lx = cf.Lx, Ly = cf.Ly;
-    constexpr bool wide = WIDE;
-    const int G = Lx >= 128 ? 32 : (Lx >> 2);
+    const int G = WIDE ? 32 : (Lx >> 2);
     const int groups = 32 / G;
     const int grp = lane / G, lg = lane - grp * G;
-    const int per_block = wide ? 1 : n_warps * groups;  // bands per block
-    const int band_raw = wide ? task.band0 : task.band0 + warp * groups + grp;
+    const int per_block = WIDE ? 1 : n_warps * groups;  // bands per block
+    const int band_raw = WIDE ? task.band0 : task.band0 + warp * groups + grp;
     // lane groups past the last band recompute the last band (so every shuffle
     // and barrier runs converged) and store nothing
     const bool active = band_raw < task.n_bands;
     const int band = active ? band_raw : task.n_bands - 1;
-    const int x = (wide ? warp * 128 : 0) + 4 * lg;
+    const int x = (WIDE ? warp * 128 : 0) + 4 * lg;
     const int y0 = band * H;
-    const int srcL = grp * G + (lg + G - 1) % G, srcR = grp * G + (lg + 1) % G;
-    const int wl = (warp + n_warps - 1) % n_warps, wr = (warp + 1) % n_warps;  // neighbour strips (wide)
+    // warp and lane of the quads beside
+    const int wL = WIDE && lane == 0 ? (warp + n_warps - 1) % n_warps : warp;
+    const int wR = WIDE && lane == 31 ? (warp + 1) % n_warps : warp;
+    const int lL = grp * G + (lg + G - 1) % G, lR = grp * G + (lg + 1) % G;
     const int64_t b = cf.b_first + task.rep;
-    const int64_t lat_off = cf.offset + (int64_t)task.rep * cf.N;
+    // one pointer and the other arrays' distances from it, which stay kernel
+    // parameters: eight pointers would take sixteen registers
+    char* const base = (char*)(R.th_in + cf.offset + (int64_t)task.rep * cf.N + x);
+    auto at = [&](int64_t dist, int o) { return reinterpret_cast<float*>(base + dist + 4 * (int64_t)o); };
     const int slot_j = task.band0 / per_block;  // this block's partial of M
     const int n_parts = (task.n_bands + per_block - 1) / per_block;
-    const float* thI = R.th_in + lat_off;
-    const float* vI = R.v_in + lat_off;
-    float* thO = BACK ? R.th_out + lat_off : nullptr;
-    float* vO = BACK ? R.v_out + lat_off : nullptr;
-    const float* tbI = R.tb_in + lat_off;
-    const float* vbI = R.vb_in + lat_off;
-    float* tbO = R.tb_out + lat_off;
-    float* vbO = R.vb_out + lat_off;
     const StepConst K = SCHED ? step_const_k(cf, R.k, noise_amp(cf, R.k)) : step_const(cf, noise_amp(cf, R.k));
     const float q2 = K.q * K.q, hp2 = K.hp * cf.p;
     const float invN = 1.0f / (float)cf.N, wE = R.wE;
-    constexpr bool observe = OBS, first = !OBS;
     const uint32_t cfgrep = ((uint32_t)cf.noise_cfg << 16) | (uint32_t)(cf.rep0 + task.rep);
+    auto noise = [&](int o) {
+        return p4(gauss4_scaled(philox4x32_10_rk(noise_counter((uint32_t)(o + x) >> 2, cfgrep, R.k, 0u), keys), K.c));
+    };
+    P4 nz = noise(wrapb(y0 - 1, Ly) * Lx);
+    dependency_wait();  // the states, adjoints and partial sums of the launch before
     // M_{k+1} from the previous launch's partials (fixed order), recorded by
     // the lattice's first block; its sign weights the deferred |M| term
-    if (threadIdx.x == 0) {
+    if (warp == 0) {
         float w = 0.f;
         if (BACK) {
             const double* mp = R.mpart + (b * 2 + ((R.k + 1) & 1)) * R.P;
             double m = 0.0;
-            for (int j = 0; j < n_parts; ++j) m += mp[j];
+            for (int j = lane; j < n_parts; j += 32) m += mp[j];
+            for (int o = 1; o < 32 && o < n_parts; o <<= 1) m += __shfl_xor_sync(kFullB, m, o);
             m /= (double)cf.N;
-            if (slot_j == 0) R.rec[b * R.rec_stride + (R.k + 1 - R.k0)].x = m;
+            if (slot_j == 0 && lane == 0) R.rec[b * R.rec_stride + (R.k + 1 - R.k0)].x = m;
             const float wq = R.wM * invN * K.q;
             w = m > 0.0 ? wq : (m < 0.0 ? -wq : 0.f);
         }
-        s_wm1 = w;
+        if (lane == 0) s_wm1 = w;  // (lane 0 has the full sum at any number of parts)
     }
     // configuration constants in registers (the cp.async statements clobber
     // memory, which would otherwise reload them from the descriptor every row)
@@ -148,237 +155,200 @@ __global__ void __launch_bounds__(512, 1) adjoint_back_kernel(const DevCfg* cfgs
     const bool stag = cf.stag != 0;
     const float wEn = wE * invN;
     const float inv_oma = 1.0f / K.oma, opa = 2.0f - K.oma;  // 1 / (1 - a), 1 + a
-    float aJx = 0.f, aJy = 0.f, ah = 0.f, abar = 0.f, bbar = 0.f, cbar = 0.f;
-    float sw2 = 0.f, sbx = 0.f, sby = 0.f, scp = 0.f, pm = 0.f;
+    // per-lane sums, two sites each (both halves added at the end)
+    const float2 z2 = make_float2(0.f, 0.f);
+    float2 aJx = z2, aJy = z2, ah = z2, abar = z2, cbar = z2, sw2 = z2, sbx = z2, sby = z2, scp = z2, pm = z2;
+    auto dot = [&](float2& acc, const P4& u, const P4& w) { acc = __ffma2_rn(u.b, w.b, __ffma2_rn(u.a, w.a, acc)); };
+    auto add = [&](float2& acc, const P4& u) { acc = __fadd2_rn(acc, __fadd2_rn(u.a, u.b)); };
 
-    // window: S1 = row t-1, S2 = t, S3 = t+1 (of theta_k); F0 = F-bar(t-2), F1 = t-1;
-    // Bm2, Bm1: bond cosines cos q(theta_y - theta_{y+1}) of rows t-2 and t-1,
-    // formed in phase A and reused by the stencil of phase B
-    SCb S1, S2, S3;
-    float4 Bm2, Bm1;
-    float4 Bx1 = make_float4(0.f, 0.f, 0.f, 0.f);  // cos q(theta_x - theta_{x+1}) of row t-1
-    float4 F0 = make_float4(0.f, 0.f, 0.f, 0.f), F1 = F0;
-    float4 th2, tbp1 = F0;  // theta_k of row t; tb partial of row t-1 (site-local terms of phase B folded in)
-    float4 t1c = F0, v1c = F0;        // BACK: theta_{k+1}, v_{k+1} of row t
-    const int Nl = Lx * Ly;
-    auto rowp = [&](int y) { return wrapb(y, Ly) * Lx; };
-    auto adv = [&](int r) { return r + Lx == Nl ? 0 : r + Lx; };
-    int r_m1 = rowp(y0 - 2), r_0 = rowp(y0 - 1), r_p1 = rowp(y0), r_p2 = rowp(y0 + 1);
-    // slot of row y: (y - y0 + 8) & 3 (the block's rows share y0 in the wide layout)
-    int sl_0 = 3, sl_p1 = 0;
-    auto publish_sc = [&](int slot, const SCb& S) {
-        if (!wide) return;
-        if (lane == 0) s_sc[slot][warp][0] = make_float2(S.s[0], S.c[0]);
-        if (lane == 31) s_sc[slot][warp][1] = make_float2(S.s[3], S.c[3]);
-    };
-    auto nbr_sc = [&](int slot, const SCb& S, float& sL, float& cL, float& sR, float& cR) {
-        sL = __shfl_sync(kFullB, S.s[3], srcL);
-        cL = __shfl_sync(kFullB, S.c[3], srcL);
-        sR = __shfl_sync(kFullB, S.s[0], srcR);
-        cR = __shfl_sync(kFullB, S.c[0], srcR);
-        if (wide) {
-            if (lane == 0) { const float2 e = s_sc[slot][wl][1]; sL = e.x; cL = e.y; }
-            if (lane == 31) { const float2 e = s_sc[slot][wr][0]; sR = e.x; cR = e.y; }
+    const int N = Lx * Ly;
+    auto adv = [&](int r) { return r + Lx == N ? 0 : r + Lx; };
+    BackWarp& me = s_warps[warp];
+    // iteration i works on row t = y0 - 1 + i (phase A) and row t - 1 (phase B); its
+    // stage holds theta_in of row t + 1, v_in of row t + 1 (BACK) or t, tb and vb
+    // of row t
+    int o_ld = wrapb(y0, Ly) * Lx, o_ldt = wrapb(y0 - 1, Ly) * Lx;  // rows t + 1 and t of the next issue
+    const int n_it = H + 2;
+    auto issue = [&](int ii, int slot) {
+        if (ii < n_it) {
+            cp_async16(&me.th[slot][lane], at(0, o_ld));
+            cp_async16(&me.v[slot][lane], at(R.d_v_in, BACK ? o_ld : o_ldt));
+            cp_async16(&me.tb[slot][lane], at(R.d_tb_in, o_ldt));
+            cp_async16(&me.vb[slot][lane], at(R.d_vb_in, o_ldt));
+            o_ldt = o_ld;
+            o_ld = adv(o_ld);
         }
-    };
-    constexpr int kStage = 4 * 32;  // float4 per warp and stage
-    float4* my_stage = s_stage + (size_t)warp * 2 * kStage;
-    // stage st: theta_in of row offset rt, v_in of row offset rvin (BACK: row
-    // t + 1, else row t), tb and vb of row offset rv
-    auto prefetch = [&](int st, int rt, int rvin, int rv) {
-        float4* p = my_stage + st * kStage;
-        cp_async16(p + 0 * 32 + lane, thI + rt + x);
-        cp_async16(p + 1 * 32 + lane, vI + rvin + x);
-        cp_async16(p + 2 * 32 + lane, tbI + rv + x);
-        cp_async16(p + 3 * 32 + lane, vbI + rv + x);
         cp_async_commit();
     };
-    if (BACK) {
-        scb4(K.q, undrift(ld4(thI + r_m1 + x), ld4(vI + r_m1 + x), K.dt), S1);
-        t1c = ld4(thI + r_0 + x);
-        v1c = ld4(vI + r_0 + x);
-        th2 = undrift(t1c, v1c, K.dt);
-        prefetch(0, r_p1, r_p1, r_0);
-    } else {
-        scb4(K.q, ld4(thI + r_m1 + x), S1);
-        th2 = ld4(thI + r_0 + x);
-        prefetch(0, r_p1, r_0, r_0);
+    int o_a = o_ldt, o_b = 0;  // rows t and t - 1
+    issue(0, 0);
+    issue(1, 1);
+    const float4* sc_l = &s_warps[wL].sc[0][lL];
+    const float4* sc_r = &s_warps[wR].sc[0][lR];
+    const float* fb_l = &s_warps[wL].fb[0][lL].w;  // the bond cosines lie 3 * 32 float4 further
+    const float* fb_r = &s_warps[wR].fb[0][lR].x;
+    RowK k0, k1, k2;
+    P4 gy{z2, z2};  // flux between the rows t - 2 and t - 1
+    P4 bym;         // bond cosines between the rows t - 1 and t
+    {
+        // rows t - 1 and t of the first iteration
+        const int r_m1 = wrapb(y0 - 2, Ly) * Lx, r_0 = o_a;
+        P4 t0;
+        if (BACK) {
+            const P4 t = undrift(p4(ld4(at(0, r_m1))), p4(ld4(at(R.d_v_in, r_m1))), K.dt);
+            quad_sc(K.q, t, k1.s, k1.c);
+            // theta_{k+1}, v_{k+1} of row t stay in the last iteration's stage
+            me.th[2][lane] = ld4(at(0, r_0));
+            me.v[2][lane] = ld4(at(R.d_v_in, r_0));
+            t0 = undrift(p4(me.th[2][lane]), p4(me.v[2][lane]), K.dt);
+        } else {
+            quad_sc(K.q, p4(ld4(at(0, r_m1))), k1.s, k1.c);
+            t0 = p4(ld4(at(0, r_0)));
+        }
+        quad_sc(K.q, t0, k2.s, k2.c);
+        me.th0[1][lane] = f4(t0);
+        me.sc[2][lane] = make_float4(k2.s.a.x, k2.c.a.x, k2.s.b.y, k2.c.b.y);
+        bym = fma4(k1.c, k2.c, mul4(k1.s, k2.s));
+        me.fb[2][lane] = me.bx[2][lane] = me.tbp[1][lane] = make_float4(0.f, 0.f, 0.f, 0.f);
     }
-    scb4(K.q, th2, S2);
-    publish_sc(sl_0, S2);
-    Bm1 = make_float4(fmaf(S1.c[0], S2.c[0], S1.s[0] * S2.s[0]), fmaf(S1.c[1], S2.c[1], S1.s[1] * S2.s[1]),
-                      fmaf(S1.c[2], S2.c[2], S1.s[2] * S2.s[2]), fmaf(S1.c[3], S2.c[3], S1.s[3] * S2.s[3]));
-    Bm2 = Bm1;
-    __syncthreads();  // s_wm1, and the edge slots of the first rows
+    __syncthreads();  // s_wm1, and the ends of the first row
     const float wM1 = s_wm1;
-    for (int t = y0 - 1; t <= y0 + H; ++t) {
-        const bool own_a = active && t >= y0 && t < y0 + H;  // phase A results stored / accumulated
-        const bool do_b = t - 1 >= y0;                      // phase B on row t-1
-        const int st = (t - y0 + 1) & 1;
-        const int yw = wrapb(t, Ly);
-        if (BACK) prefetch(st ^ 1, r_p2, r_p2, r_p1);
-        else prefetch(st ^ 1, r_p2, r_p1, r_p1);
-        cp_async_wait<1>();  // this lane's copies of stage st have landed
-        const float4* sp = my_stage + st * kStage;
-        const float4 in3 = sp[0 * 32 + lane];
-        const float4 vin = sp[1 * 32 + lane];
-        float4 th3, v1n = vin;
-        if (BACK) th3 = undrift(in3, vin, K.dt);
-        else th3 = in3;
-        scb4(K.q, th3, S3);
-        publish_sc(sl_p1, S3);
-        // ---------------- phase A on row t
-        float4 Fn = make_float4(0.f, 0.f, 0.f, 0.f), tbpn = Fn, Bn = Fn, Bxn = Fn;
+    // Ends published in iteration i are read in iteration i + 1, on the other side
+    // of iteration i's barrier: those of (sin, cos) before iteration i + 1's, those
+    // of F-bar after it.  Three slots, so that what iteration i + 3 writes was read
+    // before the barrier of iteration i + 2.
+    // (P, C, D: theta_k of the rows t - 1, t, t + 1)
+    auto body = [&](int i, int slot, RowK& P, RowK& C, RowK& D) {
+        const int prev = slot == 0 ? 2 : slot - 1;
+        cp_async_wait<kStages - 2>();  // this lane's copies of iteration i have landed
+        const bool own = active && i >= 1 && i <= H;  // row t is the band's: stored and summed
+        const P4 in = p4(me.th[slot][lane]), vin = p4(me.v[slot][lane]);
+        const int own_slot = i & 1;
+        const P4 thC = p4(me.th0[own_slot ^ 1][lane]);
         {
-            float4 tb4 = sp[2 * 32 + lane];
-            const float4 vb4 = sp[3 * 32 + lane];
+            const P4 thD = BACK ? undrift(in, vin, K.dt) : in;
+            me.th0[own_slot][lane] = f4(thD);
+            quad_sc(K.q, thD, D.s, D.c);
+        }
+        me.sc[slot][lane] = make_float4(D.s.a.x, D.c.a.x, D.s.b.y, D.c.b.y);
+        // ---------------- phase A on row t
+        P4 tb = p4(me.tb[slot][lane]);
+        const P4 vb = p4(me.vb[slot][lane]);
+        const int yw = wrapb(y0 - 1 + i, Ly);
+        const float sgn = stag && (yw & 1) ? -1.f : 1.f;  // of the quad's sites 0 and 2 (x is a multiple of 4)
+        const float2 sg = make_float2(sgn, stag ? -sgn : sgn);
+        if (BACK) {
+            // deferred |M_{k+1}| term of the adjoint of theta_{k+1} (step
+            // k + 1 > k0 is always observed)
+            const P4 a = mul4(K.q, p4(me.th[prev][lane]));
+            const float2 w = __fmul2_rn(splat2(wM1), sg);
+            tb.a = __ffma2_rn(w, make_float2(__cosf(a.a.x), __cosf(a.a.y)), tb.a);
+            tb.b = __ffma2_rn(w, make_float2(__cosf(a.b.x), __cosf(a.b.y)), tb.b);
+        }
+        const float2 l = *(reinterpret_cast<const float2*>(sc_l + prev * 32) + 1);
+        const float2 r = *reinterpret_cast<const float2*>(sc_r + prev * 32);
+        const P4 &s = C.s, &c = C.c;
+        const P4 sx{make_float2(-l.x - s.a.y, -s.a.x - s.b.x), make_float2(-s.a.y - s.b.y, -s.b.x - r.x)};
+        const P4 cx{make_float2(l.y + c.a.y, c.a.x + c.b.x), make_float2(c.a.y + c.b.y, c.b.x + r.y)};
+        const P4 sy{make_float2(-P.s.a.x - D.s.a.x, -P.s.a.y - D.s.a.y), make_float2(-P.s.b.x - D.s.b.x, -P.s.b.y - D.s.b.y)};
+        const P4 cy = add4(P.c, D.c);
+        const P4 ax = fma4(s, cx, mul4(c, sx)), ay = fma4(s, cy, mul4(c, sy));
+        const P4 pt = mul4(K.p, thC);
+        P4 sp, cp;
+        __sincosf(pt.a.x, &sp.a.x, &cp.a.x);
+        __sincosf(pt.a.y, &sp.a.y, &cp.a.y);
+        __sincosf(pt.b.x, &sp.b.x, &cp.b.x);
+        __sincosf(pt.b.y, &sp.b.y, &cp.b.y);
+        const P4 F = fma4(K.nqJx, ax, fma4(K.nqJy, ay, mul4(K.hp, sp)));
+        const P4 g = fma4(K.hdt, F, nz);
+        P4 om, vk;  // omega_k, v_k
+        if (BACK) {
+            const P4 ng = mul4(-1.0f, g);
+            om = mul4(inv_oma, add4(p4(me.v[prev][lane]), ng));
+            vk = fma4(opa, om, ng);
+        } else {
+            vk = vin;
+            om = mul4(K.inv1pa, add4(vk, g));
+        }
+        issue(i + kStages - 1, prev);  // (the slot's theta_{k+1} and v_{k+1} have been read)
+        const P4 byn = fma4(c, D.c, mul4(s, D.s));  // bond to row t + 1
+        P4 bx;
+        bx.a = make_float2(fmaf(c.a.x, c.a.y, s.a.x * s.a.y), fmaf(c.a.y, c.b.x, s.a.y * s.b.x));  // to column x + 1
+        bx.b = make_float2(fmaf(c.b.x, c.b.y, s.b.x * s.b.y), fmaf(c.b.y, r.y, s.b.y * r.x));
+        const P4 vbt = fma4(K.dt, tb, vb);
+        P4 omb = mul4(K.oma, vbt), gb = vbt, vbk{z2, z2};
+        if (OBS) {
+            omb = fma4(wEn, om, omb);
+            tb = fma4(-wEn, F, tb);
+            vbk = mul4(K.inv1pa, omb);
+            gb = add4(gb, vbk);
+        }
+        const P4 fb = mul4(K.hdt, gb);
+        // the field's diagonal Hessian term of phase B, h p^2 cos(p t) F-bar, is site-local
+        me.tbp[own_slot][lane] = f4(fma4(mul4(hp2, cp), fb, tb));
+        me.fb[slot][lane] = f4(fb);
+        me.bx[slot][lane] = f4(bx);
+        if (own) {
+            pm = __ffma2_rn(sg, __fadd2_rn(s.a, s.b), pm);
+            if (OBS) {
+                dot(sw2, om, om);
+                add(sbx, bx);
+                add(sby, byn);
+                add(scp, cp);
+            }
+            dot(aJx, fb, ax);
+            dot(aJy, fb, ay);
+            dot(ah, fb, sp);
+            // the damping's two places, -om vbt from 1 - a and -om vbk from 1 / (1 + a)
+            // ((vk + g) / (1 + a)^2 is om / (1 + a)), in one sum
+            dot(abar, om, gb);
+            dot(cbar, gb, nz);
+            st4(at(R.d_vb_out, o_a), f4(vbk));
             if (BACK) {
-                // deferred |M_{k+1}| term of the adjoint of theta_{k+1} (step
-                // k + 1 > k0 is always observed); sites 0, 2 of a quad share
-                // the staggered sign of (x + y), sites 1, 3 take the other
-                const float wa = (stag && ((x + yw) & 1)) ? -wM1 : wM1;
-                const float wb = stag ? -wa : wa;
-                tb4.x = fmaf(wa, __cosf(K.q * t1c.x), tb4.x);
-                tb4.y = fmaf(wb, __cosf(K.q * t1c.y), tb4.y);
-                tb4.z = fmaf(wa, __cosf(K.q * t1c.z), tb4.z);
-                tb4.w = fmaf(wb, __cosf(K.q * t1c.w), tb4.w);
-            }
-            float sL, cL, sR, cR;
-            nbr_sc(sl_0, S2, sL, cL, sR, cR);
-            const uint32_t quad = (uint32_t)((r_0 + x) >> 2);
-            const float4 nz = gauss4_scaled(philox4x32_10_rk(noise_counter(quad, cfgrep, R.k, 0u), keys), K.c);
-            float tbo[4], vbo[4], fbo[4], vko[4], byo[4], bxo[4];
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const float s_ = S2.s[i], c_ = S2.c[i];
-                const float sl = i == 0 ? sL : S2.s[i - 1], cl = i == 0 ? cL : S2.c[i - 1];
-                const float sr = i == 3 ? sR : S2.s[i + 1], cr = i == 3 ? cR : S2.c[i + 1];
-                const float sx = sl + sr, cx = cl + cr;
-                const float sy = S1.s[i] + S3.s[i], cy = S1.c[i] + S3.c[i];
-                const float tht = f4get(th2, i);
-                const float sinp = __sinf(K.p * tht);
-                const float cp = __cosf(K.p * tht);
-                const float ax = fmaf(s_, cx, -c_ * sx), ay = fmaf(s_, cy, -c_ * sy);
-                const float F = fmaf(K.nqJx, ax, fmaf(K.nqJy, ay, K.hp * sinp));
-                const float cn = f4get(nz, i);
-                const float g = fmaf(K.hdt, F, cn);
-                float om, vk;  // omega_k, v_k
-                if (BACK) {
-                    om = (f4get(v1c, i) - g) * inv_oma;
-                    vk = fmaf(opa, om, -g);
-                } else {
-                    vk = f4get(vin, i);
-                    om = (vk + g) * K.inv1pa;
-                }
-                byo[i] = fmaf(c_, S3.c[i], s_ * S3.s[i]);  // bond to row t + 1
-                bxo[i] = fmaf(c_, cr, s_ * sr);            // bond to column x + 1
-                const float vbt = fmaf(K.dt, f4get(tb4, i), f4get(vb4, i));
-                float omb = K.oma * vbt;
-                float gb = vbt;
-                float tbi = f4get(tb4, i);
-                if (observe) {
-                    omb = fmaf(wEn, om, omb);
-                    tbi = fmaf(-wEn, F, tbi);
-                    if (own_a) {
-                        sw2 = fmaf(om, om, sw2);
-                        sbx += bxo[i];
-                        sby += byo[i];
-                        scp += cp;
-                    }
-                }
-                if (own_a) pm += (stag && ((x + i + yw) & 1)) ? -s_ : s_;
-                float vbk = 0.f;
-                if (!first) {
-                    vbk = K.inv1pa * omb;
-                    gb += vbk;
-                    if (own_a) bbar = fmaf(vk + g, omb, bbar);
-                }
-                const float fb = K.hdt * gb;
-                if (own_a) {
-                    aJx = fmaf(fb, ax, aJx);
-                    aJy = fmaf(fb, ay, aJy);
-                    ah = fmaf(fb, sinp, ah);
-                    abar = fmaf(-om, vbt, abar);
-                    cbar = fmaf(gb, cn, cbar);
-                }
-                // the field's diagonal Hessian term of phase B, h p^2 cos(p t) F-bar, is site-local
-                tbo[i] = fmaf(hp2 * cp, fb, tbi);
-                vbo[i] = vbk;
-                fbo[i] = fb;
-                vko[i] = vk;
-            }
-            if (own_a) {
-                st4(vbO + r_0 + x, make_float4(vbo[0], vbo[1], vbo[2], vbo[3]));
-                if (BACK) {
-                    st4(thO + r_0 + x, th2);
-                    st4(vO + r_0 + x, make_float4(vko[0], vko[1], vko[2], vko[3]));
-                }
-            }
-            Fn = make_float4(fbo[0], fbo[1], fbo[2], fbo[3]);
-            Bn = make_float4(byo[0], byo[1], byo[2], byo[3]);
-            Bxn = make_float4(bxo[0], bxo[1], bxo[2], bxo[3]);
-            tbpn = make_float4(tbo[0], tbo[1], tbo[2], tbo[3]);
-            if (wide) {
-                if (lane == 0) s_fb[(t - y0 + 8) & 3][warp][0] = Fn.x;
-                if (lane == 31) {
-                    s_fb[(t - y0 + 8) & 3][warp][1] = Fn.w;
-                    s_bx[(t - y0 + 8) & 3][warp] = Bxn.w;
-                }
+                st4(at(R.d_th_out, o_a), f4(thC));
+                st4(at(R.d_v_out, o_a), f4(vk));
             }
         }
-        if (wide) __syncthreads(); else __syncwarp();
-        // ---------------- phase B on row t - 1 (needs F-bar of rows t - 2, t - 1, t)
-        if (do_b) {
-            float fL = __shfl_sync(kFullB, F1.w, srcL), fR = __shfl_sync(kFullB, F1.x, srcR);
-            float kl0 = __shfl_sync(kFullB, Bx1.w, srcL);  // bond of the site to its left
-            if (wide) {
-                if (lane == 0) {
-                    fL = s_fb[(t - 1 - y0 + 8) & 3][wl][1];
-                    kl0 = s_bx[(t - 1 - y0 + 8) & 3][wl];
-                }
-                if (lane == 31) fR = s_fb[(t - 1 - y0 + 8) & 3][wr][0];
-            }
-            float out[4];
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const float fl = i == 0 ? fL : f4get(F1, i - 1), fr = i == 3 ? fR : f4get(F1, i + 1);
-                const float fj = f4get(F1, i);
-                const float kl = i == 0 ? kl0 : f4get(Bx1, i - 1), kr = f4get(Bx1, i);
-                const float ku = f4get(Bm2, i), kd = f4get(Bm1, i);
-                const float hx = fmaf(kl, fl - fj, kr * (fr - fj));
-                const float hy = fmaf(ku, f4get(F0, i) - fj, kd * (f4get(Fn, i) - fj));
-                out[i] = f4get(tbp1, i) + fmaf(q2Jx, hx, q2Jy * hy);
-            }
-            if (active) st4(tbO + r_m1 + x, make_float4(out[0], out[1], out[2], out[3]));
+        if (WIDE) __syncthreads(); else __syncwarp();
+        // ---------------- phase B on row t - 1 (F-bar of rows t - 2, t - 1, t), from
+        // the fluxes bond * (difference of F-bar) across its four bonds
+        const int o_n = adv(o_a);
+        nz = noise(o_n);  // of row t + 1
+        {
+            const float fl = fb_l[prev * 128], bl = fb_l[(3 + prev) * 128], fr = fb_r[prev * 128];
+            const P4 f = p4(me.fb[prev][lane]), bxf = p4(me.bx[prev][lane]);
+            const float el = bl * (f.a.x - fl);
+            const P4 e = mul4(bxf, P4{make_float2(f.a.y - f.a.x, f.b.x - f.a.y), make_float2(f.b.y - f.b.x, fr - f.b.y)});
+            const P4 hx{make_float2(e.a.x - el, e.a.y - e.a.x), make_float2(e.b.x - e.a.y, e.b.y - e.b.x)};
+            const P4 gn = mul4(bym, sub4(fb, f));
+            const P4 out = fma4(q2Jx, hx, fma4(q2Jy, sub4(gn, gy), p4(me.tbp[own_slot ^ 1][lane])));
+            gy = gn;
+            if (active && i >= 2) st4(at(R.d_tb_out, o_b), f4(out));
         }
-        // shift the windows
-        Bm2 = Bm1;
-        Bm1 = Bn;
-        Bx1 = Bxn;
-        S1 = S2;
-        S2 = S3;
-        th2 = th3;
-        t1c = in3;
-        v1c = v1n;
-        F0 = F1;
-        F1 = Fn;
-        tbp1 = tbpn;
-        r_m1 = r_0;
-        r_0 = r_p1;
-        r_p1 = r_p2;
-        r_p2 = adv(r_p2);
-        sl_0 = sl_p1;
-        sl_p1 = (sl_p1 + 1) & 3;
+        bym = byn;
+        o_b = o_a;
+        o_a = o_n;
+    };
+    int slot = 0;  // i % 3
+#pragma unroll 1
+    for (int i = 0; i < n_it; ++i) {
+        body(i, slot, k1, k2, k0);
+        k1 = k2;
+        k2 = k0;
+        slot = slot == 2 ? 0 : slot + 1;
     }
+    cp_async_wait<0>();
+    launch_next();
     // per-block accumulators: FP32 warp butterflies, the warps and the steps
     // combined in FP64 in a fixed order; the partial of M_k goes to the ring
+    auto both = [](float2 v) { return v.x + v.y; };
     const float vals[kGacc + 1] = {
-        fmaf(-K.q, aJx, -wEn * sbx) * abk.x,                                // d/d J_par (J_par(k) = J_par a(k))
-        fmaf(-K.q, aJy, -wEn * sby) * abk.y,                                // d/d J_perp (J_perp b(k))
-        fmaf(K.p, ah, wEn * scp) * (SCHED ? field_scale(cf, R.k) : 1.f),    // d/d h (h_k = h s(k))
-        abar, bbar, cbar,
-        wEn * fmaf(0.5f, sw2, fmaf(-Jx, sbx, fmaf(-Jy, sby, hF * scp))),  // w_E E / N
-        pm,                                                                 // sum of sigma sin(q theta_k)
+        fmaf(-K.q, both(aJx), -wEn * both(sbx)) * abk.x,                              // d/d J_par (J_par(k) = J_par a(k))
+        fmaf(-K.q, both(aJy), -wEn * both(sby)) * abk.y,                              // d/d J_perp (J_perp b(k))
+        fmaf(K.p, both(ah), wEn * both(scp)) * (SCHED ? field_scale(cf, R.k) : 1.f),  // d/d h (h_k = h s(k))
+        -both(abar), 0.f, both(cbar),
+        wEn * fmaf(0.5f, both(sw2), fmaf(-Jx, both(sbx), fmaf(-Jy, both(sby), hF * both(scp)))),  // w_E E / N
+        both(pm),                                                                      // sum of sigma sin(q theta_k)
     };
 #pragma unroll
     for (int k = 0; k < kGacc + 1; ++k) {
@@ -401,12 +371,12 @@ __global__ void __launch_bounds__(512, 1) adjoint_back_kernel(const DevCfg* cfgs
 }
 
 cudaError_t launch_adjoint_back(const DevCfg* d_cfg, const BandTask* tasks, int n_tasks, int Lx, int H, uint64_t seed,
-                                bool back, BackArgs R, cudaStream_t st)
+                                bool back, BackArgs R, bool after, cudaStream_t st)
 {
     if (n_tasks == 0) return cudaSuccess;
     const bool wide = Lx > 128;
     const int threads = wide ? (Lx / 128) * 32 : 256;
-    const int smem = (threads / 32) * 2 * 4 * 32 * (int)sizeof(float4);
+    const int smem = (threads / 32) * (int)sizeof(BackWarp);
     const bool obs = R.k > R.k0;
     using Kern = void (*)(const DevCfg*, const BandTask*, int, BackArgs, PhiloxKeys);
     static const Kern table[2][2][2][2] = {
@@ -420,12 +390,21 @@ cudaError_t launch_adjoint_back(const DevCfg* d_cfg, const BandTask* tasks, int 
           {adjoint_back_kernel<true, true, false, true>, adjoint_back_kernel<true, true, true, true>}}},
     };
     const Kern kern = table[R.sched != 0][wide][obs][back];
-    if (smem > 48 * 1024) {
-        const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (smem > 46 * 1024) {  // (the limit belongs to the kernel, which other shapes share: always the largest)
+        const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                   kMaxBackWarps * (int)sizeof(BackWarp));
         if (e != cudaSuccess) return e;
     }
-    kern<<<(unsigned)n_tasks, threads, smem, st>>>(d_cfg, tasks, H, R, philox_round_keys(seed));
-    return cudaGetLastError();
+    auto dist = [&](const float* q) { return q ? (int64_t)((const char*)q - (const char*)R.th_in) : 0; };
+    R.d_v_in = dist(R.v_in);
+    R.d_tb_in = dist(R.tb_in);
+    R.d_vb_in = dist(R.vb_in);
+    R.d_th_out = dist(R.th_out);
+    R.d_v_out = dist(R.v_out);
+    R.d_tb_out = dist(R.tb_out);
+    R.d_vb_out = dist(R.vb_out);
+    return launch_dependent(kern, (unsigned)n_tasks, (unsigned)threads, (size_t)smem, st, after, d_cfg, tasks, H, R,
+                            philox_round_keys(seed));
 }
 
 }  // namespace xy

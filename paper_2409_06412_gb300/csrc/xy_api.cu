@@ -178,15 +178,19 @@ int even_band(int Ly, int h)
     return (Ly + nb - 1) / nb;
 }
 
-// Default band height: the tallest that still gives `min_warps` warps over the
-// lattices of the shape (a warp walks its rows one after the other; taller bands
-// recompute fewer halo rows).
-int default_band_H(int Lx, int Ly, int64_t n_lat, int64_t min_warps)
+// Default band height, for batches too small for the tuner: the lowest whose
+// warps the chip still holds at once (max_warps).  A launch of such a batch takes
+// as long as one warp needs for its H + 4 rows, so low bands are faster although
+// they recompute more halo rows, until they no longer run together (us per step at
+// H = 1, 2, 4, 8, and the warps of the best: 512^2 2.93 2.76 3.24 4.73, 1024;
+// 256^2 2.02 2.38 3.08 4.47, 512; 16 x 256^2 6.9 4.6 4.2 5.2, 2048; 1024^2 8.6 6.5
+// 5.0 5.7, 2048; 8 x 200^2 3.2 2.9 3.4 4.5, 1600).
+int default_band_H(int Lx, int Ly, int64_t n_lat, int64_t max_warps)
 {
     const int warps = Lx > 128 ? (Lx + 127) / 128 : kNarrowBandWarps;
-    for (int h : {64, 32, 16, 8})
-        if (n_lat * band_blocks(Lx, Ly, h) * warps >= min_warps) return even_band(Ly, h);
-    return even_band(Ly, 4);
+    for (int h : {1, 2, 4, 8, 16, 32})
+        if (n_lat * band_blocks(Lx, Ly, even_band(Ly, h)) * warps <= max_warps) return even_band(Ly, h);
+    return even_band(Ly, 64);
 }
 
 bool is_device_ptr(const void* p)
@@ -273,6 +277,7 @@ struct xy_lattice {
     int cur_re = 0;             // its record_every
     uint64_t cur_mask = 0;      // local steps of a chunk at which some strip-stepped lattice records
     std::vector<uint8_t> in_b;  // per configuration: its state ended the call in buffers B
+    int sms = 152;              // SMs of the device
     int kt_mode = 0;            // xy_set_temporal_blocking: 0 tuner, 1 one step, 2 two steps per launch
     // kernel timing (direct launches bracketed by events)
     bool timing = false;
@@ -333,6 +338,8 @@ int upload_call(xy_lattice* L, const CallArgs& ca)
     // a slot is reused only after the copy that read it has executed
     const int slot = L->call_next;
     L->call_next = (L->call_next + 1) % xy_lattice::kRing;
+    if (!L->call_ev[slot])  // created on first use: all of them took 30 us of an object's creation
+        CK(cudaEventCreateWithFlags(&L->call_ev[slot], cudaEventDisableTiming));
     CK(cudaEventSynchronize(L->call_ev[slot]));
     L->h_call[slot] = ca;
     L->h_call[slot].err = L->d_err;
@@ -562,9 +569,19 @@ std::vector<StepRun> step_plan(const xy_lattice* L, const StripGroup& g, int cnt
     return out;
 }
 
-// One launch of a strip group: lattices [lat0, lat0 + n_lat) of it.
+// Whether a launch over the whole group has fewer warps than the chip holds of the
+// band kernel (16 per SM).
+bool under_one_wave(const xy_lattice* L, const StripGroup& g)
+{
+    const int64_t warps = g.Lx > 128 ? (g.Lx + 127) / 128 : kNarrowBandWarps;
+    return g.band_H > 0 && (int64_t)g.band_tasks.size() * warps < (int64_t)L->sms * 16;
+}
+
+// One launch of a strip group: lattices [lat0, lat0 + n_lat) of it.  after: the
+// launch before it on the stream is of the same chunk, and this one may start while
+// that one drains.
 cudaError_t launch_group(xy_lattice* L, cudaStream_t st, StripGroup& g, int64_t lat0, int64_t n_lat, const StepRun& r,
-                         int64_t jl0, int rd_b, Buffers buf)
+                         int64_t jl0, int rd_b, Buffers buf, bool after)
 {
     ++L->launches;
     // (when every step records nothing pairs: the strip kernel has no halo rows)
@@ -572,7 +589,7 @@ cudaError_t launch_group(xy_lattice* L, cudaStream_t st, StripGroup& g, int64_t 
     if (g.band_H > 0 && (r.n == 2 || !strip)) {
         const int64_t per = (int64_t)g.band_tasks.size() / g.n_lat;
         return launch_band_step(L->d_cfg, g.d_band_tasks + lat0 * per, (int)(n_lat * per), g.Lx, g.band_H, r.rec,
-                                group_sched(L, g), r.n, rd_b != 0, g.seed, jl0 + r.off, buf, L->d_call, L->pa, st);
+                                group_sched(L, g), r.n, rd_b != 0, g.seed, jl0 + r.off, buf, L->d_call, L->pa, after, st);
     }
     const int64_t per = (int64_t)g.tasks.size() / g.n_lat;
     return launch_strip_step(L->d_cfg, g.d_tasks + lat0 * per, (int)(n_lat * per), g.H, g.variant, r.rec,
@@ -596,7 +613,7 @@ int launch_batched_steps(xy_lattice* L, cudaStream_t st, int64_t jl0, int cnt, b
         int rd = g.buf;
         for (const StepRun& r : step_plan(L, g, cnt)) {
             if ((rc = timed_begin(L, st, r.n == 2 ? XY_KCLASS_STRIP2 : XY_KCLASS_STRIP, &end))) return rc;
-            CK(launch_group(L, st, g, 0, g.n_lat, r, jl0, rd, buf));
+            CK(launch_group(L, st, g, 0, g.n_lat, r, jl0, rd, buf, false));
             if ((rc = timed_end(end, st))) return rc;
             rd ^= 1;
         }
@@ -798,7 +815,11 @@ cudaError_t launch_branch(xy_lattice* L, cudaStream_t st, const Branch& br, int6
         int rd = g.buf;
         for (const StepRun& r : step_plan(L, g, cnt)) {
             if (e != cudaSuccess) break;
-            e = launch_group(L, st, g, br.lat0, br.n_lat, r, jl0, rd, buf);
+            // the first launch follows the chunk counter's update; later ones start
+            // early where a launch leaves SMs idle (16 x 256^2: 4.6 -> 4.3 us per step).
+            // In larger batches the waiting blocks would hold the slots that other
+            // slices' blocks fill (32 x 1024^2: 3 % slower).
+            e = launch_group(L, st, g, br.lat0, br.n_lat, r, jl0, rd, buf, r.off > 0 && under_one_wave(L, g));
             rd ^= 1;
         }
         return e;
@@ -1032,7 +1053,7 @@ int autotune_lattice(xy_lattice* L)
                 float t2 = 1e30f;
                 rc = time_it(cut_tasks(g.band_tasks, n_parts), [&](cudaStream_t st, int t0, int cnt) {
                     return launch_band_step(L->d_cfg, g.d_band_tasks + t0, cnt, g.Lx, H, 0, group_sched(L, g), 2, false,
-                                            g.seed, 0, buf, L->d_call, L->pa, st);
+                                            g.seed, 0, buf, L->d_call, L->pa, false, st);
                 }, t2);
                 if (rc) break;
                 if (t2 < best2) {
@@ -1323,6 +1344,7 @@ int classify(xy_lattice* L)
     int dev = 0, sms = 148;
     if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     cudaGetLastError();
+    L->sms = sms;
     for (int c = 0; c < L->n_cfg; ++c) {
         CfgHost& h = L->cfg[c];
         const int Lx = h.desc.Lx, Ly = h.desc.Ly;
@@ -1340,7 +1362,7 @@ int classify(xy_lattice* L)
             h.H = H;
             if (H > 0)
                 max_units = std::max(max_units, strip_units_per_lattice(Lx, Ly, std::min(H, min_strip_H(Lx, Ly))));
-            if (band_shape(Lx, Ly)) max_units = std::max(max_units, band_blocks(Lx, Ly, even_band(Ly, 4)));
+            if (band_shape(Lx, Ly)) max_units = std::max(max_units, band_blocks(Lx, Ly, 1));
         } else {
             h.kind = 2;
         }
@@ -1383,7 +1405,7 @@ int classify(xy_lattice* L)
     for (auto& g : L->strip_groups) {
         int rc = g.strip_ok ? build_strip_tasks(L, g) : XY_OK;
         if (rc == XY_OK && band_shape(g.Lx, g.Ly))
-            rc = build_band_tasks(L, g, default_band_H(g.Lx, g.Ly, g.n_lat, (int64_t)sms * 16));
+            rc = build_band_tasks(L, g, default_band_H(g.Lx, g.Ly, g.n_lat, (int64_t)sms * 14 / (int64_t)L->strip_groups.size()));
         if (rc) return rc;
     }
     apply_kt_mode(L);
@@ -1506,9 +1528,6 @@ int xy_lattice_create(const xy_config_desc* cfg, int n_cfg, float* theta, float*
         cudaGetLastError();
         return bail(fail(XY_ENOMEM, "allocation failed: %s", cudaGetErrorString(e)));
     }
-    for (int i = 0; i < xy_lattice::kRing; ++i)
-        if ((e = cudaEventCreateWithFlags(&L->call_ev[i], cudaEventDisableTiming)) != cudaSuccess)
-            return bail(fail(XY_ECUDA, "event: %s", cudaGetErrorString(e)));
     int rc = classify(L);
     if (rc) return bail(rc);
     if ((e = cudaMalloc(&L->pa.part, sizeof(double2) * B * L->pa.max_units)) != cudaSuccess ||
@@ -2128,7 +2147,7 @@ int xy_adjoint_step_n(xy_lattice* L, int64_t n, int K, double wE, double wM, dou
                         A.gacc = g_tmp;
                         return launch_sliced(L, cuts, reps, [&](cudaStream_t st, int t0, int cnt) {
                             A.block_base = t0;
-                            return launch_adjoint_back(L->d_cfg, d_tk + t0, cnt, g.Lx, h, g.seed, true, A, st);
+                            return launch_adjoint_back(L->d_cfg, d_tk + t0, cnt, g.Lx, h, g.seed, true, A, false, st);
                         });
                     }
                     BandArgs R{};
@@ -2316,7 +2335,7 @@ int xy_adjoint_step_n(xy_lattice* L, int64_t n, int K, double wE, double wM, dou
                 for (size_t p = 0; p + 1 < c.size(); ++p, ++q) {
                     A.block_base = g.block_base + c[p];
                     CKA(launch_adjoint_back(L->d_cfg, g.d_tasks + c[p], c[p + 1] - c[p], g.Lx, g.H, g.seed, bk, A,
-                                            q == 0 ? L->stream : L->aux[(q - 1) % n_aux]));
+                                            bk && n_slices <= n_aux + 1, q == 0 ? L->stream : L->aux[(q - 1) % n_aux]));
                     ++L->launches;
                 }
             }
@@ -2419,7 +2438,7 @@ int xy_adjoint_step_n(xy_lattice* L, int64_t n, int K, double wE, double wM, dou
                     ++L->launches;
                 }
                 for (auto& g : L->strip_groups)
-                    CKA(launch_group(L, L->stream, g, 0, g.n_lat, StepRun{0, 1, 0}, i, 0, buf));
+                    CKA(launch_group(L, L->stream, g, 0, g.n_lat, StepRun{0, 1, 0}, i, 0, buf, false));
                 for (int c : L->plain_cfgs) {
                     CKA(launch_plain_step(L->d_cfg, L->h_dev[c], i, buf, L->d_call, L->pa, 1, L->stream));
                     ++L->launches;

@@ -128,6 +128,25 @@ struct Partials {
     int32_t max_units;
 };
 
+// Launch of a kernel that calls dependency_wait(): after = true lets it start while
+// the launch before it on the stream drains (programmatic dependent launch).
+template <class... P, class... A>
+cudaError_t launch_dependent(void (*kern)(P...), unsigned blocks, unsigned threads, size_t smem, cudaStream_t st, bool after,
+                             A... args)
+{
+    cudaLaunchConfig_t lc = {};
+    lc.gridDim = dim3(blocks);
+    lc.blockDim = dim3(threads);
+    lc.dynamicSmemBytes = smem;
+    lc.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    lc.attrs = at;
+    lc.numAttrs = after ? 1 : 0;
+    return cudaLaunchKernelEx(&lc, kern, P(args)...);
+}
+
 // ---- launchers (xy_step.cu)
 cudaError_t launch_init(const DevCfg* d_cfg, const DevCfg& h_cfg, int init_mode, float* theta, float* omega,
                         cudaStream_t st);
@@ -153,7 +172,7 @@ bool band_shape(int Lx, int Ly);
 int bands_per_block(int Lx);
 cudaError_t launch_band_step(const DevCfg* d_cfg, const BandTask* tasks, int n_tasks, int Lx, int H, int rec, bool sched,
                              int n_steps, bool rd_b, uint64_t seed, int64_t j_local, Buffers buf, const CallArgs* ca,
-                             Partials pa, cudaStream_t st);
+                             Partials pa, bool after, cudaStream_t st);
 // every task of one launch uses the noise key `seed`
 cudaError_t launch_resident_step(const DevCfg* d_cfg, const ResidentTask* tasks, int n_tasks, int Lx, int Ly,
                                  int threads, int csize, uint64_t seed, int64_t j_local, int n_steps, Buffers buf,
@@ -273,9 +292,11 @@ struct BackArgs {
     double* gacc;        // [blocks][kGacc]
     int block_base;
     int sched;           // some configuration of the tasks has a field or coupling schedule
+    // distances in bytes of the other arrays from th_in (set by launch_adjoint_back)
+    int64_t d_v_in, d_tb_in, d_vb_in, d_th_out, d_v_out, d_tb_out, d_vb_out;
 };
 cudaError_t launch_adjoint_back(const DevCfg* d_cfg, const BandTask* tasks, int n_tasks, int Lx, int H, uint64_t seed,
-                                bool back, BackArgs R, cudaStream_t st);
+                                bool back, BackArgs R, bool after, cudaStream_t st);
 // M_k of slots [0, n_states) of a segment (slot stride 2 T floats) into
 // rec[b * rec_stride + r0 + slot].x
 cudaError_t launch_segment_m(const DevCfg* d_cfg, int n_cfg, int64_t B, const float* seg, int64_t T, int n_states,

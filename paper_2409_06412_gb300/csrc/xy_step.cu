@@ -788,6 +788,13 @@ __global__ void __launch_bounds__(512, 1) band_step_kernel(const DevCfg* cfgs, c
         }
         cp_async_commit();
     };
+    // noise of the quad of a row at offset o
+    auto noise = [&](int o, int64_t kk, float c) {
+        return p4(gauss4_scaled(philox4x32_10_rk(noise_counter((uint32_t)(o + x) >> 2, cfgrep, kk, 0u), keys), c));
+    };
+    o_a = (y0 + Ly - 1) % Ly * Lx;
+    P4 cn1 = noise(o_a, k, c1), cn2;
+    dependency_wait();  // the state of the launch before
     issue(0, 0);
     issue(1, 1);
     // The ends of the quads beside come from shared memory, inside the warp as
@@ -836,12 +843,6 @@ __global__ void __launch_bounds__(512, 1) band_step_kernel(const DevCfg* cfgs, c
     const bool stag = cf.stag != 0;
     R0 r0[3];
     R1 r1[3];
-    // noise of the quad of a row at offset o
-    auto noise = [&](int o, int64_t kk, float c) {
-        return p4(gauss4_scaled(philox4x32_10_rk(noise_counter((uint32_t)(o + x) >> 2, cfgrep, kk, 0u), keys), c));
-    };
-    o_a = (y0 + Ly - 1) % Ly * Lx;
-    P4 cn1 = noise(o_a, k, c1), cn2;
     // iteration i: P0, C0, N0 = level-0 rows y - 2, y - 1, y; P1, C1, N1 =
     // level-1 rows b - 1, b, a (N1 computed here); levels: how many there are yet.
     // The wait and the two wrap tests cut the iteration into blocks of straight
@@ -916,6 +917,7 @@ __global__ void __launch_bounds__(512, 1) band_step_kernel(const DevCfg* cfgs, c
         if (i + 2 < n_it) body(L2{}, i + 2, 0, r0[1], r0[2], r0[0], r1[1], r1[2], r1[0]);
     }
     cp_async_wait<0>();
+    launch_next();
     if (REC > 0) {
         // one partial per block: warp sums, then the block's warps in order
         __shared__ double2 s_part[kBandWarps];
@@ -949,7 +951,7 @@ int bands_per_block(int Lx) { return Lx > 128 ? 1 : kNarrowBandWarps * (32 / (Lx
 // j_local takes step j (and j + 1) of the call.
 cudaError_t launch_band_step(const DevCfg* d_cfg, const BandTask* tasks, int n_tasks, int Lx, int H, int rec, bool sched,
                              int n_steps, bool rd_b, uint64_t seed, int64_t j_local, Buffers buf, const CallArgs* ca,
-                             Partials pa, cudaStream_t st)
+                             Partials pa, bool after, cudaStream_t st)
 {
     if (n_tasks == 0) return cudaSuccess;
     if (!band_shape(Lx, 1) || H < 1) return cudaErrorInvalidValue;
@@ -971,10 +973,8 @@ cudaError_t launch_band_step(const DevCfg* d_cfg, const BandTask* tasks, int n_t
                                                    (int)sizeof(BStage) * kBandWarps);
         if (e != cudaSuccess) return e;
     }
-    kern<<<(unsigned)n_tasks, 32 * warps, smem, st>>>(d_cfg, tasks, H, n_steps, rd_b ? 1 : 0,
-                                                                               j_local, buf, ca, pa,
-                                                                               philox_round_keys(seed));
-    return cudaGetLastError();
+    return launch_dependent(kern, (unsigned)n_tasks, 32 * warps, smem, st, after, d_cfg, tasks, H, n_steps, rd_b ? 1 : 0,
+                            j_local, buf, ca, pa, philox_round_keys(seed));
 }
 
 namespace {
