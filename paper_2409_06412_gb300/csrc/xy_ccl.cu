@@ -10,8 +10,9 @@
 // Passes (unions always link the larger root under the smaller, so every
 // root is its component's minimum):
 //   tile    one warp per 32 x 32 tile: the rows' spins as 32-bit masks, runs
-//           of equal spin, union-find over the runs in shared memory; every
-//           site gets its tile root, and each piece its tile-local size.
+//           of equal spin, each linked to one run of the row above, pointer
+//           jumping, and unions in shared memory for the remaining contacts;
+//           every site gets its tile root, and each piece its tile-local size.
 //           A piece that does not reach the tile's edge is a whole domain and
 //           goes into the size histogram at once; one that does goes on a
 //           short list (batch index, local size) for the merge.
@@ -142,19 +143,6 @@ __device__ __forceinline__ int find_root_tile(int* L, int x)
     return x;
 }
 
-// The same search without writes: while lanes point their own run starts at
-// their roots, a halving step elsewhere could replace such a pointer with an
-// older ancestor.
-__device__ __forceinline__ int find_root_tile_ro(const int* L, int x)
-{
-    int p = L[ph(x)];
-    while (p != x) {
-        x = p;
-        p = L[ph(x)];
-    }
-    return x;
-}
-
 // Link in a tile's forest (padded layout), with a bound on the retries:
 // every failed atomicMin means another lane lowered the same entry, so the
 // loop ends long before the bound in practice; reaching it sets XY_ETIMEOUT
@@ -231,94 +219,119 @@ __global__ void __launch_bounds__(32 * kTileWarps, 12) ccl_tile_kernel(const flo
 
     // the rows' spins as masks (lane y keeps row y); 16 loads in flight per lane
     unsigned row = 0;
+    if (tw == 32 && thh == 32) {
 #pragma unroll
-    for (int h = 0; h < 32; h += 16) {
-        float v[16];
+        for (int h = 0; h < 32; h += 16) {
+            float v[16];
 #pragma unroll
-        for (int y = 0; y < 16; ++y) v[y] = (h + y < thh && lane < tw) ? th[(h + y) * Lx + lane] : 0.0f;
+            for (int y = 0; y < 16; ++y) v[y] = th[(h + y) * Lx + lane];
 #pragma unroll
-        for (int y = 0; y < 16; ++y) {
-            const unsigned m = __ballot_sync(kAll, spin_of(v[y])) & vm;
-            if (lane == h + y) row = m;
+            for (int y = 0; y < 16; ++y) {
+                const unsigned m = __ballot_sync(kAll, spin_of(v[y]));
+                row = lane == h + y ? m : row;
+            }
+        }
+    } else {
+        for (int y = 0; y < thh; ++y) {
+            const unsigned m = __ballot_sync(kAll, spin_of(lane < tw ? th[y * Lx + lane] : 0.0f)) & vm;
+            row = lane == y ? m : row;
         }
     }
-    const unsigned st = run_starts(row, vm);  // lane y: the run starts of row y
+    const unsigned st = lane < thh ? run_starts(row, vm) : 0u;  // lane y: the run starts of row y
 
-    // every run start is a root
-    for (unsigned b = st; b; b &= b - 1) {
-        const int i = lane * 32 + __ffs(b) - 1;
-        P[ph(i)] = i;
+    // Every run is linked to the first run it touches in the row above (a smaller
+    // index), or is a root: each lane writes only its own run starts, so the tree
+    // needs no search and no atomic.  Its other contacts with the row above (at the
+    // first column where a pair of runs touches) are left in `more`: they join two
+    // pieces, or close a loop.
+    unsigned more = 0, sa;
+    {
+        const unsigned above = __shfl_up_sync(kAll, row, 1);
+        sa = __shfl_up_sync(kAll, st, 1);
+        const unsigned c = lane > 0 && lane < thh ? ~(row ^ above) & vm : 0u;
+        const unsigned u = c & ~((c << 1) & c & ~st & ~sa);
+        for (unsigned b = st; b; b &= b - 1) {
+            const unsigned later = b & (b - 1);
+            const int x = __ffs(b) - 1;
+            // contacts of this run: from its start up to the next one
+            const unsigned uu = u & (later ? (later & (0u - later)) - 1u : kAll) & (kAll << x);
+            P[lane * 33 + x] = uu ? lane * 32 - 32 + run_of(sa, __ffs(uu) - 1) : lane * 32 + x;
+            more |= uu & (uu - 1);
+        }
     }
     H[lane] = 0;
     H[lane + 32] = 0;
     __syncwarp();
-
-    // vertical contacts between rows y and y + 1 (lane y): one union per pair
-    // of runs, at the first column where they touch
-    {
-        const unsigned below = __shfl_down_sync(kAll, row, 1);
-        const unsigned sb = __shfl_down_sync(kAll, st, 1);
-        if (lane + 1 < thh) {
-            const unsigned c = ~(row ^ below) & vm;
-            unsigned u = c & ~((c << 1) & c & ~st & ~sb);
-            while (u) {
-                const int x = __ffs(u) - 1;
-                u &= u - 1;
-                union_tile(P, lane * 32 + run_of(st, x), (lane + 1) * 32 + run_of(sb, x), err);
+    // Pointer jumping: every run start points at its grandparent until all point
+    // at roots, log2 of the longest chain passes (a lane writes only its own
+    // entries, and only ancestors, so the passes need no order among the lanes).
+    // A search from each run start walked chains of up to 32 rows instead.
+    volatile int* vP = P;
+    auto jump = [&]() {
+        for (int pass = 0; pass < 33; ++pass) {
+            bool moved = false;
+            for (unsigned b = st; b; b &= b - 1) {
+                const int i = lane * 33 + __ffs(b) - 1;
+                const int p = vP[i];
+                const int g = vP[ph(p)];
+                if (g != p) {
+                    vP[i] = g;
+                    moved = true;
+                }
             }
+            __syncwarp();
+            if (!__any_sync(kAll, moved)) break;
         }
+    };
+    jump();
+    if (__any_sync(kAll, more != 0u)) {
+        for (unsigned b = more; b; b &= b - 1) {
+            const int x = __ffs(b) - 1;
+            union_tile(P, lane * 32 + run_of(st, x), lane * 32 - 32 + run_of(sa, x), err);
+        }
+        __syncwarp();
+        jump();
     }
-    __syncwarp();
 
-    // every run start points straight at its root: each lane writes only its
-    // own run starts, and only roots; the searches write nothing
     unsigned roots = 0;  // lane y: the tile roots of row y
-    if (lane < thh) {
-        for (unsigned b = st; b; b &= b - 1) {
-            const int i = lane * 32 + __ffs(b) - 1;
-            const int r = find_root_tile_ro(P, i);
-            if (r != i)
-                P[ph(i)] = r;
-            else
-                roots |= 1u << (i & 31);
-        }
+    for (unsigned b = st; b; b &= b - 1) {
+        const int x = __ffs(b) - 1;
+        if (P[lane * 33 + x] == lane * 32 + x) roots |= b & (0u - b);
     }
+    // (a tile whose unions ran out of retries still has every root in `roots`)
     __syncwarp();
     // a root's entry becomes its piece's count: -1 - (size + kEdgeFlag * edge runs)
-    for (unsigned b = roots; b; b &= b - 1) P[ph(lane * 32 + __ffs(b) - 1)] = -1;
+    for (unsigned b = roots; b; b &= b - 1) P[lane * 33 + __ffs(b) - 1] = -1;
     __syncwarp();
-    if (lane < thh) {
-        for (unsigned b = st; b; b &= b - 1) {
-            const int x = __ffs(b) - 1;
-            const int i = lane * 32 + x;
-            const int q = P[ph(i)];
-            const int r = q < 0 ? i : q;
-            const unsigned later = b & (b - 1);
-            const int end = later ? __ffs(later) - 1 : tw;
-            const bool edge = lane == 0 || lane == thh - 1 || x == 0 || end == tw;
-            atomicSub(&P[ph(r)], (end - x) + (edge ? kEdgeFlag : 0));
-        }
+    for (unsigned b = st; b; b &= b - 1) {
+        const int x = __ffs(b) - 1;
+        const int i = lane * 32 + x;
+        const int q = P[lane * 33 + x];
+        const int r = q < 0 ? i : q;
+        const unsigned later = b & (b - 1);
+        const int end = later ? __ffs(later) - 1 : tw;
+        const bool edge = lane == 0 || lane == thh - 1 || x == 0 || end == tw;
+        atomicSub(&P[ph(r)], (end - x) + (edge ? kEdgeFlag : 0));
     }
     __syncwarp();
 
-    // labels, a row at a time (coalesced): each site's root through its run
-    // start; the tile roots and spins of the edge sites go to the border pass
-    uint16_t* er = s.edge_root + (int64_t)t * 128;  // top row, bottom row, left column, right column
-#pragma unroll 4
-    for (int y = 0; y < thh; ++y) {
-        const unsigned sy = __shfl_sync(kAll, st, y);
-        if (lane < tw) {
-            const int i = y * 32 + run_of(sy, lane);
-            const int q = P[y * 33 + (i & 31)];
-            const int r = q < 0 ? i : q;
-            lab[y * Lx + lane] = (gy0 + (r >> 5)) * Lx + gx0 + (r & 31);
-            if (y == 0) er[lane] = (uint16_t)r;
-            if (y == thh - 1) er[32 + lane] = (uint16_t)r;
-            if (lane == 0) er[64 + y] = (uint16_t)r;
-            if (lane == tw - 1) er[96 + y] = (uint16_t)r;
-        }
-    }
+    // the tile roots and spins of the edge sites go to the border pass: top row,
+    // bottom row (lane = column), left column, right column (lane = row)
     {
+        uint16_t* er = s.edge_root + (int64_t)t * 128;
+        auto root_at = [&](int y, int x) {  // of the run that starts at (x, y)
+            const int q = P[y * 33 + x];
+            return (uint16_t)(q < 0 ? y * 32 + x : q);
+        };
+        const unsigned st_top = __shfl_sync(kAll, st, 0), st_bottom = __shfl_sync(kAll, st, thh - 1);
+        if (lane < tw) {
+            er[lane] = root_at(0, run_of(st_top, lane));
+            er[32 + lane] = root_at(thh - 1, run_of(st_bottom, lane));
+        }
+        if (lane < thh) {
+            er[64 + lane] = root_at(lane, 0);
+            er[96 + lane] = root_at(lane, run_of(st, tw - 1));
+        }
         const unsigned left = __ballot_sync(kAll, lane < thh && (row & 1u));
         const unsigned right = __ballot_sync(kAll, lane < thh && ((row >> (tw - 1)) & 1u));
         const unsigned top = __shfl_sync(kAll, row, 0), bottom = __shfl_sync(kAll, row, thh - 1);
@@ -359,6 +372,26 @@ __global__ void __launch_bounds__(32 * kTileWarps, 12) ccl_tile_kernel(const flo
         }
     }
     __syncwarp();
+    // labels: every run start's entry becomes its root's site in the lattice (each
+    // lane its own entries), then a row at a time (coalesced), each site through
+    // its run start
+    for (unsigned b = st; b; b &= b - 1) {
+        const int x = __ffs(b) - 1;
+        const int q = P[lane * 33 + x];
+        const int r = q < 0 ? lane * 32 + x : q;
+        P[lane * 33 + x] = (gy0 + (r >> 5)) * Lx + gx0 + (r & 31);
+    }
+    P[lane * 33 + 32] = (int)st;  // (the padding word of each row)
+    __syncwarp();
+    if (lane < tw) {
+        const unsigned upto = (2u << lane) - 1u;
+        int32_t* o = lab + lane;
+#pragma unroll 8
+        for (int y = 0; y < thh; ++y) {
+            *o = P[y * 33 + 31 - __clz((unsigned)P[y * 33 + 32] & upto)];
+            o += Lx;
+        }
+    }
 #pragma unroll
     for (int k = 0; k < 2; ++k) {
         const int sz = lane + 32 * k;
@@ -376,9 +409,14 @@ __global__ void __launch_bounds__(32 * kTileWarps, 12) ccl_tile_kernel(const flo
 // pieces is already linked: one union per pair of touching runs.  The roots'
 // entries are read at once for both edges; two roots are then linked
 // straight away, anything else goes through the general union.
+// Its threads also clear the histogram's pairs (hist, n_hist words; the compaction
+// fills the leading ones): one block per lattice spent longer on that than on the
+// pairs.
 __global__ void __launch_bounds__(256) ccl_border_kernel(int Lx, int Ly, int n_lat, int32_t* labels, CclScratch s,
-                                                         int* err)
+                                                         int64_t* hist, int64_t n_hist, int* err)
 {
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n_hist; i += (int64_t)gridDim.x * blockDim.x)
+        hist[i] = 0;
     const int lane = threadIdx.x & 31;
     const int tiles_x = (Lx + 31) >> 5, tiles_y = (Ly + 31) >> 5;
     const int tiles = tiles_x * tiles_y;
@@ -580,22 +618,23 @@ __global__ void __launch_bounds__(256, 4) ccl_flatten_kernel(int Lx, int Ly, int
 }
 
 // Pass 5: ordered compaction of the nonzero counts into (size, count) pairs,
-// one block per lattice, ascending size; the rest of the lattice's hist_cap
-// pairs is zeroed.  Sizes 1..63 are summed over their copies; larger ones
-// are found through the bitmap, one bit per size, a word per thread per
-// round in order: each round's set bits are placed by one block-wide prefix,
-// and each thread writes its word's pairs and clears what it read.
+// one block per lattice, ascending size (the rest of the lattice's hist_cap
+// pairs is zero already).  Sizes 1..63 are summed over their copies; larger ones
+// are found through the bitmap, one bit per size: a warp takes 1024 consecutive
+// words, all 32 loads of a lane in flight, the warps' bits are summed in one
+// block-wide prefix, and each warp then places its own without further barriers
+// (a round of 1024 words at a time took four barriers per round).
 __global__ void __launch_bounds__(1024) ccl_compact_kernel(int64_t N, CclScratch s, int64_t* hist, int64_t hist_cap,
                                                            int64_t* n_sizes, int* err)
 {
     __shared__ int s_warp[32];
     __shared__ int s_small[kSmallSizes];
-    __shared__ int64_t s_pos;
     const int lat = blockIdx.x;
     int32_t* cnt = s.counts + (int64_t)lat * (N + 1);
     uint32_t* bw = s.bits + (int64_t)lat * s.words;
     int64_t* out = hist ? hist + (int64_t)lat * hist_cap * 2 : nullptr;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const unsigned below = (1u << lane) - 1u;
     const int n_small = (int)(N < kSmallSizes - 1 ? N : kSmallSizes - 1);  // sizes 1..n_small
     if (threadIdx.x < kSmallSizes) s_small[threadIdx.x] = 0;
     __syncthreads();
@@ -618,75 +657,71 @@ __global__ void __launch_bounds__(1024) ccl_compact_kernel(int64_t N, CclScratch
         if (v) atomicAdd(&s_small[z], v);
     }
     __syncthreads();
-    if (threadIdx.x == 0) {
-        int64_t at = 0;
-        for (int z = 1; z < kSmallSizes; ++z)
-            if (s_small[z] != 0) {
-                if (out && at < hist_cap) {
-                    out[2 * at] = z;
-                    out[2 * at + 1] = s_small[z];
-                }
-                ++at;
-            }
-        s_pos = at;
+    int64_t pos = 0;  // pairs placed so far (the same in every thread)
+#pragma unroll
+    for (int k = 0; k < kSmallSizes / 32; ++k) {
+        const int z = lane + 32 * k;
+        const unsigned m = __ballot_sync(kAll, s_small[z] != 0);
+        const int64_t at = pos + __popc(m & below);
+        if (warp == 0 && s_small[z] != 0 && out && at < hist_cap) {
+            out[2 * at] = z;
+            out[2 * at + 1] = s_small[z];
+        }
+        pos += __popc(m);
     }
-    __syncthreads();
-    // words holding sizes >= 64: round k of a chunk gives thread j the word
-    // k * blockDim + j, so the order within a round is the order of the
-    // threads; all 32 rounds' words are read at once
+    // words holding sizes >= 64
     const int64_t w0 = kSmallSizes / 32;
-    const int nt = blockDim.x;
-    for (int64_t wc = w0; wc < s.words; wc += 32 * (int64_t)nt) {
+    for (int64_t wc = w0; wc < s.words; wc += 32 * 1024) {
+        const int64_t wbase = wc + warp * 1024 + lane;
         uint32_t wd[32];
+        int c = 0;
 #pragma unroll
         for (int k = 0; k < 32; ++k) {
-            const int64_t w = wc + (int64_t)k * nt + threadIdx.x;
+            const int64_t w = wbase + 32 * k;
             wd[k] = w < s.words ? bw[w] : 0u;
         }
-#pragma unroll 1
+#pragma unroll
+        for (int k = 0; k < 32; ++k) c += __popc(wd[k]);
+#pragma unroll
+        for (int d = 16; d > 0; d >>= 1) c += __shfl_xor_sync(kAll, c, d);
+        __syncthreads();  // the last chunk's s_warp has been read
+        if (lane == 0) s_warp[warp] = c;
+        __syncthreads();
+        int64_t at = pos;
+        for (int w = 0; w < 32; ++w) {
+            at += w < warp ? s_warp[w] : 0;
+            pos += s_warp[w];
+        }
+        if (c == 0) continue;  // the whole warp; the barriers above are met by all
+#pragma unroll
         for (int k = 0; k < 32; ++k) {
             const uint32_t word = wd[k];
-            if (!__syncthreads_or(word != 0u)) continue;  // uniform
-            const int c = __popc(word);
-            int before = c;  // inclusive prefix over the warp
+            if (!__any_sync(kAll, word != 0u)) continue;
+            const int n = __popc(word);
+            int upto = n;  // inclusive prefix over the warp
 #pragma unroll
             for (int d = 1; d < 32; d <<= 1) {
-                const int o = __shfl_up_sync(kAll, before, d);
-                if (lane >= d) before += o;
+                const int o = __shfl_up_sync(kAll, upto, d);
+                if (lane >= d) upto += o;
             }
-            if (lane == 31) s_warp[warp] = before;
-            __syncthreads();
-            int64_t at = s_pos + before - c;
-            int round = 0;
-            for (int w = 0; w < (nt >> 5); ++w) {
-                if (w < warp) at += s_warp[w];
-                round += s_warp[w];
-            }
-            const int64_t w = wc + (int64_t)k * nt + threadIdx.x;
+            int64_t a = at + upto - n;
+            const int64_t w = wbase + 32 * k;
             for (uint32_t b = word; b; b &= b - 1) {
                 const int64_t z = (w << 5) + __ffs(b) - 1;
-                if (out && at < hist_cap) {
-                    out[2 * at] = z;
-                    out[2 * at + 1] = cnt[z];
+                if (out && a < hist_cap) {
+                    out[2 * a] = z;
+                    out[2 * a + 1] = cnt[z];
                 }
                 cnt[z] = 0;
-                ++at;
+                ++a;
             }
             if (word) bw[w] = 0;
-            __syncthreads();  // every thread has read s_pos and s_warp
-            if (threadIdx.x == 0) s_pos += round;
-            __syncthreads();
+            at += __shfl_sync(kAll, upto, 31);
         }
     }
-    const int64_t total = s_pos;
-    if (out)
-        for (int64_t i = total + threadIdx.x; i < hist_cap; i += blockDim.x) {
-            out[2 * i] = 0;
-            out[2 * i + 1] = 0;
-        }
     if (threadIdx.x == 0) {
-        if (n_sizes) n_sizes[lat] = total;
-        if (out && total > hist_cap) atomicExch(err, XY_EINVAL);
+        if (n_sizes) n_sizes[lat] = pos;
+        if (out && pos > hist_cap) atomicExch(err, XY_EINVAL);
     }
 }
 
@@ -771,7 +806,8 @@ cudaError_t launch_ccl(const float* theta, int Lx, int Ly, int n_lat, int32_t* l
     if ((e = cudaMemsetAsync(s.list_n, 0, sizeof(int), st)) != cudaSuccess) return e;
     ccl_tile_kernel<<<(unsigned)((tiles + kTileWarps - 1) / kTileWarps), 32 * kTileWarps, 0, st>>>(
         theta, Lx, Ly, n_lat, labels, s, err);
-    ccl_border_kernel<<<(unsigned)((tiles + 7) / 8), 256, 0, st>>>(Lx, Ly, n_lat, labels, s, err);
+    ccl_border_kernel<<<(unsigned)((tiles + 7) / 8), 256, 0, st>>>(Lx, Ly, n_lat, labels, s, hist,
+                                                                    hist ? 2 * hist_cap * n_lat : 0, err);
     const unsigned g = (unsigned)std::min<int64_t>((s.list_cap + 255) / 256, 152 * 8);
     ccl_list_size_kernel<<<g, 256, 0, st>>>(N, labels, s, err);
     ccl_list_hist_kernel<<<g, 256, 0, st>>>(N, s, err);
