@@ -571,7 +571,11 @@ __global__ void __launch_bounds__(256) ccl_list_hist_kernel(int64_t N, CclScratc
 // itself): so the warp reads the tile's labels once (16 rows at a time per
 // lane), keeps them in shared memory, and looks every tile root up there.  A
 // site whose tile root is still a root is final and is not written.
-__global__ void __launch_bounds__(256, 4) ccl_flatten_kernel(int Lx, int Ly, int n_lat, float inv_lx, int32_t* labels)
+// A width that is a power of two (shift >= 0) gives a label's row and column by a
+// shift and a mask; others by a product and a correction.
+template <bool POW2>
+__global__ void __launch_bounds__(256, 4) ccl_flatten_kernel(int Lx, int Ly, int n_lat, float inv_lx, int shift,
+                                                             int32_t* labels)
 {
     __shared__ int T[8][32 * 33];
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
@@ -602,33 +606,44 @@ __global__ void __launch_bounds__(256, 4) ccl_flatten_kernel(int Lx, int Ly, int
     for (int y = 0; y < thh; ++y) {
         const int li = Tw[y * 33 + lane];
         const int d = li - base;  // a site of the tile at row ry, column rx: d = ry * Lx + rx
-        int ry = (int)((float)d * inv_lx);
-        if (ry * Lx > d)
-            --ry;
-        else if ((ry + 1) * Lx <= d)
-            ++ry;
-        const int rx = d - ry * Lx;
+        int ry, rx;
+        if (POW2) {
+            ry = d >> shift;
+            rx = d & (Lx - 1);
+        } else {
+            ry = (int)((float)d * inv_lx);
+            if (ry * Lx > d)
+                --ry;
+            else if ((ry + 1) * Lx <= d)
+                ++ry;
+            rx = d - ry * Lx;
+        }
         // a label outside the tile belongs to a tile root whose entry points
         // at its domain's root already: final
-        if (ry >= 0 && ry < thh && rx >= 0 && rx < tw) {
+        if ((unsigned)ry < (unsigned)thh && (unsigned)rx < (unsigned)tw) {
             const int p = Tw[ry * 33 + rx];
             if (p != li) L[base + y * Lx + lane] = p;
         }
     }
 }
 
+constexpr int kWordList = 1024;
+
 // Pass 5: ordered compaction of the nonzero counts into (size, count) pairs,
 // one block per lattice, ascending size (the rest of the lattice's hist_cap
 // pairs is zero already).  Sizes 1..63 are summed over their copies; larger ones
 // are found through the bitmap, one bit per size: a warp takes 1024 consecutive
 // words, all 32 loads of a lane in flight, the warps' bits are summed in one
-// block-wide prefix, and each warp then places its own without further barriers
-// (a round of 1024 words at a time took four barriers per round).
-__global__ void __launch_bounds__(1024) ccl_compact_kernel(int64_t N, CclScratch s, int64_t* hist, int64_t hist_cap,
+// block-wide prefix, and the words that hold any go onto a list that all warps
+// share, a lane per size: a lane that walked a dense word waited for one count
+// after the other, and a round of 1024 words at a time took four barriers.
+__global__ void __launch_bounds__(1024, 1) ccl_compact_kernel(int64_t N, CclScratch s, int64_t* hist, int64_t hist_cap,
                                                            int64_t* n_sizes, int* err)
 {
     __shared__ int s_warp[32];
     __shared__ int s_small[kSmallSizes];
+    __shared__ uint4 s_list[kWordList];  // word index, word, position of its first pair
+    __shared__ int s_n;
     const int lat = blockIdx.x;
     int32_t* cnt = s.counts + (int64_t)lat * (N + 1);
     uint32_t* bw = s.bits + (int64_t)lat * s.words;
@@ -637,6 +652,7 @@ __global__ void __launch_bounds__(1024) ccl_compact_kernel(int64_t N, CclScratch
     const unsigned below = (1u << lane) - 1u;
     const int n_small = (int)(N < kSmallSizes - 1 ? N : kSmallSizes - 1);  // sizes 1..n_small
     if (threadIdx.x < kSmallSizes) s_small[threadIdx.x] = 0;
+    if (threadIdx.x == 0) s_n = 0;
     __syncthreads();
     {
         // thread j adds copies j / 64, j / 64 + 16, ... of size j % 64: every
@@ -692,32 +708,47 @@ __global__ void __launch_bounds__(1024) ccl_compact_kernel(int64_t N, CclScratch
             at += w < warp ? s_warp[w] : 0;
             pos += s_warp[w];
         }
-        if (c == 0) continue;  // the whole warp; the barriers above are met by all
-#pragma unroll
-        for (int k = 0; k < 32; ++k) {
-            const uint32_t word = wd[k];
-            if (!__any_sync(kAll, word != 0u)) continue;
-            const int n = __popc(word);
-            int upto = n;  // inclusive prefix over the warp
-#pragma unroll
-            for (int d = 1; d < 32; d <<= 1) {
-                const int o = __shfl_up_sync(kAll, upto, d);
-                if (lane >= d) upto += o;
+        auto place = [&](int64_t w, int bit, int64_t a) {
+            const int64_t z = (w << 5) + bit;
+            if (out && a < hist_cap) {
+                out[2 * a] = z;
+                out[2 * a + 1] = cnt[z];
             }
-            int64_t a = at + upto - n;
-            const int64_t w = wbase + 32 * k;
-            for (uint32_t b = word; b; b &= b - 1) {
-                const int64_t z = (w << 5) + __ffs(b) - 1;
-                if (out && a < hist_cap) {
-                    out[2 * a] = z;
-                    out[2 * a + 1] = cnt[z];
+            cnt[z] = 0;
+        };
+        if (c != 0) {  // the whole warp
+#pragma unroll
+            for (int k = 0; k < 32; ++k) {
+                const uint32_t word = wd[k];
+                if (!__any_sync(kAll, word != 0u)) continue;
+                const int n = __popc(word);
+                int upto = n;  // inclusive prefix over the warp
+#pragma unroll
+                for (int d = 1; d < 32; d <<= 1) {
+                    const int o = __shfl_up_sync(kAll, upto, d);
+                    if (lane >= d) upto += o;
                 }
-                cnt[z] = 0;
-                ++a;
+                if (word) {
+                    const int64_t w = wbase + 32 * k;
+                    int64_t a = at + upto - n;
+                    bw[w] = 0;
+                    const int e = atomicAdd(&s_n, 1);
+                    if (e < kWordList) {
+                        s_list[e] = make_uint4((unsigned)w, word, (unsigned)a, (unsigned)(a >> 32));
+                    } else {
+                        for (uint32_t b = word; b; b &= b - 1) place(w, __ffs(b) - 1, a++);
+                    }
+                }
+                at += __shfl_sync(kAll, upto, 31);
             }
-            if (word) bw[w] = 0;
-            at += __shfl_sync(kAll, upto, 31);
         }
+        __syncthreads();
+        for (int e = warp; e < min(s_n, kWordList); e += 32) {
+            const uint4 q = s_list[e];
+            if ((q.y >> lane) & 1u) place(q.x, lane, (int64_t)(((uint64_t)q.w << 32) | q.z) + __popc(q.y & below));
+        }
+        __syncthreads();
+        if (threadIdx.x == 0) s_n = 0;
     }
     if (threadIdx.x == 0) {
         if (n_sizes) n_sizes[lat] = pos;
@@ -811,7 +842,10 @@ cudaError_t launch_ccl(const float* theta, int Lx, int Ly, int n_lat, int32_t* l
     const unsigned g = (unsigned)std::min<int64_t>((s.list_cap + 255) / 256, 152 * 8);
     ccl_list_size_kernel<<<g, 256, 0, st>>>(N, labels, s, err);
     ccl_list_hist_kernel<<<g, 256, 0, st>>>(N, s, err);
-    ccl_flatten_kernel<<<(unsigned)((tiles + 7) / 8), 256, 0, st>>>(Lx, Ly, n_lat, 1.0f / (float)Lx, labels);
+    int shift = 0;
+    while ((1 << shift) < Lx) ++shift;
+    const auto flatten = (1 << shift) == Lx ? ccl_flatten_kernel<true> : ccl_flatten_kernel<false>;
+    flatten<<<(unsigned)((tiles + 7) / 8), 256, 0, st>>>(Lx, Ly, n_lat, 1.0f / (float)Lx, shift, labels);
     ccl_compact_kernel<<<n_lat, 1024, 0, st>>>(N, s, hist, hist_cap, n_sizes, err);
     return cudaGetLastError();
 }
