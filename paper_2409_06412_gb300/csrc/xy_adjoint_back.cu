@@ -40,6 +40,9 @@ constexpr int kStages = 3;
 
 __device__ __forceinline__ int wrapb(int v, int n) { return v < 0 ? v + n : (v >= n ? v - n : v); }
 
+// (through L2: another block may have written the row, in this launch)
+__device__ __forceinline__ float4 ldcg4(const float* p) { return __ldcg(reinterpret_cast<const float4*>(p)); }
+
 __device__ __forceinline__ P4 sub4(const P4& x, const P4& y) { return fma4(-1.0f, y, x); }
 
 // theta_k = wrap(theta_{k+1} - dt v_{k+1}): the drift of step k undone, with
@@ -87,8 +90,15 @@ struct RowK {
 // formed beside phase B, whose chain is short of independent work.  Unrolled by
 // three, without copies of the window, the loop outgrew the instruction cache and
 // gained nothing.  64 lattices of 256 x 256, 8-row bands, four slices at once: 200 ->
-// 136 instructions per site, 35.8 -> 28.1 us per step (half of the issue slots).
-template <bool WIDE, bool OBS, bool BACK, bool SCHED>
+// 136 instructions per site, 35.8 -> 26.8 us per step (half of the issue slots).
+//
+// SWEEP (observed backward steps only): one launch reverses the steps R.k down to
+// R.k_last.  The blocks of a lattice are a thread-block cluster (eight at most) and
+// meet at its barrier after every step, so a small lattice pays a barrier per step
+// where a launch per step paid its start, its prologue and the drain of the one
+// before (4 lattices of 64 x 64: 8.6 -> 6.5 us per
+// step, 12 at the start).
+template <bool WIDE, bool OBS, bool BACK, bool SCHED, bool SWEEP>
 __global__ void __launch_bounds__(512, 1) adjoint_back_kernel(const DevCfg* cfgs, const BandTask* tasks, int H,
                                                               BackArgs R, PhiloxKeys keys)
 {
@@ -115,32 +125,53 @@ __global__ void __launch_bounds__(512, 1) adjoint_back_kernel(const DevCfg* cfgs
     const int wR = WIDE && lane == 31 ? (warp + 1) % n_warps : warp;
     const int lL = grp * G + (lg + G - 1) % G, lR = grp * G + (lg + 1) % G;
     const int64_t b = cf.b_first + task.rep;
-    // one pointer and the other arrays' distances from it, which stay kernel
-    // parameters: eight pointers would take sixteen registers
-    char* const base = (char*)(R.th_in + cf.offset + (int64_t)task.rep * cf.N + x);
-    auto at = [&](int64_t dist, int o) { return reinterpret_cast<float*>(base + dist + 4 * (int64_t)o); };
+    const int64_t lat_off = cf.offset + (int64_t)task.rep * cf.N + x;
     const int slot_j = task.band0 / per_block;  // this block's partial of M
     const int n_parts = (task.n_bands + per_block - 1) / per_block;
-    const StepConst K = SCHED ? step_const_k(cf, R.k, noise_amp(cf, R.k)) : step_const(cf, noise_amp(cf, R.k));
-    const float q2 = K.q * K.q, hp2 = K.hp * cf.p;
     const float invN = 1.0f / (float)cf.N, wE = R.wE;
     const uint32_t cfgrep = ((uint32_t)cf.noise_cfg << 16) | (uint32_t)(cf.rep0 + task.rep);
+    double total = 0.0;  // this thread's gradient sum over the steps
+    for (int64_t k = R.k;; --k) {
+    // one pointer and the other arrays' distances from it, which stay kernel
+    // parameters in a launch of one step: eight pointers would take sixteen registers
+    const float* in = R.th_in;
+    int64_t d_v_in = R.d_v_in, d_tb_in = R.d_tb_in, d_vb_in = R.d_vb_in, d_th_out = R.d_th_out, d_v_out = R.d_v_out,
+            d_tb_out = R.d_tb_out, d_vb_out = R.d_vb_out;
+    if (SWEEP) {
+        const int par = (int)((R.k - k) & 1);  // the buffers alternate from the first step on
+        if (k < R.k) {
+            const int64_t m = k + 1 - R.k0;  // the state of step k + 1: a checkpoint, or the last step's output
+            in = m < R.n && m % R.seg == 0 ? R.ck + 2 * R.T * (m / R.seg) : R.sbuf + 2 * R.T * (R.sb ^ par ^ 1);
+            d_v_in = 4 * R.T;
+        }
+        auto dist = [&](const float* q) { return (int64_t)((const char*)q - (const char*)in); };
+        const float* out = R.sbuf + 2 * R.T * (R.sb ^ par);
+        d_th_out = dist(out);
+        d_v_out = d_th_out + 4 * R.T;
+        d_tb_in = dist(R.adjb + 2 * R.T * (R.acur ^ par));
+        d_vb_in = d_tb_in + 4 * R.T;
+        d_tb_out = dist(R.adjb + 2 * R.T * (R.acur ^ par ^ 1));
+        d_vb_out = d_tb_out + 4 * R.T;
+    }
+    char* const base = (char*)(in + lat_off);
+    auto at = [&](int64_t dist, int o) { return reinterpret_cast<float*>(base + dist + 4 * (int64_t)o); };
+    const StepConst K = SCHED ? step_const_k(cf, k, noise_amp(cf, k)) : step_const(cf, noise_amp(cf, k));
+    const float q2 = K.q * K.q, hp2 = K.hp * cf.p;
     auto noise = [&](int o) {
-        return p4(gauss4_scaled(philox4x32_10_rk(noise_counter((uint32_t)(o + x) >> 2, cfgrep, R.k, 0u), keys), K.c));
+        return p4(gauss4_scaled(philox4x32_10_rk(noise_counter((uint32_t)(o + x) >> 2, cfgrep, k, 0u), keys), K.c));
     };
     P4 nz = noise(wrapb(y0 - 1, Ly) * Lx);
-    dependency_wait();  // the states, adjoints and partial sums of the launch before
-    // M_{k+1} from the previous launch's partials (fixed order), recorded by
+    if (!SWEEP || k == R.k) dependency_wait();  // the states, adjoints and partial sums of the launch before
+    // M_{k+1} from the previous step's partials (fixed order), recorded by
     // the lattice's first block; its sign weights the deferred |M| term
     if (warp == 0) {
         float w = 0.f;
         if (BACK) {
-            const double* mp = R.mpart + (b * 2 + ((R.k + 1) & 1)) * R.P;
+            const double* mp = R.mpart + (b * 2 + ((k + 1) & 1)) * R.P;
             double m = 0.0;
-            for (int j = lane; j < n_parts; j += 32) m += mp[j];
+            for (int j = lane; j < n_parts; j += 32) m += __ldcg(&mp[j]);
             for (int o = 1; o < 32 && o < n_parts; o <<= 1) m += __shfl_xor_sync(kFullB, m, o);
-            m /= (double)cf.N;
-            if (slot_j == 0 && lane == 0) R.rec[b * R.rec_stride + (R.k + 1 - R.k0)].x = m;
+            if (slot_j == 0 && lane == 0) R.rec[b * R.rec_stride + (k + 1 - R.k0)].x = m;  // N M_{k+1}
             const float wq = R.wM * invN * K.q;
             w = m > 0.0 ? wq : (m < 0.0 ? -wq : 0.f);
         }
@@ -148,9 +179,9 @@ __global__ void __launch_bounds__(512, 1) adjoint_back_kernel(const DevCfg* cfgs
     }
     // configuration constants in registers (the cp.async statements clobber
     // memory, which would otherwise reload them from the descriptor every row)
-    const float2 Jk = SCHED ? couplings_at(cf, R.k) : make_float2(cf.Jx, cf.Jy);
-    const float2 abk = SCHED ? coupling_scales(cf, R.k) : make_float2(1.f, 1.f);
-    const float Jx = Jk.x, Jy = Jk.y, hF = SCHED ? field_h(cf, R.k) : cf.h;
+    const float2 Jk = SCHED ? couplings_at(cf, k) : make_float2(cf.Jx, cf.Jy);
+    const float2 abk = SCHED ? coupling_scales(cf, k) : make_float2(1.f, 1.f);
+    const float Jx = Jk.x, Jy = Jk.y, hF = SCHED ? field_h(cf, k) : cf.h;
     const float q2Jx = q2 * Jx, q2Jy = q2 * Jy;
     const bool stag = cf.stag != 0;
     const float wEn = wE * invN;
@@ -172,9 +203,9 @@ __global__ void __launch_bounds__(512, 1) adjoint_back_kernel(const DevCfg* cfgs
     auto issue = [&](int ii, int slot) {
         if (ii < n_it) {
             cp_async16(&me.th[slot][lane], at(0, o_ld));
-            cp_async16(&me.v[slot][lane], at(R.d_v_in, BACK ? o_ld : o_ldt));
-            cp_async16(&me.tb[slot][lane], at(R.d_tb_in, o_ldt));
-            cp_async16(&me.vb[slot][lane], at(R.d_vb_in, o_ldt));
+            cp_async16(&me.v[slot][lane], at(d_v_in, BACK ? o_ld : o_ldt));
+            cp_async16(&me.tb[slot][lane], at(d_tb_in, o_ldt));
+            cp_async16(&me.vb[slot][lane], at(d_vb_in, o_ldt));
             o_ldt = o_ld;
             o_ld = adv(o_ld);
         }
@@ -195,15 +226,15 @@ __global__ void __launch_bounds__(512, 1) adjoint_back_kernel(const DevCfg* cfgs
         const int r_m1 = wrapb(y0 - 2, Ly) * Lx, r_0 = o_a;
         P4 t0;
         if (BACK) {
-            const P4 t = undrift(p4(ld4(at(0, r_m1))), p4(ld4(at(R.d_v_in, r_m1))), K.dt);
+            const P4 t = undrift(p4(ldcg4(at(0, r_m1))), p4(ldcg4(at(d_v_in, r_m1))), K.dt);
             quad_sc(K.q, t, k1.s, k1.c);
             // theta_{k+1}, v_{k+1} of row t stay in the last iteration's stage
-            me.th[2][lane] = ld4(at(0, r_0));
-            me.v[2][lane] = ld4(at(R.d_v_in, r_0));
+            me.th[2][lane] = ldcg4(at(0, r_0));
+            me.v[2][lane] = ldcg4(at(d_v_in, r_0));
             t0 = undrift(p4(me.th[2][lane]), p4(me.v[2][lane]), K.dt);
         } else {
-            quad_sc(K.q, p4(ld4(at(0, r_m1))), k1.s, k1.c);
-            t0 = p4(ld4(at(0, r_0)));
+            quad_sc(K.q, p4(ldcg4(at(0, r_m1))), k1.s, k1.c);
+            t0 = p4(ldcg4(at(0, r_0)));
         }
         quad_sc(K.q, t0, k2.s, k2.c);
         me.th0[1][lane] = f4(t0);
@@ -303,10 +334,10 @@ __global__ void __launch_bounds__(512, 1) adjoint_back_kernel(const DevCfg* cfgs
             // ((vk + g) / (1 + a)^2 is om / (1 + a)), in one sum
             dot(abar, om, gb);
             dot(cbar, gb, nz);
-            st4(at(R.d_vb_out, o_a), f4(vbk));
+            st4(at(d_vb_out, o_a), f4(vbk));
             if (BACK) {
-                st4(at(R.d_th_out, o_a), f4(thC));
-                st4(at(R.d_v_out, o_a), f4(vk));
+                st4(at(d_th_out, o_a), f4(thC));
+                st4(at(d_v_out, o_a), f4(vk));
             }
         }
         if (WIDE) __syncthreads(); else __syncwarp();
@@ -323,7 +354,7 @@ __global__ void __launch_bounds__(512, 1) adjoint_back_kernel(const DevCfg* cfgs
             const P4 gn = mul4(bym, sub4(fb, f));
             const P4 out = fma4(q2Jx, hx, fma4(q2Jy, sub4(gn, gy), p4(me.tbp[own_slot ^ 1][lane])));
             gy = gn;
-            if (active && i >= 2) st4(at(R.d_tb_out, o_b), f4(out));
+            if (active && i >= 2) st4(at(d_tb_out, o_b), f4(out));
         }
         bym = byn;
         o_b = o_a;
@@ -338,40 +369,48 @@ __global__ void __launch_bounds__(512, 1) adjoint_back_kernel(const DevCfg* cfgs
         slot = slot == 2 ? 0 : slot + 1;
     }
     cp_async_wait<0>();
-    launch_next();
+    if (!SWEEP || k == R.k_last) launch_next();
     // per-block accumulators: FP32 warp butterflies, the warps and the steps
     // combined in FP64 in a fixed order; the partial of M_k goes to the ring
     auto both = [](float2 v) { return v.x + v.y; };
     const float vals[kGacc + 1] = {
         fmaf(-K.q, both(aJx), -wEn * both(sbx)) * abk.x,                              // d/d J_par (J_par(k) = J_par a(k))
         fmaf(-K.q, both(aJy), -wEn * both(sby)) * abk.y,                              // d/d J_perp (J_perp b(k))
-        fmaf(K.p, both(ah), wEn * both(scp)) * (SCHED ? field_scale(cf, R.k) : 1.f),  // d/d h (h_k = h s(k))
+        fmaf(K.p, both(ah), wEn * both(scp)) * (SCHED ? field_scale(cf, k) : 1.f),  // d/d h (h_k = h s(k))
         -both(abar), 0.f, both(cbar),
         wEn * fmaf(0.5f, both(sw2), fmaf(-Jx, both(sbx), fmaf(-Jy, both(sby), hF * both(scp)))),  // w_E E / N
         both(pm),                                                                      // sum of sigma sin(q theta_k)
     };
 #pragma unroll
-    for (int k = 0; k < kGacc + 1; ++k) {
-        const float w = warp_sumf_b(vals[k]);
-        if (lane == 0) s_red[k][warp] = w;
+    for (int i = 0; i < kGacc + 1; ++i) {
+        const float w = warp_sumf_b(vals[i]);
+        if (lane == 0) s_red[i][warp] = w;
     }
     __syncthreads();
     if (threadIdx.x < kGacc + 1) {
-        double acc = 0.0;
-        for (int w2 = 0; w2 < n_warps; ++w2) acc += s_red[threadIdx.x][w2];
-        if (threadIdx.x == kGacc) {
-            R.mpart[(b * 2 + (R.k & 1)) * R.P + slot_j] = acc;
-        } else {
-            // c-bar (summed against c_k n_k) enters the eta gradient through
-            // d c_k / d eta = c_k / (2 eta)
-            if (threadIdx.x == 5) acc *= cf.eta_d > 0.0 ? 1.0 / (2.0 * cf.eta_d) : 0.0;
-            R.gacc[(int64_t)(R.block_base + blockIdx.x) * kGacc + threadIdx.x] += acc;
-        }
+        double p4s[4] = {0.0, 0.0, 0.0, 0.0};  // (an FP64 addition takes dozens of cycles: four chains)
+        for (int w2 = 0; w2 < n_warps; ++w2) p4s[w2 & 3] += s_red[threadIdx.x][w2];
+        const double acc = (p4s[0] + p4s[1]) + (p4s[2] + p4s[3]);
+        if (threadIdx.x == kGacc) R.mpart[(b * 2 + (k & 1)) * R.P + slot_j] = acc;
+        total += acc;
     }
+    if (!SWEEP || k == R.k_last) break;
+    // every block of the lattice has written its rows and its partial of M_k
+    // (released to the cluster by the arrival)
+    __syncwarp();
+    asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;\n" ::: "memory");
+    }
+    if (threadIdx.x < kGacc) R.gacc[(int64_t)(R.block_base + blockIdx.x) * kGacc + threadIdx.x] += total;
 }
 
+// Blocks of a lattice that one launch may sweep over its steps: the cluster size, or
+// 0 where they are too many for a (portable) cluster.
+int back_sweep_cluster(int blocks_per_lattice) { return blocks_per_lattice <= 8 ? blocks_per_lattice : 0; }
+
+// sweep > 0: steps R.k .. R.k_last in one launch, clusters of `sweep` blocks (a
+// lattice's blocks, consecutive tasks); 0: step R.k.
 cudaError_t launch_adjoint_back(const DevCfg* d_cfg, const BandTask* tasks, int n_tasks, int Lx, int H, uint64_t seed,
-                                bool back, BackArgs R, bool after, cudaStream_t st)
+                                bool back, int sweep, BackArgs R, bool after, cudaStream_t st)
 {
     if (n_tasks == 0) return cudaSuccess;
     const bool wide = Lx > 128;
@@ -379,17 +418,17 @@ cudaError_t launch_adjoint_back(const DevCfg* d_cfg, const BandTask* tasks, int 
     const int smem = (threads / 32) * (int)sizeof(BackWarp);
     const bool obs = R.k > R.k0;
     using Kern = void (*)(const DevCfg*, const BandTask*, int, BackArgs, PhiloxKeys);
-    static const Kern table[2][2][2][2] = {
-        {{{adjoint_back_kernel<false, false, false, false>, adjoint_back_kernel<false, false, true, false>},
-          {adjoint_back_kernel<false, true, false, false>, adjoint_back_kernel<false, true, true, false>}},
-         {{adjoint_back_kernel<true, false, false, false>, adjoint_back_kernel<true, false, true, false>},
-          {adjoint_back_kernel<true, true, false, false>, adjoint_back_kernel<true, true, true, false>}}},
-        {{{adjoint_back_kernel<false, false, false, true>, adjoint_back_kernel<false, false, true, true>},
-          {adjoint_back_kernel<false, true, false, true>, adjoint_back_kernel<false, true, true, true>}},
-         {{adjoint_back_kernel<true, false, false, true>, adjoint_back_kernel<true, false, true, true>},
-          {adjoint_back_kernel<true, true, false, true>, adjoint_back_kernel<true, true, true, true>}}},
-    };
-    const Kern kern = table[R.sched != 0][wide][obs][back];
+#define BACK_ROW(W, S)                                                                                       \
+    {{adjoint_back_kernel<W, false, false, S, false>, adjoint_back_kernel<W, false, true, S, false>},        \
+     {adjoint_back_kernel<W, true, false, S, false>, adjoint_back_kernel<W, true, true, S, false>}}
+    static const Kern table[2][2][2][2] = {{BACK_ROW(false, false), BACK_ROW(true, false)},
+                                           {BACK_ROW(false, true), BACK_ROW(true, true)}};
+#undef BACK_ROW
+    static const Kern sweeps[2][2] = {
+        {adjoint_back_kernel<false, true, true, false, true>, adjoint_back_kernel<true, true, true, false, true>},
+        {adjoint_back_kernel<false, true, true, true, true>, adjoint_back_kernel<true, true, true, true, true>}};
+    if (sweep > 0 && (!back || R.k_last <= R.k0 || n_tasks % sweep != 0)) return cudaErrorInvalidValue;
+    const Kern kern = sweep > 0 ? sweeps[R.sched != 0][wide] : table[R.sched != 0][wide][obs][back];
     if (smem > 46 * 1024) {  // (the limit belongs to the kernel, which other shapes share: always the largest)
         const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                    kMaxBackWarps * (int)sizeof(BackWarp));
@@ -403,7 +442,7 @@ cudaError_t launch_adjoint_back(const DevCfg* d_cfg, const BandTask* tasks, int 
     R.d_v_out = dist(R.v_out);
     R.d_tb_out = dist(R.tb_out);
     R.d_vb_out = dist(R.vb_out);
-    return launch_dependent(kern, (unsigned)n_tasks, (unsigned)threads, (size_t)smem, st, after, d_cfg, tasks, H, R,
+    return launch_dependent(kern, (unsigned)n_tasks, (unsigned)threads, (size_t)smem, st, after, sweep, d_cfg, tasks, H, R,
                             philox_round_keys(seed));
 }
 

@@ -1138,6 +1138,18 @@ int autotune_lattice(xy_lattice* L)
     return rc;
 }
 
+// The task tables that no tuner run has built (groups too small for it, or the
+// tuner switched off).
+int ensure_tasks(xy_lattice* L)
+{
+    for (auto& g : L->strip_groups) {
+        int rc = g.strip_ok && g.tasks.empty() ? build_strip_tasks(L, g) : XY_OK;
+        if (rc == XY_OK && g.band_H > 0 && g.band_tasks.empty()) rc = build_band_tasks(L, g, g.band_H);
+        if (rc) return rc;
+    }
+    return XY_OK;
+}
+
 constexpr int kChunk = 64;             // steps of a captured chunk at most (the bits of cur_mask)
 constexpr int kResidentSteps = 1 << 14;  // steps of one resident launch at most
 
@@ -1250,8 +1262,9 @@ int fixup_parity(xy_lattice* L)
 int advance_core(xy_lattice* L, int64_t n, int record_every, double2* rec_dev, int64_t rec_stride,
                  bool do_moments, int64_t t0, bool m_only = false)
 {
-    if (L->path == XY_PATH_BATCHED && !L->tuned) {
-        int rc0 = autotune_lattice(L);
+    if (L->path == XY_PATH_BATCHED) {
+        int rc0 = L->tuned ? XY_OK : autotune_lattice(L);
+        if (rc0 == XY_OK) rc0 = ensure_tasks(L);
         if (rc0) return rc0;
     }
     int64_t n_max = 0;
@@ -1402,12 +1415,11 @@ int classify(xy_lattice* L)
         CK(cudaMemcpy(g.d_tasks, g.tasks.data(), sizeof(ResidentTask) * g.tasks.size(), cudaMemcpyHostToDevice));
         CK(prepare_resident(g.Lx, g.Ly, g.threads, g.csize, nullptr));
     }
-    for (auto& g : L->strip_groups) {
-        int rc = g.strip_ok ? build_strip_tasks(L, g) : XY_OK;
-        if (rc == XY_OK && band_shape(g.Lx, g.Ly))
-            rc = build_band_tasks(L, g, default_band_H(g.Lx, g.Ly, g.n_lat, (int64_t)sms * 14 / (int64_t)L->strip_groups.size()));
-        if (rc) return rc;
-    }
+    // (the task tables of the strip groups are built at the first batched step:
+    // the tuner, which runs there, chooses their heights)
+    for (auto& g : L->strip_groups)
+        if (band_shape(g.Lx, g.Ly))
+            g.band_H = default_band_H(g.Lx, g.Ly, g.n_lat, (int64_t)sms * 14 / (int64_t)L->strip_groups.size());
     apply_kt_mode(L);
     return XY_OK;
 }
@@ -2030,19 +2042,6 @@ int xy_adjoint_step_n(xy_lattice* L, int64_t n, int K, double wE, double wM, dou
             for (int r = 0; r < L->cfg[c].desc.n_replicas; ++r)
                 for (int b0 = 0; b0 < nb; b0 += per_block) out.push_back(BandTask{c, r, b0, nb});
     };
-    // default band height: the largest H <= 64 dividing Ly that still gives 8
-    // warps per SM over the batch (each warp walks its rows serially)
-    auto default_H = [&](const AdjGroup& g) {
-        const int warps_per_band = g.wide ? g.Lx / 128 : 1;
-        const int groups = g.wide ? 1 : 32 / (g.Lx / 4);
-        int H = 1;
-        for (int h : {64, 32, 16, 8, 4, 2, 1}) {
-            if (g.Ly % h != 0) continue;
-            H = h;
-            if (g.n_lat * (g.Ly / h) * warps_per_band / groups >= (int64_t)sms * 8) break;
-        }
-        return H;
-    };
     // states of a segment: integrated backward from the checkpoint at its end
     // inside the reverse kernel (band shapes only), or recomputed forward
     // from the checkpoint at its start and stored
@@ -2060,6 +2059,28 @@ int xy_adjoint_step_n(xy_lattice* L, int64_t n, int K, double wE, double wM, dou
         damp = std::max(damp, L->h_dev[c].eta_d * L->h_dev[c].dt_d * (double)std::min<int64_t>(K, n));
     const bool back = L->adj_mode != XY_ADJOINT_RECOMPUTE && adj_plain.empty() && !adj_groups.empty() &&
                       (L->adj_mode == XY_ADJOINT_BACKWARD || damp <= kAutoBackMaxDamping);
+    // default band height: the largest H <= 64 dividing Ly that still gives 8
+    // warps per SM over the batch (each warp walks its rows serially)
+    auto default_H = [&](const AdjGroup& g) {
+        const int warps_per_band = g.wide ? g.Lx / 128 : 1;
+        const int groups = g.wide ? 1 : 32 / (g.Lx / 4);
+        // backward integration of lattices whose blocks fit a cluster, all at once:
+        // the lowest such band, up to 4 rows (a step then takes as long as H + 2 rows)
+        for (int h : {1, 2, 4}) {
+            if (!back || g.Ly % h != 0) continue;
+            const int per_block = g.wide ? 1 : 8 * groups;
+            const int blocks = (g.Ly / h + per_block - 1) / per_block;
+            const int64_t warps = g.n_lat * blocks * (g.wide ? g.Lx / 128 : 8);
+            if (back_sweep_cluster(blocks) > 0 && warps <= (int64_t)sms * 12 / (int64_t)adj_groups.size()) return h;
+        }
+        int H = 1;
+        for (int h : {64, 32, 16, 8, 4, 2, 1}) {
+            if (g.Ly % h != 0) continue;
+            H = h;
+            if (g.n_lat * (g.Ly / h) * warps_per_band / groups >= (int64_t)sms * 8) break;
+        }
+        return H;
+    };
     float *ck = nullptr, *seg = nullptr, *adjb = nullptr, *Fb = nullptr, *sbuf = nullptr;
     double2* arec = nullptr;
     double *gacc = nullptr, *mpart = nullptr;
@@ -2147,7 +2168,7 @@ int xy_adjoint_step_n(xy_lattice* L, int64_t n, int K, double wE, double wM, dou
                         A.gacc = g_tmp;
                         return launch_sliced(L, cuts, reps, [&](cudaStream_t st, int t0, int cnt) {
                             A.block_base = t0;
-                            return launch_adjoint_back(L->d_cfg, d_tk + t0, cnt, g.Lx, h, g.seed, true, A, false, st);
+                            return launch_adjoint_back(L->d_cfg, d_tk + t0, cnt, g.Lx, h, g.seed, true, 0, A, false, st);
                         });
                     }
                     BandArgs R{};
@@ -2302,6 +2323,15 @@ int xy_adjoint_step_n(xy_lattice* L, int64_t n, int K, double wE, double wM, dou
         }
         if (n_aux > 0) CKA(cudaEventRecord(L->fork_ev, L->stream));
         for (int i = 0; i < n_aux; ++i) CKA(cudaStreamWaitEvent(L->aux[i], L->fork_ev, 0));
+        // Groups whose lattices are clusters that all run at once sweep the steps
+        // k0 + n - 1 .. k0 + 1 in one launch per slice.
+        std::vector<int> sweep(adj_groups.size(), 0);
+        for (size_t gi = 0; gi < adj_groups.size(); ++gi) {
+            const AdjGroup& g = adj_groups[gi];
+            const int warps = g.wide ? g.Lx / 128 : 8;
+            if (n >= 3 && (int64_t)g.tasks.size() * warps <= (int64_t)sms * 12 / (int64_t)adj_groups.size())
+                sweep[gi] = back_sweep_cluster((int)(g.tasks.size() / g.n_lat));
+        }
         for (int64_t k = k0 + n; k >= k0; --k) {
             const bool bk = k < k0 + n;
             const int64_t m = k + 1 - k0;
@@ -2311,7 +2341,14 @@ int xy_adjoint_step_n(xy_lattice* L, int64_t n, int K, double wE, double wM, dou
             }
             float* out_th = sbuf + 2 * T * sb;
             int q = 0;  // slice of the sweep
-            for (auto& g : adj_groups) {
+            for (size_t gi = 0; gi < adj_groups.size(); ++gi) {
+                AdjGroup& g = adj_groups[gi];
+                const auto& c = cuts[gi];
+                if (sweep[gi] > 0 && bk && k > k0 && k < k0 + n - 1) {  // in the sweep's launch at k0 + n - 1
+                    q += (int)c.size() - 1;
+                    continue;
+                }
+                const bool sweeps = sweep[gi] > 0 && bk && k == k0 + n - 1;
                 BackArgs A{};
                 A.sched = any_sched(L, g.cfgs);
                 A.th_in = in_th;
@@ -2331,11 +2368,22 @@ int xy_adjoint_step_n(xy_lattice* L, int64_t n, int K, double wE, double wM, dou
                 A.wE = (float)wE;
                 A.wM = (float)wM;
                 A.gacc = gacc;
-                const auto& c = cuts[&g - adj_groups.data()];
+                if (sweeps) {
+                    A.k_last = k0 + 1;
+                    A.seg = K;
+                    A.n = n;
+                    A.T = T;
+                    A.ck = ck;
+                    A.sbuf = sbuf;
+                    A.adjb = adjb;
+                    A.sb = sb;
+                    A.acur = acur;
+                }
                 for (size_t p = 0; p + 1 < c.size(); ++p, ++q) {
                     A.block_base = g.block_base + c[p];
-                    CKA(launch_adjoint_back(L->d_cfg, g.d_tasks + c[p], c[p + 1] - c[p], g.Lx, g.H, g.seed, bk, A,
-                                            bk && n_slices <= n_aux + 1, q == 0 ? L->stream : L->aux[(q - 1) % n_aux]));
+                    CKA(launch_adjoint_back(L->d_cfg, g.d_tasks + c[p], c[p + 1] - c[p], g.Lx, g.H, g.seed, bk,
+                                            sweeps ? sweep[gi] : 0, A, bk && n_slices <= n_aux + 1,
+                                            q == 0 ? L->stream : L->aux[(q - 1) % n_aux]));
                     ++L->launches;
                 }
             }
@@ -2472,8 +2520,13 @@ int xy_adjoint_step_n(xy_lattice* L, int64_t n, int K, double wE, double wM, dou
     // objective: w_E E summed by the reverse sweep, w_M |M_k| from the forward records
     double obj = 0.0;
     for (int c = 0; c < L->n_cfg; ++c) obj += acc[kGacc * c + 6];
-    for (int64_t b = 0; b < L->B; ++b)
-        for (int64_t k = 1; k <= n; ++k) obj += wM * std::fabs(hrec[b * R_ + k].x);
+    // (the backward sweep records the lattices' sums N M_k and leaves the factor of
+    // d c_k / d eta = c_k / (2 eta) out of the noise's sum: no FP64 division per step)
+    for (const DevCfg& d : L->h_dev) {
+        const double unit = back ? 1.0 / (double)d.N : 1.0;
+        for (int64_t b = d.b_first; b < d.b_first + d.n_rep; ++b)
+            for (int64_t k = 1; k <= n; ++k) obj += wM * std::fabs(hrec[b * R_ + k].x * unit);
+    }
     *objective = obj * inv_norm;
     for (int c = 0; c < L->n_cfg; ++c) {
         const xy_params& p = L->cfg[c].prm;
@@ -2482,7 +2535,8 @@ int xy_adjoint_step_n(xy_lattice* L, int64_t n, int K, double wE, double wM, dou
         grads[4 * c + 0] = ac[0] * inv_norm;
         grads[4 * c + 1] = ac[1] * inv_norm;
         grads[4 * c + 2] = ac[2] * inv_norm;
-        grads[4 * c + 3] = (0.5 * p.dt * (ac[3] - bb * bb * ac[4]) + ac[5]) * inv_norm;
+        const double noise = back ? (p.eta > 0.0 ? ac[5] / (2.0 * p.eta) : 0.0) : ac[5];
+        grads[4 * c + 3] = (0.5 * p.dt * (ac[3] - bb * bb * ac[4]) + noise) * inv_norm;
     }
     // restore the idle window
     set_window_idle(L);

@@ -129,21 +129,31 @@ struct Partials {
 };
 
 // Launch of a kernel that calls dependency_wait(): after = true lets it start while
-// the launch before it on the stream drains (programmatic dependent launch).
+// the launch before it on the stream drains (programmatic dependent launch);
+// cluster > 0: in clusters of so many blocks.
 template <class... P, class... A>
 cudaError_t launch_dependent(void (*kern)(P...), unsigned blocks, unsigned threads, size_t smem, cudaStream_t st, bool after,
-                             A... args)
+                             int cluster, A... args)
 {
     cudaLaunchConfig_t lc = {};
     lc.gridDim = dim3(blocks);
     lc.blockDim = dim3(threads);
     lc.dynamicSmemBytes = smem;
     lc.stream = st;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchAttribute at[2];
+    int n = 0;
+    if (after) {
+        at[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        at[n++].val.programmaticStreamSerializationAllowed = 1;
+    }
+    if (cluster > 0) {
+        at[n].id = cudaLaunchAttributeClusterDimension;
+        at[n].val.clusterDim.x = (unsigned)cluster;
+        at[n].val.clusterDim.y = 1;
+        at[n++].val.clusterDim.z = 1;
+    }
     lc.attrs = at;
-    lc.numAttrs = after ? 1 : 0;
+    lc.numAttrs = n;
     return cudaLaunchKernelEx(&lc, kern, P(args)...);
 }
 
@@ -292,11 +302,21 @@ struct BackArgs {
     double* gacc;        // [blocks][kGacc]
     int block_base;
     int sched;           // some configuration of the tasks has a field or coupling schedule
+    // a sweep over several steps: the last one, the segment length and the number of
+    // steps of the call, the sites of all lattices (the distance from theta to v and
+    // from tb to vb), the checkpoints, the two recovered states and the two adjoint
+    // states, with the ones that step k writes (sb) and reads (acur)
+    int64_t k_last, seg, n, T;
+    const float* ck;
+    float* sbuf;
+    float* adjb;
+    int sb, acur;
     // distances in bytes of the other arrays from th_in (set by launch_adjoint_back)
     int64_t d_v_in, d_tb_in, d_vb_in, d_th_out, d_v_out, d_tb_out, d_vb_out;
 };
 cudaError_t launch_adjoint_back(const DevCfg* d_cfg, const BandTask* tasks, int n_tasks, int Lx, int H, uint64_t seed,
-                                bool back, BackArgs R, bool after, cudaStream_t st);
+                                bool back, int sweep, BackArgs R, bool after, cudaStream_t st);
+int back_sweep_cluster(int blocks_per_lattice);
 // M_k of slots [0, n_states) of a segment (slot stride 2 T floats) into
 // rec[b * rec_stride + r0 + slot].x
 cudaError_t launch_segment_m(const DevCfg* d_cfg, int n_cfg, int64_t B, const float* seg, int64_t T, int n_states,

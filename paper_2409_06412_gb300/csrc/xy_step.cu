@@ -973,7 +973,7 @@ cudaError_t launch_band_step(const DevCfg* d_cfg, const BandTask* tasks, int n_t
                                                    (int)sizeof(BStage) * kBandWarps);
         if (e != cudaSuccess) return e;
     }
-    return launch_dependent(kern, (unsigned)n_tasks, 32 * warps, smem, st, after, d_cfg, tasks, H, n_steps, rd_b ? 1 : 0,
+    return launch_dependent(kern, (unsigned)n_tasks, 32 * warps, smem, st, after, 0, d_cfg, tasks, H, n_steps, rd_b ? 1 : 0,
                             j_local, buf, ca, pa, philox_round_keys(seed));
 }
 
