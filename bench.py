@@ -346,7 +346,7 @@ def run_ours(args):
 
     extra = {}
     if rank == 0:
-        # dominant kernel, timed live with events on its stream (the strip
+        # dominant kernel, timed live with events on its stream (the band
         # stepper carries every lattice with L >= 256)
         s_before = lat.observe()[1]
         lat.set_kernel_timing(True)
@@ -356,28 +356,40 @@ def run_ours(args):
         lat.set_kernel_timing(False)
         su_strip, su_res = done_su(s_before, lat.observe()[1])
         hbm, peak_kind = peaks()
-        # the strip stepper runs one launch per lattice shape per BBK step:
-        # the site-updates it did (from the step counters) and its summed
-        # launch time give bytes per launch over the average launch duration
+        # lattices with L >= 256 take two BBK steps per launch (the band
+        # stepper: the state crosses HBM once per pair, 8 B per site-update)
+        # and single steps where a pair does not fit (16 B): the site-updates
+        # (from the step counters) and the summed launch times give bytes per
+        # launch over the average launch duration.  The pairs are bound by the
+        # issue of instructions; the fraction of the copy bandwidth says how far
+        # below that bound they keep HBM.
         n_bbk = 3 * INNER
-        strip_s = ms[1] / 1e3 / n_bbk                      # strip time per BBK step
-        n_launch = max(1, int(nl[1]))
-        achieved = BYTES_PER_SU * su_strip / (ms[1] / 1e3) / 1e9
-        traffic = ncu_traffic("strip_step_kernel")
-        extra["roofline"] = {"bound": "hbm", "achieved": round(achieved, 1), "peak": hbm, "unit": "GB/s",
-                             "frac": round(achieved / hbm, 4), "peak_kind": f"{peak_kind} copy bandwidth",
-                             "kernel": "strip_step_kernel",
+        strip_ms = ms[1] + ms[6]
+        strip_s = strip_ms / 1e3 / n_bbk                   # strip and band time per BBK step
+        n_launch = max(1, int(nl[1] + nl[6]))
+        n_steps = max(1, int(nl[1] + 2 * nl[6]))           # steps those launches took, all shapes
+        bytes_su = BYTES_PER_SU * (nl[1] + nl[6]) / n_steps
+        achieved = bytes_su * su_strip / (strip_ms / 1e3) / 1e9
+        traffic = ncu_traffic("band_step_kernel")
+        extra["roofline"] = {"bound": "issue" if nl[6] > nl[1] else "hbm", "achieved": round(achieved, 1), "peak": hbm,
+                             "unit": "GB/s", "frac": round(achieved / hbm, 4),
+                             "peak_kind": f"{peak_kind} copy bandwidth",
+                             "kernel": "band_step_kernel" if nl[6] > nl[1] else "strip_step_kernel",
+                             "bytes_per_site_update": round(float(bytes_su), 3),
+                             "site_updates_per_s": su_strip / (strip_ms / 1e3),
+                             "one_step_frac": round(BYTES_PER_SU * su_strip / (strip_ms / 1e3) / 1e9 / hbm, 4),
                              "traffic": (round(traffic * su_strip / n_launch) if traffic else None),
-                             "algorithmic_bytes_per_launch": int(BYTES_PER_SU * su_strip / n_launch),
-                             "launch_ms": round(ms[1] / n_launch, 4),
-                             "launches_per_bbk_step": max(1, round(nl[1] / n_bbk))}
+                             "algorithmic_bytes_per_launch": int(bytes_su * su_strip / n_launch),
+                             "launch_ms": round(strip_ms / n_launch, 4),
+                             "launches_per_bbk_step": round(n_launch / n_bbk, 2)}
         # The event-timed launches run one after another on the library's
         # stream; in the captured graphs of the timed region the lattice
         # shapes' slices run concurrently, so a whole BBK step there takes less
         # than the serial launches add up to.  Both are reported: frac is the
-        # kernel's own (serial launches), step_frac the whole step's at 16 B/su.
+        # kernel's own (serial launches) at the bytes it moves, one_step_frac the
+        # same and step_frac the whole step's at the 16 B/su of one step per pass.
         graph_ms_bbk = elapsed / (args.steps * INNER) * 1e3
-        extra["roofline"]["serial_ms_per_bbk_step"] = round((ms[0] + ms[1]) / n_bbk, 4)
+        extra["roofline"]["serial_ms_per_bbk_step"] = round((ms[0] + strip_ms) / n_bbk, 4)
         extra["roofline"]["graph_ms_per_bbk_step"] = round(graph_ms_bbk, 4)
         extra["roofline"]["step_frac"] = round(value / world * BYTES_PER_SU / 1e9 / hbm, 4)
         extra["roofline"]["gap"] = ("serial_ms_per_bbk_step exceeds graph_ms_per_bbk_step because the graphs run the "

@@ -365,7 +365,7 @@ int xy_synchronize(xy_lattice* lat);
 int64_t xy_kernel_launches(xy_lattice* lat);
 
 #define XY_KCLASS_RESIDENT 0  /* resident stepper launches */
-#define XY_KCLASS_STRIP 1     /* strip stepper launches */
+#define XY_KCLASS_STRIP 1     /* one-step launches of the strip and band steppers */
 #define XY_KCLASS_PLAIN 2     /* plain stepper launches */
 #define XY_KCLASS_ADJ_FWD 3   /* adjoint: forward pass with checkpoints and records (one span per call) */
 #define XY_KCLASS_ADJ_RECOMP 4 /* adjoint: recompute of the checkpoint segments (one span per call) */

@@ -3,7 +3,7 @@
 // with the per-step order-parameter and energy reductions (Sec. IV.A,
 // Eq. lattice-average; App. B, Eq. ensemble-average-calculation).
 //
-// Three steppers share the per-site arithmetic of xy_device.cuh and give
+// Four steppers share the per-site arithmetic of xy_device.cuh and give
 // bit-identical states:
 //   plain    one thread per quad (4 sites), neighbours from global memory/L2,
 //            one launch per step per configuration (the reference path);
@@ -11,7 +11,11 @@
 //            Lx <= 128) sweeping down H rows with a sliding window of
 //            (sin q t, cos q t) rows in registers; x neighbours by warp
 //            shuffles, one force and one Philox call per quad per step;
-//            all lattices of all configurations in one launch;
+//            all lattices of all configurations in one launch; single steps of
+//            lattices whose width fills whole warps;
+//   band     a block per band of rows across the whole width (any width up to
+//            2048), two steps per launch with the intermediate one in registers,
+//            and the steps that record;
 //   resident one thread block, or a thread-block cluster of up to 16
 //            blocks sharing rows through distributed shared memory, per
 //            whole lattice held in shared memory, stepping many steps per
