@@ -254,8 +254,9 @@ int xy_set_coupling_schedule(xy_lattice* lat, int cfg, const int64_t* step_knots
  * intermediate step in registers, so the state crosses HBM once per two steps
  * (8 bytes per site-update instead of 16); the two bands' boundary rows of the
  * intermediate step are computed twice.  States are bit-identical either way,
- * and so are records: a step that records is the first step of its launch.  A
- * run that ends between the two steps of a launch takes the first one only.
+ * and so are records: a launch sums those of either of its steps with the same
+ * roundings as a launch of one.  A run that ends between the two steps of a launch
+ * takes the first one only.
  *   kt = 0 (default): the autotuner times one and two steps per launch (and
  *          the band height) per lattice shape and keeps the faster; small
  *          batches, which it does not time, take two;

@@ -552,8 +552,8 @@ std::vector<uint8_t> group_flags(const xy_lattice* L)
 }
 
 // The launches of a strip group over `cnt` local steps: pairs of steps where the
-// group pairs them and the second one does not record (a launch sums records of
-// its first step), single steps elsewhere.
+// group pairs them (a launch sums the records of either step, with the same
+// roundings as a single one), a single step at the end of an odd count.
 struct StepRun {
     int off, n, rec;
 };
@@ -562,8 +562,8 @@ std::vector<StepRun> step_plan(const xy_lattice* L, const StripGroup& g, int cnt
     std::vector<StepRun> out;
     auto rec_at = [&](int i) { return L->cur_rec && ((L->cur_mask >> (i & 63)) & 1u) ? L->cur_rec : 0; };
     for (int i = 0; i < cnt;) {
-        const int n = g.kt2 && g.band_H > 0 && i + 1 < cnt && !rec_at(i + 1) ? 2 : 1;
-        out.push_back(StepRun{i, n, rec_at(i)});
+        const int n = g.kt2 && g.band_H > 0 && i + 1 < cnt ? 2 : 1;
+        out.push_back(StepRun{i, n, std::max(rec_at(i), n == 2 ? rec_at(i + 1) : 0)});
         i += n;
     }
     return out;
@@ -584,9 +584,7 @@ cudaError_t launch_group(xy_lattice* L, cudaStream_t st, StripGroup& g, int64_t 
                          int64_t jl0, int rd_b, Buffers buf, bool after)
 {
     ++L->launches;
-    // (when every step records nothing pairs: the strip kernel has no halo rows)
-    const bool strip = g.strip_ok && (!r.rec || L->cur_re == 1);
-    if (g.band_H > 0 && (r.n == 2 || !strip)) {
+    if (g.band_H > 0 && (r.n == 2 || r.rec || !g.strip_ok)) {
         const int64_t per = (int64_t)g.band_tasks.size() / g.n_lat;
         return launch_band_step(L->d_cfg, g.d_band_tasks + lat0 * per, (int)(n_lat * per), g.Lx, g.band_H, r.rec,
                                 group_sched(L, g), r.n, rd_b != 0, g.seed, jl0 + r.off, buf, L->d_call, L->pa, after, st);
@@ -1544,12 +1542,13 @@ int xy_lattice_create(const xy_config_desc* cfg, int n_cfg, float* theta, float*
     }
     int rc = classify(L);
     if (rc) return bail(rc);
-    if ((e = cudaMalloc(&L->pa.part, sizeof(double2) * B * L->pa.max_units)) != cudaSuccess ||
-        (e = cudaMalloc(&L->pa.count, sizeof(unsigned) * B)) != cudaSuccess) {
+    L->pa.n_lat = B;
+    if ((e = cudaMalloc(&L->pa.part, sizeof(double2) * 2 * B * L->pa.max_units)) != cudaSuccess ||
+        (e = cudaMalloc(&L->pa.count, sizeof(unsigned) * 2 * B)) != cudaSuccess) {
         cudaGetLastError();
         return bail(fail(XY_ENOMEM, "allocation failed: %s", cudaGetErrorString(e)));
     }
-    if ((e = cudaMemsetAsync(L->pa.count, 0, sizeof(unsigned) * B, L->stream)) != cudaSuccess ||
+    if ((e = cudaMemsetAsync(L->pa.count, 0, sizeof(unsigned) * 2 * B, L->stream)) != cudaSuccess ||
         (e = cudaMemsetAsync(L->d_moments, 0, sizeof(double) * 6 * n_cfg, L->stream)) != cudaSuccess ||
         (e = cudaMemsetAsync(L->d_err, 0, sizeof(int), L->stream)) != cudaSuccess)
         return bail(fail(XY_ECUDA, "memset: %s", cudaGetErrorString(e)));

@@ -122,10 +122,12 @@ struct Buffers {
 };
 
 // Observable partial sums of one lattice assembled by "last unit" reduction.
+// A launch that records both of its steps uses a second set for the second one.
 struct Partials {
-    double2* part;       // [B][max_units]
-    unsigned* count;     // [B]
+    double2* part;       // [2][B][max_units]
+    unsigned* count;     // [2][B]
     int32_t max_units;
+    int64_t n_lat;       // B
 };
 
 // Launch of a kernel that calls dependency_wait(): after = true lets it start while

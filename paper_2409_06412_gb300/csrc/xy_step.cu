@@ -605,18 +605,18 @@ cudaError_t launch_strip_step(const DevCfg* d_cfg, const StripTask* tasks, int n
     const PhiloxKeys keys = philox_round_keys(seed);
     using Kern = void (*)(const DevCfg*, const StripTask*, int, int, int64_t, Buffers, const CallArgs*, Partials,
                           PhiloxKeys);
-    // Launches that record run at most 3 blocks per SM: capped at 64
-    // registers the recording code spills inside the row loop.
+    // Launches that record run two blocks per SM: capped at 80 or 64 registers the
+    // recording code spills inside the row loop.
     static const Kern table[2][3][3] = {
         {
             {strip_step_kernel<2, 0, false>, strip_step_kernel<2, 1, false>, strip_step_kernel<2, 2, false>},
-            {strip_step_kernel<3, 0, false>, strip_step_kernel<3, 1, false>, strip_step_kernel<3, 2, false>},
-            {strip_step_kernel<4, 0, false>, strip_step_kernel<3, 1, false>, strip_step_kernel<3, 2, false>},
+            {strip_step_kernel<3, 0, false>, strip_step_kernel<2, 1, false>, strip_step_kernel<2, 2, false>},
+            {strip_step_kernel<4, 0, false>, strip_step_kernel<2, 1, false>, strip_step_kernel<2, 2, false>},
         },
         {
             {strip_step_kernel<2, 0, true>, strip_step_kernel<2, 1, true>, strip_step_kernel<2, 2, true>},
-            {strip_step_kernel<3, 0, true>, strip_step_kernel<3, 1, true>, strip_step_kernel<3, 2, true>},
-            {strip_step_kernel<4, 0, true>, strip_step_kernel<3, 1, true>, strip_step_kernel<3, 2, true>},
+            {strip_step_kernel<3, 0, true>, strip_step_kernel<2, 1, true>, strip_step_kernel<2, 2, true>},
+            {strip_step_kernel<4, 0, true>, strip_step_kernel<2, 1, true>, strip_step_kernel<2, 2, true>},
         },
     };
     const int vi = variant >= 4 ? 2 : (variant == 3 ? 1 : 0);
@@ -704,8 +704,8 @@ struct R1 {  // a level-1 row: theta_{k+1}, v_{k+1} and (sin q t, cos q t)
 
 }  // namespace
 
-// REC: 0 = the launch records nothing, 1 = M, 2 = M and E of step k (summed over
-// the band's own rows of level 1); SCHED: some configuration of the launch has a
+// REC: 0 = the launch records nothing, 1 = M, 2 = M and E, of step k (summed over
+// the band's own rows of level 1), of step k + 1 (level 2) or of both; SCHED: some configuration of the launch has a
 // field or coupling schedule.  n_steps: 1 or 2.  rd_b: the state is in buffers B.
 // Threads are capped so that every block size keeps 16 warps per SM (128
 // registers).
@@ -840,11 +840,34 @@ __global__ void __launch_bounds__(512, 1) band_step_kernel(const DevCfg* cfgs, c
         else if (!mbar_wait(&s_bar, (uint32_t)(phase & 1)) && lane == 0) atomicExch(cap->err, XY_ETIMEOUT);
     };
     const int own2 = two ? own : 0;  // rows of level 2 that this lane writes
-    float pm = 0.f, pe = 0.f;
-    const float2 Jk = SCHED ? couplings_at(cf, k) : make_float2(cf.Jx, cf.Jy);
-    const float hk = SCHED ? field_h(cf, k) : cf.h;
+    // records: which of the two steps, their couplings and field, and the sums
+    const int re = REC > 0 ? cap->record_every : 0;
+    const bool rec1 = REC > 0 && re > 0 && k % re == 0;
+    const bool rec2 = REC > 0 && re > 0 && two && (k + 1) % re == 0;
+    float pm1 = 0.f, pe1 = 0.f, pm2 = 0.f, pe2 = 0.f;
+    const float2 J1 = SCHED ? couplings_at(cf, k) : make_float2(cf.Jx, cf.Jy);
+    const float h1 = SCHED ? field_h(cf, k) : cf.h;
+    const float2 J2 = SCHED ? couplings_at(cf, k + 1) : J1;
+    const float h2 = SCHED ? field_h(cf, k + 1) : h1;
     const float e_ref = cf.e_ref;
     const bool stag = cf.stag != 0;
+    // a row's terms of M and E: (s, c) of the quad and of the quad below, the ends of
+    // the quad to the right, omega and the angles; y: row of the lattice
+    auto observe = [&](float& pm, float& pe, float2 J, float h, int y, const P4& s, const P4& c, const P4& Ns, const P4& Nc,
+                       float sR, float cR, const P4& om, const P4& th) {
+        const float ev = __fadd_rn(s.a.x, s.b.x), od = __fadd_rn(s.a.y, s.b.y);
+        pm = __fadd_rn(pm, !stag ? __fadd_rn(ev, od) : ((y & 1) ? __fadd_rn(od, -ev) : __fadd_rn(ev, -od)));
+        if (REC == 2) {
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const float sq = p4get(s, q), cq = p4get(c, q);
+                const float sr = q == 3 ? sR : p4get(s, q + 1), cr = q == 3 ? cR : p4get(c, q + 1);
+                const float bx = fmaf(cq, cr, __fmul_rn(sq, sr));
+                const float by = fmaf(cq, p4get(Nc, q), __fmul_rn(sq, p4get(Ns, q)));
+                pe = __fadd_rn(pe, site_energy_rel(p4get(om, q), bx, by, cosp_of(K1.p, p4get(th, q)), J.x, J.y, h, e_ref));
+            }
+        }
+    };
     R0 r0[3];
     R1 r1[3];
     // iteration i: P0, C0, N0 = level-0 rows y - 2, y - 1, y; P1, C1, N1 =
@@ -871,22 +894,8 @@ __global__ void __launch_bounds__(512, 1) band_step_kernel(const DevCfg* cfgs, c
             N1.th = o.theta;
             N1.v = o.v;
             const int ra = i - 3;  // row of the band
-            if (REC > 0 && ra >= 0 && ra < own) {
-                const int odd = stag ? (x + y0 + ra) & 1 : 0;
-                const float ev = __fadd_rn(C0.s.a.x, C0.s.b.x), od = __fadd_rn(C0.s.a.y, C0.s.b.y);
-                pm = __fadd_rn(pm, !stag ? __fadd_rn(ev, od) : (odd ? __fadd_rn(od, -ev) : __fadd_rn(ev, -od)));
-                if (REC == 2) {
-#pragma unroll
-                    for (int q = 0; q < 4; ++q) {
-                        const float s = p4get(C0.s, q), c = p4get(C0.c, q);
-                        const float sr = q == 3 ? sR : p4get(C0.s, q + 1), cr = q == 3 ? cR : p4get(C0.c, q + 1);
-                        const float bx = fmaf(c, cr, __fmul_rn(s, sr));
-                        const float by = fmaf(c, p4get(N0.c, q), __fmul_rn(s, p4get(N0.s, q)));
-                        pe = __fadd_rn(pe, site_energy_rel(p4get(o.omega, q), bx, by, cosp_of(K1.p, p4get(C0.th, q)),
-                                                           Jk.x, Jk.y, hk, e_ref));
-                    }
-                }
-            }
+            if (REC > 0 && rec1 && ra >= 0 && ra < own)
+                observe(pm1, pe1, J1, h1, y0 + ra, C0.s, C0.c, N0.s, N0.c, sR, cR, o.omega, C0.th);
             quad_sc(K1.q, N1.th, N1.s, N1.c);
             publish(N1.s, N1.c, slot, 1);
             edges_published();
@@ -901,6 +910,8 @@ __global__ void __launch_bounds__(512, 1) band_step_kernel(const DevCfg* cfgs, c
             float sL, cL, sR, cR;
             x_nbrs(prev, 1, sL, cL, sR, cR);
             const QuadOut o = quad_update(K2, C1.th, C1.v, cn2, C1.s, C1.c, sL, cL, sR, cR, P1.s, P1.c, N1.s, N1.c);
+            if (REC > 0 && rec2 && i - 4 < own2)
+                observe(pm2, pe2, J2, h2, y0 + i - 4, C1.s, C1.c, N1.s, N1.c, sR, cR, o.omega, C1.th);
             if (i - 4 < own2) {
                 st4_stream(thD + o_b, f4(o.theta));
                 st4_stream(omD + o_b, f4(o.v));
@@ -923,24 +934,31 @@ __global__ void __launch_bounds__(512, 1) band_step_kernel(const DevCfg* cfgs, c
     cp_async_wait<0>();
     launch_next();
     if (REC > 0) {
-        // one partial per block: warp sums, then the block's warps in order
-        __shared__ double2 s_part[kBandWarps];
-        const double wm = warp_sumf(pm), we = warp_sumf(pe);
-        if (lane == 0) s_part[warp] = make_double2(wm, we);
+        // one partial per block and step: warp sums, then the block's warps in order;
+        // warp 0 commits step k, warp 1 (a narrow block has four, a wide one two at
+        // least) step k + 1, which has partials and a counter of its own
+        __shared__ double2 s_part[2][kBandWarps];
+        if (rec1) {
+            const double wm = warp_sumf(pm1), we = warp_sumf(pe1);
+            if (lane == 0) s_part[0][warp] = make_double2(wm, we);
+        }
+        if (rec2) {
+            const double wm = warp_sumf(pm2), we = warp_sumf(pe2);
+            if (lane == 0) s_part[1][warp] = make_double2(wm, we);
+        }
         __syncthreads();
-        if (warp == 0) {
+        if (warp < 2 && (warp == 0 ? rec1 : rec2)) {
             double bm = 0.0, be = 0.0;
             for (int w = 0; w < nw; ++w) {
-                bm += s_part[w].x;
-                be += s_part[w].y;
+                bm += s_part[warp][w].x;
+                be += s_part[warp][w].y;
             }
             const CallArgs ca = *cap;
-            if (ca.record_every <= 0 || k % ca.record_every != 0) return;  // uniform
             const int per_block = WIDE ? 1 : nw * (32 / Q);
             const int64_t b = cf.b_first + task.rep;
-            const int64_t r = (k - cf.rec_first) / ca.record_every;
-            commit_partial(pa, b, task.band0 / per_block, (task.n_bands + per_block - 1) / per_block, bm, be,
-                           ca.rec_dev + b * ca.rec_stride + r, cf.N, REC == 2 ? (double)cf.e_ref : 0.0);
+            const int64_t r = (k + warp - cf.rec_first) / ca.record_every;
+            commit_partial(pa, b + warp * pa.n_lat, task.band0 / per_block, (task.n_bands + per_block - 1) / per_block, bm,
+                           be, ca.rec_dev + b * ca.rec_stride + r, cf.N, REC == 2 ? (double)cf.e_ref : 0.0);
         }
     }
 }
