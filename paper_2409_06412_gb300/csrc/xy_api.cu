@@ -1375,7 +1375,6 @@ int classify(xy_lattice* L)
             h.H = H;
             if (H > 0)
                 max_units = std::max(max_units, strip_units_per_lattice(Lx, Ly, std::min(H, min_strip_H(Lx, Ly))));
-            if (band_shape(Lx, Ly)) max_units = std::max(max_units, band_blocks(Lx, Ly, 1));
         } else {
             h.kind = 2;
         }
@@ -1417,9 +1416,14 @@ int classify(xy_lattice* L)
     }
     // (the task tables of the strip groups are built at the first batched step:
     // the tuner, which runs there, chooses their heights)
-    for (auto& g : L->strip_groups)
-        if (band_shape(g.Lx, g.Ly))
-            g.band_H = default_band_H(g.Lx, g.Ly, g.n_lat, (int64_t)sms * 14 / (int64_t)L->strip_groups.size());
+    for (auto& g : L->strip_groups) {
+        if (!band_shape(g.Lx, g.Ly)) continue;
+        g.band_H = default_band_H(g.Lx, g.Ly, g.n_lat, (int64_t)sms * 14 / (int64_t)L->strip_groups.size());
+        // record partials: one per block of bands, at the default height or at the
+        // tuner's lowest
+        L->pa.max_units = std::max({L->pa.max_units, band_blocks(g.Lx, g.Ly, g.band_H),
+                                    band_blocks(g.Lx, g.Ly, even_band(g.Ly, 4))});
+    }
     apply_kt_mode(L);
     return XY_OK;
 }
