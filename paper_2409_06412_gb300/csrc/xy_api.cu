@@ -273,6 +273,7 @@ struct xy_lattice {
         int64_t kernels;
     };
     std::vector<Graph> graphs;  // captured chunks, by chunk length and recording
+    std::vector<Graph> seen;    // kinds of chunk met once and launched directly (no exec)
     int cur_rec = 0;            // records of the current window: 0 none, 1 M, 2 M and E
     int cur_re = 0;             // its record_every
     uint64_t cur_mask = 0;      // local steps of a chunk at which some strip-stepped lattice records
@@ -832,6 +833,7 @@ cudaError_t launch_branch(xy_lattice* L, cudaStream_t st, const Branch& br, int6
 }
 
 constexpr size_t kMaxGraphs = 64;
+constexpr size_t kFreeGraphs = 8;
 
 void drop_graphs(xy_lattice* L)
 {
@@ -844,14 +846,29 @@ void drop_graphs(xy_lattice* L)
 // branches (chunk_branches) and joins before the chunk counter advances, so
 // their kernels overlap (one branch's launches fill the SMs another's leave
 // idle as its launch drains) instead of taking turns every step.
-int get_graph(xy_lattice* L, int chunk, xy_lattice::Graph** out)
+// once: this kind of chunk may not come again (the rest of a call whose length
+// varies): past the first few kinds it is captured from its second time on, and
+// *out is null before.
+int get_graph(xy_lattice* L, int chunk, bool once, xy_lattice::Graph** out)
 {
+    *out = nullptr;
     const std::vector<uint8_t> gf = group_flags(L);
     for (auto& g : L->graphs)
         if (g.chunk == chunk && g.rec == L->cur_rec && g.rec_mask == L->cur_mask && g.groups == gf) {
             *out = &g;
             return XY_OK;
         }
+    if (once && L->graphs.size() >= kFreeGraphs) {
+        const xy_lattice::Graph kind{chunk, L->cur_rec, L->cur_mask, gf, nullptr, 0};
+        bool seen = false;
+        for (const auto& k : L->seen)
+            seen = seen || (k.chunk == chunk && k.rec == kind.rec && k.rec_mask == kind.rec_mask && k.groups == gf);
+        if (!seen) {
+            if (L->seen.size() >= 4 * kMaxGraphs) L->seen.clear();
+            L->seen.push_back(kind);
+            return XY_OK;
+        }
+    }
     if (L->graphs.size() >= kMaxGraphs) {  // uneven record steps make many kinds of chunk: start afresh
         CK(cudaStreamSynchronize(L->stream));
         drop_graphs(L);
@@ -1171,9 +1188,10 @@ int run_window(xy_lattice* L, int64_t n_max)
             }
         return XY_OK;
     }
-    // A chunk of steps is captured once as a graph and replayed; steps between
-    // two records that the chunks do not fill evenly are cut into equal chunks,
-    // so that a window takes few kinds of them.
+    // Chunks of steps are captured as graphs and replayed: whole ones at once, and
+    // so is what is left of a call or between two records for the first few kinds of
+    // it (a program that repeats its calls has few), later kinds from their second
+    // time on, so that calls of ever new lengths do not capture a graph each.
     for (auto& g : L->strip_groups) g.buf = 0;
     L->in_b.assign((size_t)L->n_cfg, 0);
     if (L->strip_groups.empty() && L->plain_cfgs.empty() && !L->res_groups.empty()) {
@@ -1218,17 +1236,18 @@ int run_window(xy_lattice* L, int64_t n_max)
         if (re > 0 && re <= kChunk) {
             cnt = std::min<int64_t>(kChunk / re * re, n_max - pos);
         } else {
-            const int64_t span = next_record(pos + 1) - pos;  // up to the next record
-            const int64_t parts = (span + kChunk - 1) / kChunk;
-            cnt = std::min(span, ((span + parts - 1) / parts + 1) / 2 * 2);
+            cnt = std::min<int64_t>(kChunk, next_record(pos + 1) - pos);  // up to the next record
         }
         uint64_t mask = 0;
         for (int64_t r = re > 0 ? next_record(pos) : n_max; r < pos + cnt; r = next_record(r + 1)) mask |= 1ull << (r - pos);
         L->cur_mask = mask;
+        const bool whole = cnt == (re > 0 && re <= kChunk ? kChunk / re * re : kChunk);
+        xy_lattice::Graph* g = nullptr;
         if (cnt >= 2 && !L->timing) {
-            xy_lattice::Graph* g = nullptr;
-            int rc = get_graph(L, (int)cnt, &g);
+            int rc = get_graph(L, (int)cnt, !whole, &g);
             if (rc) return rc;
+        }
+        if (g) {
             CK(cudaGraphLaunch(g->exec, L->stream));
             L->launches += g->kernels;
         } else {
