@@ -412,6 +412,10 @@ __device__ __forceinline__ void cp_async_wait()
 // that launch has completed and its writes are visible; what comes before it may
 // read only what no launch of the same chunk of steps writes.  launch_next() lets
 // the following launch start once every block has called it or ended.
+// Every block of such a kernel calls dependency_wait(), also one that has nothing to
+// do: what comes after a chain of launches waits for its last launch only, and that
+// one completes after the others because each of its blocks has waited for the one
+// before.  (A launch whose blocks all left without waiting could complete first.)
 __device__ __forceinline__ void dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void launch_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 

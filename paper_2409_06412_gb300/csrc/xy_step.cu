@@ -721,7 +721,10 @@ __global__ void __launch_bounds__(512, 1) band_step_kernel(const DevCfg* cfgs, c
     const BandTask task = tasks[blockIdx.x];
     const DevCfg& cf = cfgs[task.cfg];
     const int64_t j = cap->j_base + j_local;
-    if (j >= cf.n_call) return;
+    if (j >= cf.n_call) {  // the run has ended (for all warps of the block)
+        dependency_wait();  // a launch of such blocks alone must not complete before the one it follows
+        return;
+    }
     const bool two = n_steps == 2 && j + 1 < cf.n_call;
     if (APART) {
         if (threadIdx.x == 0) mbar_init(&s_bar, nw);
