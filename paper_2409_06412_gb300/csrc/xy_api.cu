@@ -301,6 +301,7 @@ struct xy_lattice {
     };
     enum { kAdjCk, kAdjSbuf, kAdjSeg, kAdjB, kAdjFb, kAdjRec, kAdjGacc, kAdjMpart, kAdjTasks, kSfLats, kSfPart, kSlots };
     DevSlot slot[kSlots];
+    std::vector<SfLattice> h_sf;  // host side of kSfLats
 };
 
 namespace {
@@ -328,6 +329,11 @@ cudaError_t reserve_slot(xy_lattice* L, int i, size_t bytes, void** out)
     return cudaSuccess;
 }
 
+// Tables go to the device by copies on the object's stream, in order with what reads
+// them there or on streams forked from it: a plain copy from pageable memory may return
+// before the data has landed, and orders no non-blocking stream.  The host side of a
+// table stays as it is until its copy has been made (on the object, or to the end of a
+// call that waits for the stream).
 int upload_cfg(xy_lattice* L)
 {
     CK(cudaMemcpyAsync(L->d_cfg, L->h_dev.data(), sizeof(DevCfg) * L->n_cfg, cudaMemcpyHostToDevice, L->stream));
@@ -1333,7 +1339,8 @@ int build_strip_tasks(xy_lattice* L, StripGroup& g)
         CK(cudaMalloc(&g.d_tasks, sizeof(StripTask) * g.tasks.size()));
         g.d_cap = g.tasks.size();
     }
-    CK(cudaMemcpy(g.d_tasks, g.tasks.data(), sizeof(StripTask) * g.tasks.size(), cudaMemcpyHostToDevice));
+    CK(cudaMemcpyAsync(g.d_tasks, g.tasks.data(), sizeof(StripTask) * g.tasks.size(), cudaMemcpyHostToDevice,
+                       L->stream));
     drop_graphs(L);
     return XY_OK;
 }
@@ -1355,7 +1362,8 @@ int build_band_tasks(xy_lattice* L, StripGroup& g, int H)
         CK(cudaMalloc(&g.d_band_tasks, sizeof(BandTask) * g.band_tasks.size()));
         g.d_band_cap = g.band_tasks.size();
     }
-    CK(cudaMemcpy(g.d_band_tasks, g.band_tasks.data(), sizeof(BandTask) * g.band_tasks.size(), cudaMemcpyHostToDevice));
+    CK(cudaMemcpyAsync(g.d_band_tasks, g.band_tasks.data(), sizeof(BandTask) * g.band_tasks.size(),
+                       cudaMemcpyHostToDevice, L->stream));
     drop_graphs(L);
     return XY_OK;
 }
@@ -1430,7 +1438,8 @@ int classify(xy_lattice* L)
     }
     for (auto& g : L->res_groups) {
         CK(cudaMalloc(&g.d_tasks, sizeof(ResidentTask) * g.tasks.size()));
-        CK(cudaMemcpy(g.d_tasks, g.tasks.data(), sizeof(ResidentTask) * g.tasks.size(), cudaMemcpyHostToDevice));
+        CK(cudaMemcpyAsync(g.d_tasks, g.tasks.data(), sizeof(ResidentTask) * g.tasks.size(), cudaMemcpyHostToDevice,
+                           L->stream));
         CK(prepare_resident(g.Lx, g.Ly, g.threads, g.csize, nullptr));
     }
     // (the task tables of the strip groups are built at the first batched step:
@@ -1951,12 +1960,14 @@ int xy_structure_factor(xy_lattice* L, int b_first, int b_count, int K, double r
     // demand; cudaFree waits for the device, so no launch still uses the old block)
     void *lats = nullptr, *scratch = nullptr;
     if (!L->slot[xy_lattice::kSfLats].p) {
-        std::vector<SfLattice> h;
+        std::vector<SfLattice>& h = L->h_sf;
+        h.clear();
         h.reserve((size_t)L->B);
         for (const DevCfg& d : L->h_dev)
             for (int r = 0; r < d.n_rep; ++r) h.push_back(SfLattice{d.offset + r * d.N, d.Lx, d.Ly});
         cudaError_t e0 = reserve_slot(L, xy_lattice::kSfLats, sizeof(SfLattice) * h.size(), &lats);
-        if (e0 == cudaSuccess) e0 = cudaMemcpy(lats, h.data(), sizeof(SfLattice) * h.size(), cudaMemcpyHostToDevice);
+        if (e0 == cudaSuccess)
+            e0 = cudaMemcpyAsync(lats, h.data(), sizeof(SfLattice) * h.size(), cudaMemcpyHostToDevice, L->stream);
         if (e0 != cudaSuccess) {
             cudaGetLastError();
             cudaFree(L->slot[xy_lattice::kSfLats].p);
@@ -2222,7 +2233,8 @@ int xy_adjoint_step_n(xy_lattice* L, int64_t n, int K, double wE, double wM, dou
                     if (e != cudaSuccess) break;
                     band_tasks(g, h, tk);
                     cuts = cut_tasks(tk, n_parts);
-                    e = cudaMemcpy(d_tk, tk.data(), sizeof(BandTask) * tk.size(), cudaMemcpyHostToDevice);
+                    e = cudaMemcpyAsync(d_tk, tk.data(), sizeof(BandTask) * tk.size(), cudaMemcpyHostToDevice,
+                                        L->stream);
                     int reps = 2;
                     float t_best = 1e30f;
                     for (int round = 0; round < 5 && e == cudaSuccess; ++round) {
@@ -2274,7 +2286,8 @@ int xy_adjoint_step_n(xy_lattice* L, int64_t n, int K, double wE, double wM, dou
         for (auto& g : adj_groups) {
             if (e != cudaSuccess) break;
             g.d_tasks = tasks;
-            e = cudaMemcpy(g.d_tasks, g.tasks.data(), sizeof(BandTask) * g.tasks.size(), cudaMemcpyHostToDevice);
+            e = cudaMemcpyAsync(g.d_tasks, g.tasks.data(), sizeof(BandTask) * g.tasks.size(), cudaMemcpyHostToDevice,
+                                L->stream);
             tasks += g.tasks.size();
         }
     }
