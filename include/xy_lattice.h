@@ -136,7 +136,9 @@ int xy_step_n(xy_lattice* lat, int64_t n, int record_every, double* rec, int64_t
  * moments[c][0..5] = sums over replicas and recorded steps >= t0 of
  * (1, M^2, M^4, E, E^2, |M|); the paper's Binder ratio (Eq. Def-Binder-Cum) is
  * U = (m[2]/m[0]) / (m[1]/m[0])^2.  step_now[c] (nullable) = current step.
- * Returns XY_ENAN if any moment is not finite. */
+ * Returns XY_ENAN if any moment is not finite, XY_ETIMEOUT if a bounded wait of a
+ * stepper launch ran out (the state is then not valid: calls that use it report
+ * this until xy_load replaces it). */
 int xy_observe(xy_lattice* lat, double* moments, int64_t* step_now);
 
 /* Clear the running moments of every configuration. */
@@ -407,6 +409,12 @@ int xy_debug_noise(uint64_t seed, int cfg, int replica, int64_t k, int tag, int6
  * returns XY_ETIMEOUT with incomplete labels (indices stay in range, nothing
  * faults).  For testing the timeout path; the paper has no counterpart. */
 int xy_debug_set_union_limit(int iters);
+
+/* Diagnostics: what a stepper launch does whose bounded wait ran out: `code`
+ * (XY_ETIMEOUT there) is reported by every later call that uses the state, until
+ * xy_load replaces it; 0 takes it back.  For testing that path without a
+ * failing launch; the paper has no counterpart. */
+int xy_debug_set_step_error(xy_lattice* lat, int code);
 
 /* Diagnostics: the Box-Muller map of the steppers (App. A.1 noise) applied to
  * given Philox words: words (device uint32[n_quads][4], 16-byte aligned) ->

@@ -72,6 +72,7 @@ SIGNATURES = {
     "xy_debug_philox": (_i32, [_vp, _u32, _u32, _i64, _vp, _vp]),
     "xy_debug_gauss4": (_i32, [_vp, _i64, ctypes.c_float, _vp, _vp]),
     "xy_debug_set_union_limit": (_i32, [_i32]),
+    "xy_debug_set_step_error": (_i32, [_vp, _i32]),
     "xy_debug_slice_parts": (_i32, [_vp, _i32, _i32, _i32, _vp]),
     "xy_debug_slice_cuts": (_i32, [_vp, _i32, _i32, _vp, _vp]),
 }

@@ -256,7 +256,8 @@ struct xy_lattice {
     double* d_moments = nullptr;
     double2* rec_buf = nullptr;
     size_t rec_cap = 0;
-    int* d_err = nullptr;
+    int* d_err = nullptr;       // of the labelling passes, cleared by every call
+    int* step_err = nullptr;    // of the steppers: pinned host memory that kernels write and the host reads without a copy
     int path = XY_PATH_BATCHED;
     int adj_mode = XY_ADJOINT_AUTO;
     std::vector<ResGroup> res_groups;
@@ -349,7 +350,7 @@ int upload_call(xy_lattice* L, const CallArgs& ca)
         CK(cudaEventCreateWithFlags(&L->call_ev[slot], cudaEventDisableTiming));
     CK(cudaEventSynchronize(L->call_ev[slot]));
     L->h_call[slot] = ca;
-    L->h_call[slot].err = L->d_err;
+    L->h_call[slot].err = L->step_err;
     CK(cudaMemcpyAsync(L->d_call, &L->h_call[slot], sizeof(CallArgs), cudaMemcpyHostToDevice, L->stream));
     CK(cudaEventRecord(L->call_ev[slot], L->stream));
     return XY_OK;
@@ -452,8 +453,19 @@ void fill_power_f32(DevCfg& d, const CfgHost& h)
     d.pw_ef = (float)h.pw[5];
 }
 
+// A bounded wait of a stepper that ran out: the state is not to be used any more.
+// The code stays until xy_load replaces the state; a call that waits for the
+// stream sees every launch before it, others those that have run.
+int step_status(const xy_lattice* L)
+{
+    const int err = *static_cast<const volatile int*>(L->step_err);
+    return err ? fail(err, "a launch of the stepper gave up (code %d): the state is not valid", err) : XY_OK;
+}
+
 int check_ready(xy_lattice* L)
 {
+    const int rc = step_status(L);
+    if (rc) return rc;
     for (int c = 0; c < L->n_cfg; ++c) {
         if (!L->cfg[c].has_prm) return fail(XY_EINVAL, "configuration %d has no parameters (xy_set_params)", c);
         if (!L->cfg[c].has_sched) return fail(XY_EINVAL, "configuration %d has no schedule (xy_set_schedule)", c);
@@ -1565,13 +1577,15 @@ int xy_lattice_create(const xy_config_desc* cfg, int n_cfg, float* theta, float*
     cudaError_t e;
     if ((e = cudaMalloc(&L->d_cfg, sizeof(DevCfg) * n_cfg)) != cudaSuccess ||
         (e = cudaMalloc(&L->d_call, sizeof(CallArgs))) != cudaSuccess ||
-        (e = cudaMallocHost(&L->h_call, sizeof(CallArgs) * xy_lattice::kRing)) != cudaSuccess ||
+        (e = cudaMallocHost(&L->h_call, sizeof(CallArgs) * xy_lattice::kRing + sizeof(int))) != cudaSuccess ||
         (e = cudaMalloc(&L->d_moments, sizeof(double) * 6 * n_cfg)) != cudaSuccess ||
         (e = cudaMalloc(&L->d_err, sizeof(int))) != cudaSuccess ||
         (e = cudaStreamCreateWithFlags(&L->cap_stream, cudaStreamNonBlocking)) != cudaSuccess) {
         cudaGetLastError();
         return bail(fail(XY_ENOMEM, "allocation failed: %s", cudaGetErrorString(e)));
     }
+    L->step_err = reinterpret_cast<int*>(L->h_call + xy_lattice::kRing);
+    *L->step_err = XY_OK;
     int rc = classify(L);
     if (rc) return bail(rc);
     L->pa.n_lat = B;
@@ -1751,6 +1765,7 @@ int xy_step_n(xy_lattice* L, int64_t n, int record_every, double* rec, int64_t t
     if (rec && !dev_rec) {
         CK(cudaMemcpyAsync(rec, rd, sizeof(double2) * L->B * R, cudaMemcpyDeviceToHost, L->stream));
         CK(cudaStreamSynchronize(L->stream));
+        return step_status(L);
     }
     return XY_OK;
 }
@@ -1759,8 +1774,6 @@ int xy_observe(xy_lattice* L, double* moments, int64_t* step_now)
 {
     if (!L) return fail(XY_EINVAL, "NULL lattice");
     CK(cudaStreamSynchronize(L->stream));
-    int err = 0;
-    CK(cudaMemcpy(&err, L->d_err, sizeof(int), cudaMemcpyDeviceToHost));
     if (step_now)
         for (int c = 0; c < L->n_cfg; ++c) step_now[c] = L->cfg[c].step;
     if (moments) {
@@ -1768,8 +1781,7 @@ int xy_observe(xy_lattice* L, double* moments, int64_t* step_now)
         for (int i = 0; i < 6 * L->n_cfg; ++i)
             if (!std::isfinite(moments[i])) return fail(XY_ENAN, "moment %d of configuration %d is not finite", i % 6, i / 6);
     }
-    if (err) return fail(err, "a device-side check failed (code %d)", err);
-    return XY_OK;
+    return step_status(L);
 }
 
 int xy_reset_moments(xy_lattice* L)
@@ -1807,6 +1819,7 @@ int xy_label_domains(xy_lattice* L, int b_first, int b_count, int32_t* labels, i
     if (!L) return fail(XY_EINVAL, "NULL lattice");
     if (b_first < 0 || b_count <= 0 || b_first + (int64_t)b_count > L->B) return fail(XY_EINVAL, "lattice range out of bounds");
     if (hist && hist_cap <= 0) return fail(XY_EINVAL, "hist_cap must be > 0");
+    if (const int bad = step_status(L)) return bad;
     int Lx = -1, Ly = -1;
     int64_t site0 = -1;
     for (int c = 0; c < L->n_cfg; ++c) {
@@ -1900,7 +1913,7 @@ int xy_label_domains(xy_lattice* L, int b_first, int b_count, int32_t* labels, i
     if (err == XY_EINVAL) return fail(XY_EINVAL, "a lattice has more distinct domain sizes than hist_cap");
     if (err == XY_ENOMEM) return fail(XY_ENOMEM, "labelling: the list of pieces on tile edges overflowed");
     if (err) return fail(err, "labelling: a bounded union loop ran out of iterations");
-    return XY_OK;
+    return step_status(L);
 }
 
 int xy_autocorr_time(const double* rec, int64_t n_series, int64_t R, int component, int transform, int64_t skip,
@@ -1946,6 +1959,7 @@ int xy_structure_factor(xy_lattice* L, int b_first, int b_count, int K, double r
         return fail(XY_EINVAL, "lattice range out of bounds");
     if (K < 1) return fail(XY_EINVAL, "K must be >= 1");
     if (!std::isfinite(rotor)) return fail(XY_EINVAL, "rotor multiplicity must be finite");
+    if (const int bad = step_status(L)) return bad;
     int max_x = 0, max_y = 0;
     for (int c = 0; c < L->n_cfg; ++c) {
         const DevCfg& d = L->h_dev[c];
@@ -2008,7 +2022,7 @@ int xy_structure_factor(xy_lattice* L, int b_first, int b_count, int K, double r
         cudaGetLastError();
         return fail(XY_ECUDA, "structure factor: %s", cudaGetErrorString(e));
     }
-    return XY_OK;
+    return dev ? XY_OK : step_status(L);
 }
 
 int xy_adjoint_step_n(xy_lattice* L, int64_t n, int K, double wE, double wM, double* objective, double* grads)
@@ -2580,7 +2594,7 @@ int xy_adjoint_step_n(xy_lattice* L, int64_t n, int K, double wE, double wM, dou
     RCA(upload_cfg(L));
 #undef CKA
 #undef RCA
-    return XY_OK;
+    return step_status(L);
 }
 
 // ---- snapshots
@@ -2665,7 +2679,7 @@ int xy_save(xy_lattice* L, void* buf, size_t* size)
     CK(cudaMemcpyAsync(p, L->omA, sizeof(float) * L->total_sites, cudaMemcpyDeviceToHost, L->stream));
     CK(cudaStreamSynchronize(L->stream));
     *size = need;
-    return XY_OK;
+    return step_status(L);
 }
 
 int xy_load(xy_lattice* L, const void* buf, size_t size)
@@ -2734,6 +2748,7 @@ int xy_load(xy_lattice* L, const void* buf, size_t size)
     p += sizeof(float) * L->total_sites;
     CK(cudaMemcpyAsync(L->omA, p, sizeof(float) * L->total_sites, cudaMemcpyHostToDevice, L->stream));
     CK(cudaStreamSynchronize(L->stream));
+    *static_cast<volatile int*>(L->step_err) = XY_OK;
     set_window_idle(L);
     return upload_cfg(L);
 }
@@ -2742,10 +2757,17 @@ int xy_synchronize(xy_lattice* L)
 {
     if (!L) return fail(XY_EINVAL, "NULL lattice");
     CK(cudaStreamSynchronize(L->stream));
-    return XY_OK;
+    return step_status(L);
 }
 
 int64_t xy_kernel_launches(xy_lattice* L) { return L ? L->launches : -1; }
+
+int xy_debug_set_step_error(xy_lattice* L, int code)
+{
+    if (!L) return fail(XY_EINVAL, "NULL lattice");
+    *static_cast<volatile int*>(L->step_err) = code;
+    return XY_OK;
+}
 
 int xy_set_autotune(xy_lattice* L, int on)
 {

@@ -72,7 +72,7 @@ struct CallArgs {
     int64_t k_shift;    // added to the step index (segment recompute of the adjoint)
     int record_every;   // 0: no observables
     int fixed_parity;   // 1: always read buffers A and write buffers B (plain and resident kernels)
-    int* err;           // device error flag (read by xy_observe)
+    int* err;           // error word of the steppers (pinned host memory)
     int m_only;         // 1: records carry M only (E left 0)
 };
 

@@ -669,8 +669,8 @@ struct BStage {
 };
 // A barrier of the block's warps with arrival and wait apart.  The wait is
 // bounded: every warp arrives once per phase whatever its data, so the bound is
-// reached only if the launch itself is broken; the caller then says so and goes
-// on with what the edge slots hold.
+// reached only if the launch itself is broken; the caller then says so, goes on to
+// the end of the band and stores nothing more.
 __device__ __forceinline__ void mbar_init(uint64_t* bar, int count)
 {
     asm volatile("mbarrier.init.shared.b64 [%0], %1;" ::"r"((unsigned)__cvta_generic_to_shared(bar)), "r"(count) : "memory");
@@ -821,6 +821,7 @@ __global__ void __launch_bounds__(512, 1) band_step_kernel(const DevCfg* cfgs, c
     auto publish = [&](const P4& Cs, const P4& Cc, int slot, int lev) {
         (lev ? stg.e1 : stg.e0)[slot][lane] = make_float4(Cs.a.x, Cc.a.x, Cs.b.y, Cc.b.y);
     };
+    int own2 = two ? own : 0;  // rows of level 2 that this lane writes
     // The ends of iteration i are published in slot i % 3 before its barrier (a
     // narrow band's warp: before its __syncwarp) and read after it, in iteration
     // i + 1.  Blocks of up to 8 warps meet at a block barrier there.  In wider ones
@@ -840,9 +841,11 @@ __global__ void __launch_bounds__(512, 1) band_step_kernel(const DevCfg* cfgs, c
     auto edges_ready = [&](int phase) {
         if (!WIDE) return;
         if (!APART) __syncthreads();
-        else if (!mbar_wait(&s_bar, (uint32_t)(phase & 1)) && lane == 0) atomicExch(cap->err, XY_ETIMEOUT);
+        else if (!mbar_wait(&s_bar, (uint32_t)(phase & 1))) {
+            *static_cast<volatile int*>(cap->err) = XY_ETIMEOUT;
+            own = own2 = 0;  // what this warp computes from here on is not stored
+        }
     };
-    const int own2 = two ? own : 0;  // rows of level 2 that this lane writes
     // records: which of the two steps, their couplings and field, and the sums
     const int re = REC > 0 ? cap->record_every : 0;
     const bool rec1 = REC > 0 && re > 0 && k % re == 0;
