@@ -377,6 +377,19 @@ __device__ __forceinline__ float site_energy_rel(float omega, float bx, float by
     return fmaf(__fmul_rn(0.5f, omega), omega, e);
 }
 
+// The four sites of a quad at once, with the same roundings: (s, c) of the quad, of
+// the quad below (N) and of the site to its right (sR, cR).
+__device__ __forceinline__ P4 quad_energy_rel(float p, float2 J, float h, float e_ref, const P4& s, const P4& c,
+                                              const P4& Ns, const P4& Nc, float sR, float cR, const P4& om, const P4& th)
+{
+    const P4 sr{make_float2(s.a.y, s.b.x), make_float2(s.b.y, sR)}, cr{make_float2(c.a.y, c.b.x), make_float2(c.b.y, cR)};
+    const P4 bx = fma4(c, cr, mul4(s, sr)), by = fma4(c, Nc, mul4(s, Ns));
+    const P4 pt = mul4(p, th);
+    const P4 cp{make_float2(__cosf(pt.a.x), __cosf(pt.a.y)), make_float2(__cosf(pt.b.x), __cosf(pt.b.y))};
+    const P4 ref{splat2(-e_ref), splat2(-e_ref)};
+    return fma4(mul4(0.5f, om), om, fma4(-J.y, by, fma4(-J.x, bx, fma4(h, cp, ref))));
+}
+
 // Jk: the couplings (couplings_at) and hk the field (field_h) of the recorded step
 __device__ __forceinline__ float site_energy(const DevCfg& cf, float2 Jk, float hk, float omega, float s, float c,
                                              float sR, float cR, float sD, float cD, float cosp)

@@ -95,8 +95,8 @@ __device__ __forceinline__ double warp_sum(double v)
     return v;
 }
 
-// FP32 warp sum in the same order.  A warp's partial covers at most a few
-// thousand sites, each term of magnitude O(1), so FP32 keeps it to ~1e-6
+// FP32 warp sum in the same order.  A warp's partial covers at most 8192 sites (64
+// rows of a strip), each term of magnitude O(1), so FP32 keeps it to ~1e-6
 // relative; the partials of different warps and blocks are combined in FP64.
 // (FP64 issues at a small fraction of the FP32 rate on this GPU, so a double
 // butterfly per warp and per step is not free.)
@@ -693,6 +693,54 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity)
     return false;
 }
 
+// Sums of (M, E) terms as pairs of FP32 values, (sum, what its roundings left out):
+// the error-free addition of Knuth (The Art of Computer Programming, vol. 2, Sec.
+// 4.2.2).  A band's lane adds up to 128 rows of four sites and its warp 32 lanes; in
+// single FP32 sums that cost a record up to 1.5e-8 of its size (FP64 additions issue
+// at 1/64 of the rate).  So a record is good to the FP32 sum of each quad's four
+// terms, whatever the height of the bands.
+__device__ __forceinline__ void add_exact(float2& sum, float2& rest, float2 v)
+{
+    const float2 m1 = splat2(-1.0f);
+    const float2 t = __fadd2_rn(sum, v);
+    const float2 vv = __ffma2_rn(m1, sum, t);
+    const float2 sv = __ffma2_rn(m1, vv, t);
+    rest = __fadd2_rn(rest, __fadd2_rn(__ffma2_rn(m1, sv, sum), __ffma2_rn(m1, vv, v)));
+    sum = t;
+}
+__device__ __forceinline__ void add_exact(float& sum, float& rest, float v)
+{
+    const float t = __fadd_rn(sum, v);
+    const float vv = __fadd_rn(t, -sum);
+    const float sv = __fadd_rn(t, -vv);
+    rest = __fadd_rn(rest, __fadd_rn(__fadd_rn(sum, -sv), __fadd_rn(v, -vv)));
+    sum = t;
+}
+// The lanes' sums of (M, E) of two levels over the warp: the halves of the warp take a
+// level each, the quarters M or E of it, so that four lane groups reduce one value
+// each.  Returns M (lanes 0..7) and E (8..15) of level 0, M (16..23) and E (24..31) of
+// level 1.
+__device__ __forceinline__ double warp_sum_pairs(const float2 (&sum)[2], const float2 (&rest)[2], int lane)
+{
+    auto xchg = [](float v, int o) { return __shfl_xor_sync(kFull, v, o); };
+    const bool hi = (lane & 16) != 0, en = (lane & 8) != 0;
+    const float2 give = hi ? sum[0] : sum[1], give_r = hi ? rest[0] : rest[1];
+    float2 s2 = hi ? sum[1] : sum[0];
+    float2 r2 = __fadd2_rn(hi ? rest[1] : rest[0], make_float2(xchg(give_r.x, 16), xchg(give_r.y, 16)));
+    add_exact(s2, r2, make_float2(xchg(give.x, 16), xchg(give.y, 16)));
+    float s = en ? s2.y : s2.x, r = en ? r2.y : r2.x;
+    const float so = xchg(en ? s2.x : s2.y, 8);
+    r = __fadd_rn(r, xchg(en ? r2.x : r2.y, 8));
+    add_exact(s, r, so);
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) {
+        const float sx = xchg(s, o), rx = xchg(r, o);
+        r = __fadd_rn(r, rx);
+        add_exact(s, r, sx);
+    }
+    return (double)s + (isfinite(r) ? (double)r : 0.0);  // (a sum that is not finite has no rest)
+}
+
 struct R0 {  // a level-0 row: theta_k and its (sin q t, cos q t)
     P4 th;
     P4 s, c;
@@ -850,29 +898,29 @@ __global__ void __launch_bounds__(512, 1) band_step_kernel(const DevCfg* cfgs, c
     const int re = REC > 0 ? cap->record_every : 0;
     const bool rec1 = REC > 0 && re > 0 && k % re == 0;
     const bool rec2 = REC > 0 && re > 0 && two && (k + 1) % re == 0;
-    float pm1 = 0.f, pe1 = 0.f, pm2 = 0.f, pe2 = 0.f;
+    float2 sum[2] = {}, rest[2] = {};  // (M, E) of each level
     const float2 J1 = SCHED ? couplings_at(cf, k) : make_float2(cf.Jx, cf.Jy);
     const float h1 = SCHED ? field_h(cf, k) : cf.h;
     const float2 J2 = SCHED ? couplings_at(cf, k + 1) : J1;
     const float h2 = SCHED ? field_h(cf, k + 1) : h1;
     const float e_ref = cf.e_ref;
     const bool stag = cf.stag != 0;
-    // a row's terms of M and E: (s, c) of the quad and of the quad below, the ends of
-    // the quad to the right, omega and the angles; y: row of the lattice
-    auto observe = [&](float& pm, float& pe, float2 J, float h, int y, const P4& s, const P4& c, const P4& Ns, const P4& Nc,
+    using L0 = std::integral_constant<int, 0>;
+    using L1 = std::integral_constant<int, 1>;
+    using L2 = std::integral_constant<int, 2>;
+    // a row's terms of M and E, added to the sums of a level: (s, c) of the quad and of
+    // the quad below, the ends of the quad to the right, omega and the angles; y: row of
+    // the lattice
+    auto observe = [&](auto level, float2 J, float h, int y, const P4& s, const P4& c, const P4& Ns, const P4& Nc,
                        float sR, float cR, const P4& om, const P4& th) {
         const float ev = __fadd_rn(s.a.x, s.b.x), od = __fadd_rn(s.a.y, s.b.y);
-        pm = __fadd_rn(pm, !stag ? __fadd_rn(ev, od) : ((y & 1) ? __fadd_rn(od, -ev) : __fadd_rn(ev, -od)));
+        const float pm = !stag ? __fadd_rn(ev, od) : ((y & 1) ? __fadd_rn(od, -ev) : __fadd_rn(ev, -od));
+        float pe = 0.f;
         if (REC == 2) {
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const float sq = p4get(s, q), cq = p4get(c, q);
-                const float sr = q == 3 ? sR : p4get(s, q + 1), cr = q == 3 ? cR : p4get(c, q + 1);
-                const float bx = fmaf(cq, cr, __fmul_rn(sq, sr));
-                const float by = fmaf(cq, p4get(Nc, q), __fmul_rn(sq, p4get(Ns, q)));
-                pe = __fadd_rn(pe, site_energy_rel(p4get(om, q), bx, by, cosp_of(K1.p, p4get(th, q)), J.x, J.y, h, e_ref));
-            }
+            const P4 e = quad_energy_rel(K1.p, J, h, e_ref, s, c, Ns, Nc, sR, cR, om, th);
+            pe = __fadd_rn(__fadd_rn(__fadd_rn(e.a.x, e.a.y), e.b.x), e.b.y);
         }
+        add_exact(sum[decltype(level)::value], rest[decltype(level)::value], make_float2(pm, pe));
     };
     R0 r0[3];
     R1 r1[3];
@@ -901,7 +949,7 @@ __global__ void __launch_bounds__(512, 1) band_step_kernel(const DevCfg* cfgs, c
             N1.v = o.v;
             const int ra = i - 3;  // row of the band
             if (REC > 0 && rec1 && ra >= 0 && ra < own)
-                observe(pm1, pe1, J1, h1, y0 + ra, C0.s, C0.c, N0.s, N0.c, sR, cR, o.omega, C0.th);
+                observe(L0{}, J1, h1, y0 + ra, C0.s, C0.c, N0.s, N0.c, sR, cR, o.omega, C0.th);
             quad_sc(K1.q, N1.th, N1.s, N1.c);
             publish(N1.s, N1.c, slot, 1);
             edges_published();
@@ -917,7 +965,7 @@ __global__ void __launch_bounds__(512, 1) band_step_kernel(const DevCfg* cfgs, c
             x_nbrs(prev, 1, sL, cL, sR, cR);
             const QuadOut o = quad_update(K2, C1.th, C1.v, cn2, C1.s, C1.c, sL, cL, sR, cR, P1.s, P1.c, N1.s, N1.c);
             if (REC > 0 && rec2 && i - 4 < own2)
-                observe(pm2, pe2, J2, h2, y0 + i - 4, C1.s, C1.c, N1.s, N1.c, sR, cR, o.omega, C1.th);
+                observe(L1{}, J2, h2, y0 + i - 4, C1.s, C1.c, N1.s, N1.c, sR, cR, o.omega, C1.th);
             if (i - 4 < own2) {
                 st4_stream(thD + o_b, f4(o.theta));
                 st4_stream(omD + o_b, f4(o.v));
@@ -925,9 +973,6 @@ __global__ void __launch_bounds__(512, 1) band_step_kernel(const DevCfg* cfgs, c
             o_b += Lx;
         }
     };
-    using L0 = std::integral_constant<int, 0>;
-    using L1 = std::integral_constant<int, 1>;
-    using L2 = std::integral_constant<int, 2>;
     body(L0{}, 0, 0, r0[1], r0[2], r0[0], r1[1], r1[2], r1[0]);
     body(L0{}, 1, 1, r0[2], r0[0], r0[1], r1[2], r1[0], r1[1]);
     body(L1{}, 2, 2, r0[0], r0[1], r0[2], r1[0], r1[1], r1[2]);
@@ -944,14 +989,8 @@ __global__ void __launch_bounds__(512, 1) band_step_kernel(const DevCfg* cfgs, c
         // warp 0 commits step k, warp 1 (a narrow block has four, a wide one two at
         // least) step k + 1, which has partials and a counter of its own
         __shared__ double2 s_part[2][kBandWarps];
-        if (rec1) {
-            const double wm = warp_sumf(pm1), we = warp_sumf(pe1);
-            if (lane == 0) s_part[0][warp] = make_double2(wm, we);
-        }
-        if (rec2) {
-            const double wm = warp_sumf(pm2), we = warp_sumf(pe2);
-            if (lane == 0) s_part[1][warp] = make_double2(wm, we);
-        }
+        const double w = warp_sum_pairs(sum, rest, lane);
+        if ((lane & 7) == 0) (&s_part[lane >> 4][warp].x)[(lane >> 3) & 1] = w;
         __syncthreads();
         if (warp < 2 && (warp == 0 ? rec1 : rec2)) {
             double bm = 0.0, be = 0.0;
