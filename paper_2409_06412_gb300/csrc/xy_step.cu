@@ -636,8 +636,11 @@ cudaError_t launch_strip_step(const DevCfg* d_cfg, const StripTask* tasks, int n
 // only row written back: 8 bytes per site-update instead of 16.  The two extra
 // level-1 rows are recomputed by the neighbouring bands too (2 / H more level-1
 // work).  The per-site arithmetic is that of every other stepper, so states are
-// bit-identical to two single steps.  A launch of one step (or the last step of
-// a configuration whose run ends after it) writes level 1 instead.
+// bit-identical to two single steps.  A configuration whose run ends after the first
+// step of a launch writes level 1 instead.  A launch of one step loads rows y0 - 1
+// .. y0 + H and has no level 2 (STEPS = 1; a
+// launch of two that dropped its second took longer: 8 x 1024^2, 100 single steps with
+// a record each, 4.9 -> 2.9 ms).
 //
 // WIDE (Lx > 128): a block is one band, its ceil(Lx / 128) warps side by side
 // with the row's quads dealt out evenly (any Lx that is a multiple of 4: no warp
@@ -754,13 +757,13 @@ struct R1 {  // a level-1 row: theta_{k+1}, v_{k+1} and (sin q t, cos q t)
 
 // REC: 0 = the launch records nothing, 1 = M, 2 = M and E, of step k (summed over
 // the band's own rows of level 1), of step k + 1 (level 2) or of both; SCHED: some configuration of the launch has a
-// field or coupling schedule.  n_steps: 1 or 2.  rd_b: the state is in buffers B.
+// field or coupling schedule.  STEPS: 1 or 2.  rd_b: the state is in buffers B.
 // Threads are capped so that every block size keeps 16 warps per SM (128
 // registers).
 // APART: a wide band's warps arrive and wait apart.
-template <bool WIDE, bool APART, int REC, bool SCHED>
-__global__ void __launch_bounds__(512, 1) band_step_kernel(const DevCfg* cfgs, const BandTask* tasks, int H, int n_steps,
-                                                           int rd_b, int64_t j_local, Buffers buf, const CallArgs* cap,
+template <int STEPS, bool WIDE, bool APART, int REC, bool SCHED>
+__global__ void __launch_bounds__(512, 1) band_step_kernel(const DevCfg* cfgs, const BandTask* tasks, int H, int rd_b,
+                                                           int64_t j_local, Buffers buf, const CallArgs* cap,
                                                            Partials pa, PhiloxKeys keys)
 {
     extern __shared__ BStage s_bstage[];  // one per warp
@@ -773,7 +776,7 @@ __global__ void __launch_bounds__(512, 1) band_step_kernel(const DevCfg* cfgs, c
         dependency_wait();  // a launch of such blocks alone must not complete before the one it follows
         return;
     }
-    const bool two = n_steps == 2 && j + 1 < cf.n_call;
+    const bool two = STEPS == 2 && j + 1 < cf.n_call;
     if (APART) {
         if (threadIdx.x == 0) mbar_init(&s_bar, nw);
         __syncthreads();
@@ -823,16 +826,16 @@ __global__ void __launch_bounds__(512, 1) band_step_kernel(const DevCfg* cfgs, c
     float* omD = (rd_b ? buf.omA : buf.omB) + lat_off + x;
     const uint32_t cfgrep = ((uint32_t)cf.noise_cfg << 16) | (uint32_t)(cf.rep0 + task.rep);
     BStage& stg = s_bstage[warp];
-    const int n_it = H + 4;
+    const int n_it = H + 2 * STEPS;
     const int N = Lx * Ly;
     // row offsets: o_ld of the row loaded next, o_v of the row whose v is loaded
     // next, o_a of the level-1 row (all wrap at the lattice's end), o_b of the
     // level-2 row (a row of the band: never wraps)
-    int o_ld = (y0 + 2 * Ly - 2) % Ly * Lx;
+    int o_ld = (y0 + 2 * Ly - STEPS) % Ly * Lx;
     int o_v = o_ld, o_a = 0, o_b = y0 * Lx;
     auto next_row = [&](int o) { return o + Lx == N ? 0 : o + Lx; };
-    // prefetch of iteration ii into slot ii % kBStages: theta_k of row y0 - 2 + ii
-    // and (ii >= 2) v_k of row y0 - 3 + ii; an empty group past the last row
+    // prefetch of iteration ii into slot ii % kBStages: theta_k of row y0 - STEPS + ii
+    // and (ii >= 2) v_k of the row above; an empty group past the last row
     // keeps the group count uniform
     auto issue = [&](int ii, int slot) {
         if (ii < n_it) {
@@ -847,7 +850,7 @@ __global__ void __launch_bounds__(512, 1) band_step_kernel(const DevCfg* cfgs, c
     auto noise = [&](int o, int64_t kk, float c) {
         return p4(gauss4_scaled(philox4x32_10_rk(noise_counter((uint32_t)(o + x) >> 2, cfgrep, kk, 0u), keys), c));
     };
-    o_a = (y0 + Ly - 1) % Ly * Lx;
+    o_a = (y0 + Ly - (STEPS - 1)) % Ly * Lx;
     P4 cn1 = noise(o_a, k, c1), cn2;
     dependency_wait();  // the state of the launch before
     issue(0, 0);
@@ -924,11 +927,12 @@ __global__ void __launch_bounds__(512, 1) band_step_kernel(const DevCfg* cfgs, c
     };
     R0 r0[3];
     R1 r1[3];
-    // iteration i: P0, C0, N0 = level-0 rows y - 2, y - 1, y; P1, C1, N1 =
+    // iteration i: P0, C0, N0 = level-0 rows y - 2, y - 1, y = y0 - STEPS + i; P1, C1, N1 =
     // level-1 rows b - 1, b, a (N1 computed here); levels: how many there are yet.
     // The wait and the two wrap tests cut the iteration into blocks of straight
     // code; each of the two updates, a chain of dependent instructions, gets the
-    // noise that the other one needs next to fill it.
+    // noise that the other one needs next to fill it (a launch of one step: the noise
+    // of the next row).
     auto body = [&](auto levels, int i, int slot, R0& P0, R0& C0, R0& N0, R1& P1, R1& C1, R1& N1) {
         constexpr int LV = decltype(levels)::value;
         issue(i + kBStages - 1, slot == 0 ? kBStages - 1 : slot - 1);
@@ -944,23 +948,26 @@ __global__ void __launch_bounds__(512, 1) band_step_kernel(const DevCfg* cfgs, c
             float sL, cL, sR, cR;
             x_nbrs(prev, 0, sL, cL, sR, cR);
             if (LV >= 2) cn2 = noise(o_b, k + 1, c2);
+            if (STEPS == 1) cn2 = noise(next_row(o_a), k, c1);
             const QuadOut o = quad_update(K1, C0.th, va, cn1, C0.s, C0.c, sL, cL, sR, cR, P0.s, P0.c, N0.s, N0.c);
             N1.th = o.theta;
             N1.v = o.v;
-            const int ra = i - 3;  // row of the band
+            const int ra = i - 1 - STEPS;  // row of the band
             if (REC > 0 && rec1 && ra >= 0 && ra < own)
                 observe(L0{}, J1, h1, y0 + ra, C0.s, C0.c, N0.s, N0.c, sR, cR, o.omega, C0.th);
-            quad_sc(K1.q, N1.th, N1.s, N1.c);
-            publish(N1.s, N1.c, slot, 1);
+            if (STEPS == 2) {
+                quad_sc(K1.q, N1.th, N1.s, N1.c);
+                publish(N1.s, N1.c, slot, 1);
+            }
             edges_published();
             if (!two && ra >= 0 && ra < own) {
                 st4_stream(thD + o_a, f4(N1.th));
                 st4_stream(omD + o_a, f4(N1.v));
             }
             o_a = next_row(o_a);
-            cn1 = noise(o_a, k, c1);
+            cn1 = STEPS == 1 ? cn2 : noise(o_a, k, c1);
         }
-        if (LV >= 2) {  // level 2 on row b = y - 2 (dropped by a launch of one step)
+        if (LV >= 2) {  // level 2 on row b = y - 2
             float sL, cL, sR, cR;
             x_nbrs(prev, 1, sL, cL, sR, cR);
             const QuadOut o = quad_update(K2, C1.th, C1.v, cn2, C1.s, C1.c, sL, cL, sR, cR, P1.s, P1.c, N1.s, N1.c);
@@ -975,12 +982,20 @@ __global__ void __launch_bounds__(512, 1) band_step_kernel(const DevCfg* cfgs, c
     };
     body(L0{}, 0, 0, r0[1], r0[2], r0[0], r1[1], r1[2], r1[0]);
     body(L0{}, 1, 1, r0[2], r0[0], r0[1], r1[2], r1[0], r1[1]);
-    body(L1{}, 2, 2, r0[0], r0[1], r0[2], r1[0], r1[1], r1[2]);
-    body(L1{}, 3, 0, r0[1], r0[2], r0[0], r1[1], r1[2], r1[0]);
-    for (int i = 4; i < n_it; i += 3) {
-        body(L2{}, i, 1, r0[2], r0[0], r0[1], r1[2], r1[0], r1[1]);
-        if (i + 1 < n_it) body(L2{}, i + 1, 2, r0[0], r0[1], r0[2], r1[0], r1[1], r1[2]);
-        if (i + 2 < n_it) body(L2{}, i + 2, 0, r0[1], r0[2], r0[0], r1[1], r1[2], r1[0]);
+    if (STEPS == 1) {
+        for (int i = 2; i < n_it; i += 3) {
+            body(L1{}, i, 2, r0[0], r0[1], r0[2], r1[0], r1[1], r1[2]);
+            if (i + 1 < n_it) body(L1{}, i + 1, 0, r0[1], r0[2], r0[0], r1[1], r1[2], r1[0]);
+            if (i + 2 < n_it) body(L1{}, i + 2, 1, r0[2], r0[0], r0[1], r1[2], r1[0], r1[1]);
+        }
+    } else {
+        body(L1{}, 2, 2, r0[0], r0[1], r0[2], r1[0], r1[1], r1[2]);
+        body(L1{}, 3, 0, r0[1], r0[2], r0[0], r1[1], r1[2], r1[0]);
+        for (int i = 4; i < n_it; i += 3) {
+            body(L2{}, i, 1, r0[2], r0[0], r0[1], r1[2], r1[0], r1[1]);
+            if (i + 1 < n_it) body(L2{}, i + 1, 2, r0[0], r0[1], r0[2], r1[0], r1[1], r1[2]);
+            if (i + 2 < n_it) body(L2{}, i + 2, 0, r0[1], r0[2], r0[0], r1[1], r1[2], r1[0]);
+        }
     }
     cp_async_wait<0>();
     launch_next();
@@ -1022,16 +1037,20 @@ cudaError_t launch_band_step(const DevCfg* d_cfg, const BandTask* tasks, int n_t
 {
     if (n_tasks == 0) return cudaSuccess;
     if (!band_shape(Lx, 1) || H < 1) return cudaErrorInvalidValue;
-    using Kern = void (*)(const DevCfg*, const BandTask*, int, int, int, int64_t, Buffers, const CallArgs*, Partials,
-                          PhiloxKeys);
-#define BAND_ROW(W, A, S) {band_step_kernel<W, A, 0, S>, band_step_kernel<W, A, 1, S>, band_step_kernel<W, A, 2, S>}
-    static const Kern table[3][2][3] = {
-        {BAND_ROW(false, false, false), BAND_ROW(false, false, true)},
-        {BAND_ROW(true, false, false), BAND_ROW(true, false, true)},
-        {BAND_ROW(true, true, false), BAND_ROW(true, true, true)},
-    };
+    using Kern = void (*)(const DevCfg*, const BandTask*, int, int, int64_t, Buffers, const CallArgs*, Partials, PhiloxKeys);
+#define BAND_ROW(N, W, A, S) \
+    {band_step_kernel<N, W, A, 0, S>, band_step_kernel<N, W, A, 1, S>, band_step_kernel<N, W, A, 2, S>}
+#define BAND_TABLE(N)                                                          \
+    {                                                                          \
+        {BAND_ROW(N, false, false, false), BAND_ROW(N, false, false, true)},   \
+        {BAND_ROW(N, true, false, false), BAND_ROW(N, true, false, true)},     \
+        {BAND_ROW(N, true, true, false), BAND_ROW(N, true, true, true)},       \
+    }
+    static const Kern table[2][3][2][3] = {BAND_TABLE(1), BAND_TABLE(2)};
+#undef BAND_TABLE
 #undef BAND_ROW
-    const Kern kern = table[Lx <= 128 ? 0 : (Lx <= 1024 ? 1 : 2)][sched ? 1 : 0][rec < 0 ? 0 : (rec > 2 ? 2 : rec)];
+    const Kern kern = table[n_steps == 2 ? 1 : 0][Lx <= 128 ? 0 : (Lx <= 1024 ? 1 : 2)][sched ? 1 : 0]
+                           [rec < 0 ? 0 : (rec > 2 ? 2 : rec)];
     const int warps = Lx > 128 ? (Lx + 127) / 128 : kNarrowBandWarps;
     const size_t smem = sizeof(BStage) * (size_t)warps;
     if (smem > 46 * 1024) {  // 8 warps or more: with the static part above the default limit
@@ -1040,8 +1059,8 @@ cudaError_t launch_band_step(const DevCfg* d_cfg, const BandTask* tasks, int n_t
                                                    (int)sizeof(BStage) * kBandWarps);
         if (e != cudaSuccess) return e;
     }
-    return launch_dependent(kern, (unsigned)n_tasks, 32 * warps, smem, st, after, 0, d_cfg, tasks, H, n_steps, rd_b ? 1 : 0,
-                            j_local, buf, ca, pa, philox_round_keys(seed));
+    return launch_dependent(kern, (unsigned)n_tasks, 32 * warps, smem, st, after, 0, d_cfg, tasks, H, rd_b ? 1 : 0, j_local,
+                            buf, ca, pa, philox_round_keys(seed));
 }
 
 namespace {
