@@ -162,6 +162,7 @@ struct StripGroup {
     BandTask* d_band_tasks = nullptr;
     size_t d_band_cap = 0;
     int buf = 0;           // 0: the state is in buffers A, 1: in buffers B (within a call)
+    bool ends = false;     // the chunk at hand is the call's last and some lattice runs to its end
 };
 
 // Blocks of band tasks per lattice for bands of H rows.
@@ -558,21 +559,35 @@ bool any_sched(const xy_lattice* L, const std::vector<int>& cfgs)
 }
 bool group_sched(const xy_lattice* L, const StripGroup& g) { return any_sched(L, g.cfgs); }
 
-// Entry g: what a captured chunk fixes of strip group g besides its steps (the
-// kernels chosen by schedule presence, the pairing and the buffers it starts from).
-std::vector<uint8_t> group_flags(const xy_lattice* L)
+// Steps of a group's chunk of `cnt` that run in pairs: all but an odd last one where
+// the group pairs them, except that a call's last chunk splits one pair when its
+// launches would end in buffers B.  Two single steps move 32 bytes a site, and so do a
+// pair and the copy back to A, whose two copies per configuration are launches too
+// (calls of two steps: 8 x 1024^2 95 -> 69, 4 x 100^2 29 -> 24 us).
+int paired_steps(const StripGroup& g, int cnt)
+{
+    if (!g.kt2 || g.band_H == 0) return 0;
+    const int pairs = cnt / 2, launches = pairs + cnt % 2;
+    return 2 * (g.ends && pairs > 0 && ((g.buf + launches) & 1) ? pairs - 1 : pairs);
+}
+
+// Entry g: what a captured chunk of `cnt` steps fixes of strip group g besides its
+// length (the kernels chosen by schedule presence, the pairing and the buffers it
+// starts from).
+std::vector<uint8_t> group_flags(const xy_lattice* L, int cnt)
 {
     std::vector<uint8_t> f(L->strip_groups.size());
     for (size_t g = 0; g < f.size(); ++g) {
         const StripGroup& sg = L->strip_groups[g];
-        f[g] = (uint8_t)((group_sched(L, sg) ? 1 : 0) | (sg.kt2 ? 2 : 0) | (sg.buf ? 4 : 0));
+        const bool split = sg.kt2 && paired_steps(sg, cnt) < cnt / 2 * 2;
+        f[g] = (uint8_t)((group_sched(L, sg) ? 1 : 0) | (sg.kt2 ? 2 : 0) | (sg.buf ? 4 : 0) | (split ? 8 : 0));
     }
     return f;
 }
 
-// The launches of a strip group over `cnt` local steps: pairs of steps where the
-// group pairs them (a launch sums the records of either step, with the same
-// roundings as a single one), a single step at the end of an odd count.
+// The launches of a strip group over `cnt` local steps: pairs of steps (a launch sums
+// the records of either step, with the same roundings as a single one), then single
+// steps.
 struct StepRun {
     int off, n, rec;
 };
@@ -580,8 +595,9 @@ std::vector<StepRun> step_plan(const xy_lattice* L, const StripGroup& g, int cnt
 {
     std::vector<StepRun> out;
     auto rec_at = [&](int i) { return L->cur_rec && ((L->cur_mask >> (i & 63)) & 1u) ? L->cur_rec : 0; };
+    const int paired = paired_steps(g, cnt);
     for (int i = 0; i < cnt;) {
-        const int n = g.kt2 && g.band_H > 0 && i + 1 < cnt ? 2 : 1;
+        const int n = i < paired ? 2 : 1;
         out.push_back(StepRun{i, n, std::max(rec_at(i), n == 2 ? rec_at(i + 1) : 0)});
         i += n;
     }
@@ -870,7 +886,7 @@ void drop_graphs(xy_lattice* L)
 int get_graph(xy_lattice* L, int chunk, bool once, xy_lattice::Graph** out)
 {
     *out = nullptr;
-    const std::vector<uint8_t> gf = group_flags(L);
+    const std::vector<uint8_t> gf = group_flags(L, chunk);
     for (auto& g : L->graphs)
         if (g.chunk == chunk && g.rec == L->cur_rec && g.rec_mask == L->cur_mask && g.groups == gf) {
             *out = &g;
@@ -1259,6 +1275,10 @@ int run_window(xy_lattice* L, int64_t n_max)
         uint64_t mask = 0;
         for (int64_t r = re > 0 ? next_record(pos) : n_max; r < pos + cnt; r = next_record(r + 1)) mask |= 1ull << (r - pos);
         L->cur_mask = mask;
+        for (auto& g : L->strip_groups) {
+            g.ends = false;
+            for (int c : g.cfgs) g.ends = g.ends || (pos + cnt == n_max && L->h_dev[c].n_call == n_max);
+        }
         const bool whole = cnt == (re > 0 && re <= kChunk ? kChunk / re * re : kChunk);
         xy_lattice::Graph* g = nullptr;
         if (cnt >= 2 && !L->timing) {
