@@ -155,6 +155,11 @@ struct StripGroup {
     std::vector<StripTask> tasks = {};
     StripTask* d_tasks = nullptr;
     size_t d_cap = 0;
+    // strips of the steps that record, of shapes that the band kernel does not take
+    int rec_H = 0;
+    std::vector<StripTask> rec_tasks = {};
+    StripTask* d_rec_tasks = nullptr;
+    size_t d_rec_cap = 0;
     int band_H = 0;
     bool kt2_auto = true;  // the tuner's choice: steps in pairs
     bool kt2 = true;       // the choice in force (xy_set_temporal_blocking)
@@ -624,9 +629,11 @@ cudaError_t launch_group(xy_lattice* L, cudaStream_t st, StripGroup& g, int64_t 
         return launch_band_step(L->d_cfg, g.d_band_tasks + lat0 * per, (int)(n_lat * per), g.Lx, g.band_H, r.rec,
                                 group_sched(L, g), r.n, rd_b != 0, g.seed, jl0 + r.off, buf, L->d_call, L->pa, after, st);
     }
-    const int64_t per = (int64_t)g.tasks.size() / g.n_lat;
-    return launch_strip_step(L->d_cfg, g.d_tasks + lat0 * per, (int)(n_lat * per), g.H, g.variant, r.rec,
-                             group_sched(L, g), rd_b != 0, g.seed, jl0 + r.off, buf, L->d_call, L->pa, st);
+    const std::vector<StripTask>& tasks = r.rec ? g.rec_tasks : g.tasks;
+    const int64_t per = (int64_t)tasks.size() / g.n_lat;
+    return launch_strip_step(L->d_cfg, (r.rec ? g.d_rec_tasks : g.d_tasks) + lat0 * per, (int)(n_lat * per),
+                             r.rec ? g.rec_H : g.H, g.variant, r.rec, group_sched(L, g), rd_b != 0, g.seed, jl0 + r.off,
+                             buf, L->d_call, L->pa, st);
 }
 
 // Launch the batched kernels for local steps [jl0, jl0 + cnt) of the current window.
@@ -1359,22 +1366,36 @@ int advance_core(xy_lattice* L, int64_t n, int record_every, double2* rec_dev, i
 
 int build_strip_tasks(xy_lattice* L, StripGroup& g)
 {
-    g.tasks.clear();
-    const int nu = strip_units_per_lattice(g.Lx, g.Ly, g.H);
-    for (int c : g.cfgs)
-        for (int r = 0; r < L->cfg[c].desc.n_replicas; ++r)
-            for (int u0 = 0; u0 < nu; u0 += 8) g.tasks.push_back(StripTask{c, r, u0, nu});
-    if (g.tasks.size() > g.d_cap) {
-        cudaFree(g.d_tasks);
-        g.d_tasks = nullptr;
-        g.d_cap = 0;
-        CK(cudaMalloc(&g.d_tasks, sizeof(StripTask) * g.tasks.size()));
-        g.d_cap = g.tasks.size();
+    auto build = [&](int H, std::vector<StripTask>& tasks, StripTask*& d_tasks, size_t& cap) -> int {
+        tasks.clear();
+        const int nu = strip_units_per_lattice(g.Lx, g.Ly, H);
+        for (int c : g.cfgs)
+            for (int r = 0; r < L->cfg[c].desc.n_replicas; ++r)
+                for (int u0 = 0; u0 < nu; u0 += 8) tasks.push_back(StripTask{c, r, u0, nu});
+        if (tasks.size() > cap) {
+            cudaFree(d_tasks);
+            d_tasks = nullptr;
+            cap = 0;
+            CK(cudaMalloc(&d_tasks, sizeof(StripTask) * tasks.size()));
+            cap = tasks.size();
+        }
+        CK(cudaMemcpyAsync(d_tasks, tasks.data(), sizeof(StripTask) * tasks.size(), cudaMemcpyHostToDevice, L->stream));
+        return XY_OK;
+    };
+    int rc = build(g.H, g.tasks, g.d_tasks, g.d_cap);
+    if (rc == XY_OK && g.band_H == 0) {
+        // Steps that record hold two blocks on an SM where others hold three or four, so
+        // their strips are twice as high where that still fills the chip: fewer halo
+        // rows and ends of strips (every step recorded, 100 steps: 4 x 2176^2 6.86 -> 6.41,
+        // 64 x 2176 x 64 3.99 -> 3.46 ms).
+        const int groups = g.Lx >= 128 ? 1 : 32 / (g.Lx / 4);
+        const bool twice = 2 * g.H <= 64 && g.Ly % (2 * g.H * groups) == 0 &&
+                           g.n_lat * strip_units_per_lattice(g.Lx, g.Ly, 2 * g.H) >= (int64_t)L->sms * 16;
+        g.rec_H = twice ? 2 * g.H : g.H;
+        rc = build(g.rec_H, g.rec_tasks, g.d_rec_tasks, g.d_rec_cap);
     }
-    CK(cudaMemcpyAsync(g.d_tasks, g.tasks.data(), sizeof(StripTask) * g.tasks.size(), cudaMemcpyHostToDevice,
-                       L->stream));
     drop_graphs(L);
-    return XY_OK;
+    return rc;
 }
 
 // Tasks of the band kernel for bands of H rows (from now on the group's height),
@@ -1499,6 +1520,7 @@ void free_lattice(xy_lattice* L)
     for (auto& g : L->res_groups) cudaFree(g.d_tasks);
     for (auto& g : L->strip_groups) {
         cudaFree(g.d_tasks);
+        cudaFree(g.d_rec_tasks);
         cudaFree(g.d_band_tasks);
     }
     cudaFree(L->thB);

@@ -95,9 +95,9 @@ __device__ __forceinline__ double warp_sum(double v)
     return v;
 }
 
-// FP32 warp sum in the same order.  A warp's partial covers at most 8192 sites (64
-// rows of a strip), each term of magnitude O(1), so FP32 keeps it to ~1e-6
-// relative; the partials of different warps and blocks are combined in FP64.
+// FP32 warp sum in the same order.  A warp's partial covers few sites (the plain
+// stepper's quads, the resident one's rows of a lattice), each term of magnitude O(1),
+// so FP32 keeps it to ~1e-6 relative; the partials of different warps and blocks are combined in FP64.
 // (FP64 issues at a small fraction of the FP32 rate on this GPU, so a double
 // butterfly per warp and per step is not free.)
 __device__ __forceinline__ float warp_sumf(float v)
@@ -105,6 +105,55 @@ __device__ __forceinline__ float warp_sumf(float v)
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v = __fadd_rn(v, __shfl_xor_sync(kFull, v, o));
     return v;
+}
+
+// Sums of (M, E) terms as pairs of FP32 values, (sum, what its roundings left out):
+// the error-free addition of Knuth (The Art of Computer Programming, vol. 2, Sec.
+// 4.2.2).  A lane of a band or strip adds up to 128 rows of four sites and its warp 32
+// lanes; in single FP32 sums that cost a record up to 1.5e-8 of its size (FP64
+// additions issue at 1/64 of the rate).  So a record is good to the FP32 sum of each
+// quad's four terms, whatever the height of the band or strip.
+__device__ __forceinline__ void add_exact(float2& sum, float2& rest, float2 v)
+{
+    const float2 m1 = splat2(-1.0f);
+    const float2 t = __fadd2_rn(sum, v);
+    const float2 vv = __ffma2_rn(m1, sum, t);
+    const float2 sv = __ffma2_rn(m1, vv, t);
+    rest = __fadd2_rn(rest, __fadd2_rn(__ffma2_rn(m1, sv, sum), __ffma2_rn(m1, vv, v)));
+    sum = t;
+}
+__device__ __forceinline__ void add_exact(float& sum, float& rest, float v)
+{
+    const float t = __fadd_rn(sum, v);
+    const float vv = __fadd_rn(t, -sum);
+    const float sv = __fadd_rn(t, -vv);
+    rest = __fadd_rn(rest, __fadd_rn(__fadd_rn(sum, -sv), __fadd_rn(v, -vv)));
+    sum = t;
+}
+
+// The lanes' sums of (M, E) of two levels over the warp: the halves of the warp take a
+// level each, the quarters M or E of it, so that four lane groups reduce one value
+// each.  Returns M (lanes 0..7) and E (8..15) of level 0, M (16..23) and E (24..31) of
+// level 1.
+__device__ __forceinline__ double warp_sum_pairs(const float2 (&sum)[2], const float2 (&rest)[2], int lane)
+{
+    auto xchg = [](float v, int o) { return __shfl_xor_sync(kFull, v, o); };
+    const bool hi = (lane & 16) != 0, en = (lane & 8) != 0;
+    const float2 give = hi ? sum[0] : sum[1], give_r = hi ? rest[0] : rest[1];
+    float2 s2 = hi ? sum[1] : sum[0];
+    float2 r2 = __fadd2_rn(hi ? rest[1] : rest[0], make_float2(xchg(give_r.x, 16), xchg(give_r.y, 16)));
+    add_exact(s2, r2, make_float2(xchg(give.x, 16), xchg(give.y, 16)));
+    float s = en ? s2.y : s2.x, r = en ? r2.y : r2.x;
+    const float so = xchg(en ? s2.x : s2.y, 8);
+    r = __fadd_rn(r, xchg(en ? r2.x : r2.y, 8));
+    add_exact(s, r, so);
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) {
+        const float sx = xchg(s, o), rx = xchg(r, o);
+        r = __fadd_rn(r, rx);
+        add_exact(s, r, sx);
+    }
+    return (double)s + (isfinite(r) ? (double)r : 0.0);  // (a sum that is not finite has no rest)
 }
 
 // Commit one unit's (M, E) partial of lattice b; the unit that arrives last
@@ -389,7 +438,7 @@ struct StripCtx {
     StepConst K;
     float Jx, Jy, hF, eref;  // energy constants in registers (stores may alias the descriptor)
     bool stag;
-    float pm, pe;
+    float2 sum, rest;  // (M, E)
 };
 
 // All rows of the unit, one row per iteration with a sliding window of three
@@ -469,24 +518,18 @@ __device__ __forceinline__ void strip_rows(StripCtx& X, const DevCfg& cf, const 
         }
         const float4 cn = gauss4_scaled(philox4x32_10_rk(noise_counter(quad, X.cfgrep, X.k, 0u), keys), X.K.c);
         const QuadOut o = quad_update(X.K, C.th, p4(v), p4(cn), C.s, C.c, sL, cL, sR, cR, P.s, P.c, N.s, N.c);
-        if (REC == 2) {
-#pragma unroll
-            for (int s = 0; s < 4; ++s) {
-                const float cs = p4get(C.s, s), cc = p4get(C.c, s);
-                const float sr = s == 3 ? sR : p4get(C.s, s + 1);
-                const float cr = s == 3 ? cR : p4get(C.c, s + 1);
-                const float bx = fmaf(cc, cr, __fmul_rn(cs, sr));
-                const float by = fmaf(cc, p4get(N.c, s), __fmul_rn(cs, p4get(N.s, s)));
-                X.pe = __fadd_rn(X.pe, site_energy_rel(p4get(o.omega, s), bx, by, cosp_of(X.K.p, p4get(C.th, s)), X.Jx,
-                                                       X.Jy, X.hF, X.eref));
-            }
-        }
         if (REC) {
             // order parameter of the row: sites x + 0, x + 2 have the parity of
             // y (x is a multiple of 4), sites x + 1, x + 3 the other one
             const float ev = __fadd_rn(C.s.a.x, C.s.b.x), od = __fadd_rn(C.s.a.y, C.s.b.y);
             const float m = !X.stag ? __fadd_rn(ev, od) : ((y & 1) ? __fadd_rn(od, -ev) : __fadd_rn(ev, -od));
-            X.pm = __fadd_rn(X.pm, m);
+            float pe = 0.f;
+            if (REC == 2) {
+                const P4 e = quad_energy_rel(X.K.p, make_float2(X.Jx, X.Jy), X.hF, X.eref, C.s, C.c, N.s, N.c, sR, cR,
+                                             o.omega, C.th);
+                pe = __fadd_rn(__fadd_rn(__fadd_rn(e.a.x, e.a.y), e.b.x), e.b.y);
+            }
+            add_exact(X.sum, X.rest, make_float2(m, pe));
         }
         st4_stream(p_to + X.x, f4(o.theta));
         st4_stream(p_vo + X.x, f4(o.v));
@@ -548,8 +591,7 @@ __global__ void __launch_bounds__(256, MINB) strip_step_kernel(const DevCfg* cfg
     X.srcR = grp * G + (X.lg + 1) % G;
     X.rec = ca.record_every > 0 && (X.k % ca.record_every) == 0;
     X.cfgrep = ((uint32_t)cf.noise_cfg << 16) | (uint32_t)(cf.rep0 + task.rep);
-    X.pm = 0.f;
-    X.pe = 0.f;
+    X.sum = X.rest = make_float2(0.f, 0.f);
     if (REC > 0 && X.rec) {  // block-uniform
         const float2 Jk = SCHED ? couplings_at(cf, X.k) : make_float2(cf.Jx, cf.Jy);
         X.Jx = Jk.x;
@@ -560,8 +602,9 @@ __global__ void __launch_bounds__(256, MINB) strip_step_kernel(const DevCfg* cfg
         if (live) strip_rows<REC>(X, cf, keys, ybeg, H, s_stage[warp]);
         // one partial per block: warp sums, then the block's warps in order
         __shared__ double2 s_part[8];
-        const double wm = warp_sumf(X.pm), we = warp_sumf(X.pe);
-        if (lane == 0) s_part[warp] = make_double2(wm, we);
+        const float2 sum[2] = {X.sum, {}}, rest[2] = {X.rest, {}};
+        const double w = warp_sum_pairs(sum, rest, lane);
+        if ((lane & 23) == 0) (&s_part[warp].x)[lane >> 3] = w;  // lanes 0 and 8
         __syncthreads();
         if (warp == 0) {
             const int nw = (int)(blockDim.x >> 5);
@@ -605,8 +648,9 @@ cudaError_t launch_strip_step(const DevCfg* d_cfg, const StripTask* tasks, int n
     const PhiloxKeys keys = philox_round_keys(seed);
     using Kern = void (*)(const DevCfg*, const StripTask*, int, int, int64_t, Buffers, const CallArgs*, Partials,
                           PhiloxKeys);
-    // Launches that record run two blocks per SM: capped at 80 or 64 registers the
-    // recording code spills inside the row loop.
+    // Launches that record run two blocks per SM: capped at 80 registers the recording
+    // code spills inside the row loop (100 steps of 4 x 2176^2, every second one
+    // recorded: 6.2 ms at three blocks, 5.9 at two).
     static const Kern table[2][3][3] = {
         {
             {strip_step_kernel<2, 0, false>, strip_step_kernel<2, 1, false>, strip_step_kernel<2, 2, false>},
@@ -694,54 +738,6 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity)
         if (done) return true;
     }
     return false;
-}
-
-// Sums of (M, E) terms as pairs of FP32 values, (sum, what its roundings left out):
-// the error-free addition of Knuth (The Art of Computer Programming, vol. 2, Sec.
-// 4.2.2).  A band's lane adds up to 128 rows of four sites and its warp 32 lanes; in
-// single FP32 sums that cost a record up to 1.5e-8 of its size (FP64 additions issue
-// at 1/64 of the rate).  So a record is good to the FP32 sum of each quad's four
-// terms, whatever the height of the bands.
-__device__ __forceinline__ void add_exact(float2& sum, float2& rest, float2 v)
-{
-    const float2 m1 = splat2(-1.0f);
-    const float2 t = __fadd2_rn(sum, v);
-    const float2 vv = __ffma2_rn(m1, sum, t);
-    const float2 sv = __ffma2_rn(m1, vv, t);
-    rest = __fadd2_rn(rest, __fadd2_rn(__ffma2_rn(m1, sv, sum), __ffma2_rn(m1, vv, v)));
-    sum = t;
-}
-__device__ __forceinline__ void add_exact(float& sum, float& rest, float v)
-{
-    const float t = __fadd_rn(sum, v);
-    const float vv = __fadd_rn(t, -sum);
-    const float sv = __fadd_rn(t, -vv);
-    rest = __fadd_rn(rest, __fadd_rn(__fadd_rn(sum, -sv), __fadd_rn(v, -vv)));
-    sum = t;
-}
-// The lanes' sums of (M, E) of two levels over the warp: the halves of the warp take a
-// level each, the quarters M or E of it, so that four lane groups reduce one value
-// each.  Returns M (lanes 0..7) and E (8..15) of level 0, M (16..23) and E (24..31) of
-// level 1.
-__device__ __forceinline__ double warp_sum_pairs(const float2 (&sum)[2], const float2 (&rest)[2], int lane)
-{
-    auto xchg = [](float v, int o) { return __shfl_xor_sync(kFull, v, o); };
-    const bool hi = (lane & 16) != 0, en = (lane & 8) != 0;
-    const float2 give = hi ? sum[0] : sum[1], give_r = hi ? rest[0] : rest[1];
-    float2 s2 = hi ? sum[1] : sum[0];
-    float2 r2 = __fadd2_rn(hi ? rest[1] : rest[0], make_float2(xchg(give_r.x, 16), xchg(give_r.y, 16)));
-    add_exact(s2, r2, make_float2(xchg(give.x, 16), xchg(give.y, 16)));
-    float s = en ? s2.y : s2.x, r = en ? r2.y : r2.x;
-    const float so = xchg(en ? s2.x : s2.y, 8);
-    r = __fadd_rn(r, xchg(en ? r2.x : r2.y, 8));
-    add_exact(s, r, so);
-#pragma unroll
-    for (int o = 4; o > 0; o >>= 1) {
-        const float sx = xchg(s, o), rx = xchg(r, o);
-        r = __fadd_rn(r, rx);
-        add_exact(s, r, sx);
-    }
-    return (double)s + (isfinite(r) ? (double)r : 0.0);  // (a sum that is not finite has no rest)
 }
 
 struct R0 {  // a level-0 row: theta_k and its (sin q t, cos q t)
