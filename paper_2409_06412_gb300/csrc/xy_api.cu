@@ -1421,18 +1421,11 @@ int build_band_tasks(xy_lattice* L, StripGroup& g, int H)
     return XY_OK;
 }
 
-// smallest strip height the autotuner may pick for a shape
-int min_strip_H(int Lx, int Ly)
-{
-    const int groups = Lx >= 128 ? 1 : 32 / (Lx / 4);
-    for (int H : {4, 8, 16, 32, 64, 2, 1})
-        if (Ly % (H * groups) == 0) return H;
-    return 1;
-}
-
 int classify(xy_lattice* L)
 {
     // default kernel per configuration; see the design notes for the rules
+    // record partials per lattice and step: one per 256 quads (plain stepper), which is
+    // enough for one per block of eight strips, or one per block of bands (below)
     int max_units = 1;
     int dev = 0, sms = 148;
     if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -1453,8 +1446,6 @@ int classify(xy_lattice* L)
         } else if (H > 0 || band_shape(Lx, Ly)) {
             h.kind = 1;
             h.H = H;
-            if (H > 0)
-                max_units = std::max(max_units, strip_units_per_lattice(Lx, Ly, std::min(H, min_strip_H(Lx, Ly))));
         } else {
             h.kind = 2;
         }
