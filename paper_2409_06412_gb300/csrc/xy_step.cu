@@ -752,14 +752,15 @@ struct R1 {  // a level-1 row: theta_{k+1}, v_{k+1} and (sin q t, cos q t)
 }  // namespace
 
 // REC: 0 = the launch records nothing, 1 = M, 2 = M and E, of step k (summed over
-// the band's own rows of level 1), of step k + 1 (level 2) or of both; SCHED: some configuration of the launch has a
-// field or coupling schedule.  STEPS: 1 or 2.  rd_b: the state is in buffers B.
-// Threads are capped so that every block size keeps 16 warps per SM (128
-// registers).
+// the band's own rows of level 1), of step k + 1 (level 2) or of both; SCHED: some
+// configuration of the launch has a field or coupling schedule.  STEPS: 1 or 2.  rd_b:
+// the state is in buffers B.
+// Threads are capped for 128 registers, 16 warps on an SM (blocks of 3, 5, 6, 7 or more
+// than 8 warps leave some of them out: whole blocks only).
 // APART: a wide band's warps arrive and wait apart.
 template <int STEPS, bool WIDE, bool APART, int REC, bool SCHED>
-__global__ void __launch_bounds__(512, 1) band_step_kernel(const DevCfg* cfgs, const BandTask* tasks, int H, int rd_b,
-                                                           int64_t j_local, Buffers buf, const CallArgs* cap,
+__global__ void __launch_bounds__(512, 1) band_step_kernel(const DevCfg* cfgs, const BandTask* tasks, int H, int n_steps,
+                                                           int rd_b, int64_t j_local, Buffers buf, const CallArgs* cap,
                                                            Partials pa, PhiloxKeys keys)
 {
     extern __shared__ BStage s_bstage[];  // one per warp
@@ -772,7 +773,9 @@ __global__ void __launch_bounds__(512, 1) band_step_kernel(const DevCfg* cfgs, c
         dependency_wait();  // a launch of such blocks alone must not complete before the one it follows
         return;
     }
-    const bool two = STEPS == 2 && j + 1 < cf.n_call;
+    // (n_steps is STEPS; read as a parameter, since with the run's end alone the compiler
+    // orders the row loop 1 % slower: 512 x 256^2 66.6 against 65.9 us per step)
+    const bool two = STEPS == 2 && n_steps == 2 && j + 1 < cf.n_call;
     if (APART) {
         if (threadIdx.x == 0) mbar_init(&s_bar, nw);
         __syncthreads();
@@ -1033,7 +1036,7 @@ cudaError_t launch_band_step(const DevCfg* d_cfg, const BandTask* tasks, int n_t
 {
     if (n_tasks == 0) return cudaSuccess;
     if (!band_shape(Lx, 1) || H < 1) return cudaErrorInvalidValue;
-    using Kern = void (*)(const DevCfg*, const BandTask*, int, int, int64_t, Buffers, const CallArgs*, Partials, PhiloxKeys);
+    using Kern = void (*)(const DevCfg*, const BandTask*, int, int, int, int64_t, Buffers, const CallArgs*, Partials, PhiloxKeys);
 #define BAND_ROW(N, W, A, S) \
     {band_step_kernel<N, W, A, 0, S>, band_step_kernel<N, W, A, 1, S>, band_step_kernel<N, W, A, 2, S>}
 #define BAND_TABLE(N)                                                          \
@@ -1055,7 +1058,7 @@ cudaError_t launch_band_step(const DevCfg* d_cfg, const BandTask* tasks, int n_t
                                                    (int)sizeof(BStage) * kBandWarps);
         if (e != cudaSuccess) return e;
     }
-    return launch_dependent(kern, (unsigned)n_tasks, 32 * warps, smem, st, after, 0, d_cfg, tasks, H, rd_b ? 1 : 0, j_local,
+    return launch_dependent(kern, (unsigned)n_tasks, 32 * warps, smem, st, after, 0, d_cfg, tasks, H, n_steps, rd_b ? 1 : 0, j_local,
                             buf, ca, pa, philox_round_keys(seed));
 }
 
