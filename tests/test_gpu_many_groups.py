@@ -38,3 +38,9 @@ def _compare(shapes, seeds, calls=((1, 0), (2, 1), (70, 9), (130, 0))):
                                           ([(128, 64, 40), (16, 16, 5)], 2)], ids=str)
 def test_resident_groups(shapes, seeds):
     _compare(shapes, seeds)
+
+
+@pytest.mark.parametrize("shapes,seeds", [([(256, 24, 2)], 12), ([(96, 40, 3), (64, 64, 1)], 7),
+                                          ([(100, 12, 1), (2176, 4, 1), (2052, 3, 1)], 4)], ids=str)
+def test_more_groups_than_streams(shapes, seeds):
+    _compare(shapes, seeds)
