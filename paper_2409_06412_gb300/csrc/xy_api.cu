@@ -911,6 +911,7 @@ int launch_resident_forked(xy_lattice* L, int64_t jl0, int cnt)
 
 constexpr size_t kMaxGraphs = 64;
 constexpr size_t kFreeGraphs = 8;
+constexpr size_t kRestGraphs = 48;  // rests are captured up to here; the other places are whole chunks'
 
 void drop_graphs(xy_lattice* L)
 {
@@ -924,8 +925,8 @@ void drop_graphs(xy_lattice* L)
 // their kernels overlap (one branch's launches fill the SMs another's leave
 // idle as its launch drains) instead of taking turns every step.
 // once: this kind of chunk may not come again (the rest of a call whose length
-// varies): past the first few kinds it is captured from its second time on, and
-// *out is null before.
+// varies): past the first few kinds it is captured from its second time on, while
+// there is room, and *out is null else.
 int get_graph(xy_lattice* L, int chunk, bool once, xy_lattice::Graph** out)
 {
     *out = nullptr;
@@ -935,6 +936,7 @@ int get_graph(xy_lattice* L, int chunk, bool once, xy_lattice::Graph** out)
             *out = &g;
             return XY_OK;
         }
+    if (once && L->graphs.size() >= kRestGraphs) return XY_OK;
     if (once && L->graphs.size() >= kFreeGraphs) {
         const xy_lattice::Graph kind{chunk, L->cur_rec, L->cur_mask, gf, nullptr, 0};
         bool seen = false;
@@ -1247,6 +1249,12 @@ int ensure_tasks(xy_lattice* L)
 }
 
 constexpr int kChunk = 64;             // steps of a captured chunk at most (the bits of cur_mask)
+// Record intervals above this start their whole chunks at a record, so that these are
+// of one kind whatever step a call begins at (127 steps, one record in 50, call after
+// call: each began at another of 50 phases and captured its chunks anew; 64 lattices
+// of 8^2 804 -> 310 us per call, 8 x 200 x 152 785 -> 411).  Shorter ones have few phases, whose
+// kinds are all kept, and start with the call.
+constexpr int kFewPhases = 16;
 constexpr int kResidentSteps = 1 << 14;  // steps of one resident launch at most
 
 // Advance every configuration by its n_call of the current window (already
@@ -1314,7 +1322,10 @@ int run_window(xy_lattice* L, int64_t n_max)
     int64_t pos = 0;
     while (pos < n_max) {
         int64_t cnt;
-        if (re > 0 && re <= kChunk) {
+        const int64_t at = re > kFewPhases && re <= kChunk ? next_record(pos) : pos;
+        if (at > pos && at < n_max) {
+            cnt = std::min<int64_t>(kChunk, at - pos);  // up to the first record
+        } else if (re > 0 && re <= kChunk) {
             cnt = std::min<int64_t>(kChunk / re * re, n_max - pos);
         } else {
             cnt = std::min<int64_t>(kChunk, next_record(pos + 1) - pos);  // up to the next record
