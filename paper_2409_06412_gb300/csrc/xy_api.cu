@@ -1068,11 +1068,12 @@ int autotune_lattice(xy_lattice* L)
         if ((int64_t)g.Lx * g.Ly * g.n_lat < ((int64_t)1 << 21)) continue;  // too small to matter
         const int n_parts = parts[&g - L->strip_groups.data()];
         // milliseconds of one launch per slice: the best of 5 timings, each over
-        // enough launches to span `span` milliseconds (single launches of a small
-        // batch differ by less than their timing noise; and over a few launches the
-        // slices' start and end count as much as what a long run repeats: 32 lattices
-        // of 1024^2 then took 32-row bands, 5 % slower than 64-row ones in long runs)
-        auto time_it = [&](const std::vector<int>& cuts, float span, auto&& run, float& out) -> int {
+        // enough launches to span `span` milliseconds, `most` of them (single launches
+        // of a small batch differ by less than their timing noise; and over a few
+        // launches the slices' start and end count as much as what a long run repeats:
+        // 32 lattices of 1024^2 then took 32-row bands, 5 % slower than 64-row ones in
+        // long runs)
+        auto time_it = [&](const std::vector<int>& cuts, float span, int most, auto&& run, float& out) -> int {
             int reps = 3;
             out = 1e30f;
             for (int round = 0; round < 5; ++round) {
@@ -1085,7 +1086,7 @@ int autotune_lattice(xy_lattice* L)
                 CK(cudaEventElapsedTime(&ms, e0, e1));
                 L->launches += (int64_t)(1 + reps) * ((int)cuts.size() - 1);
                 out = std::min(out, ms / reps);
-                if (round == 0 && ms < span) reps = std::min(64, (int)(span / std::max(ms / reps, 1e-3f)) + 1);
+                if (round == 0 && ms < span) reps = std::min(most, (int)(span / std::max(ms / reps, 1e-3f)) + 1);
             }
             return XY_OK;
         };
@@ -1109,7 +1110,9 @@ int autotune_lattice(xy_lattice* L)
                 const std::vector<int> cuts = cut_tasks(g.tasks, n_parts);
                 for (int v : {2, 3, 4}) {
                     float t = 1e30f;
-                    rc = time_it(cuts, 0.5f, [&](cudaStream_t st, int t0, int cnt) {
+                    // (where strips take every step their choice decides: over 64 launches of 8
+                    // us 2 x 2176 x 512 took 8-row strips every other time, 9.5 for 8.5 us a step)
+                    rc = time_it(cuts, g.band_H == 0 ? 3.0f : 0.5f, g.band_H == 0 ? 512 : 64, [&](cudaStream_t st, int t0, int cnt) {
                         return launch_strip_step(L->d_cfg, g.d_tasks + t0, cnt, H, v, 0, group_sched(L, g), false, g.seed, 0,
                                                  buf, L->d_call, L->pa, st);
                     }, t);
@@ -1140,7 +1143,7 @@ int autotune_lattice(xy_lattice* L)
         if (h2 == 0) {
             float t1 = 1e30f, best2 = 1e30f;
             if (g.strip_ok)
-                rc = time_it(cut_tasks(g.tasks, n_parts), 3.0f, [&](cudaStream_t st, int t0, int cnt) {
+                rc = time_it(cut_tasks(g.tasks, n_parts), 3.0f, 64, [&](cudaStream_t st, int t0, int cnt) {
                     return launch_strip_step(L->d_cfg, g.d_tasks + t0, cnt, g.H, g.variant, 0, group_sched(L, g), false,
                                              g.seed, 0, buf, L->d_call, L->pa, st);
                 }, t1);
@@ -1149,7 +1152,7 @@ int autotune_lattice(xy_lattice* L)
                 const int H = even_band(g.Ly, h);
                 if ((rc = build_band_tasks(L, g, H))) break;
                 float t2 = 1e30f;
-                rc = time_it(cut_tasks(g.band_tasks, n_parts), 3.0f, [&](cudaStream_t st, int t0, int cnt) {
+                rc = time_it(cut_tasks(g.band_tasks, n_parts), 3.0f, 64, [&](cudaStream_t st, int t0, int cnt) {
                     return launch_band_step(L->d_cfg, g.d_band_tasks + t0, cnt, g.Lx, H, 0, group_sched(L, g), 2, false,
                                             g.seed, 0, buf, L->d_call, L->pa, false, st);
                 }, t2);
@@ -1252,8 +1255,8 @@ constexpr int kChunk = 64;             // steps of a captured chunk at most (the
 // Record intervals above this start their whole chunks at a record, so that these are
 // of one kind whatever step a call begins at (127 steps, one record in 50, call after
 // call: each began at another of 50 phases and captured its chunks anew; 64 lattices
-// of 8^2 804 -> 310 us per call, 8 x 200 x 152 785 -> 411).  Shorter ones have few phases, whose
-// kinds are all kept, and start with the call.
+// of 8^2 804 -> 310 us per call, 8 x 200 x 152 785 -> 411).  Shorter ones have few
+// phases, whose kinds are all kept, and start with the call.
 constexpr int kFewPhases = 16;
 constexpr int kResidentSteps = 1 << 14;  // steps of one resident launch at most
 
