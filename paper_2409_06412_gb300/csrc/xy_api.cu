@@ -2059,32 +2059,37 @@ int xy_structure_factor(xy_lattice* L, int b_first, int b_count, int K, double r
         max_x = std::max(max_x, d.Lx);
         max_y = std::max(max_y, d.Ly);
     }
-    // the table of all lattices and the partial sums stay on the object (grown on
-    // demand; cudaFree waits for the device, so no launch still uses the old block)
-    void *lats = nullptr, *scratch = nullptr;
-    if (!L->slot[xy_lattice::kSfLats].p) {
-        std::vector<SfLattice>& h = L->h_sf;
-        h.clear();
+    // The table of all lattices and the partial sums stay on the object (the sums grown
+    // on demand; cudaFree waits for the device, so no launch still uses the old block).
+    // A caller's graph replays after the block may have grown, so a captured call takes
+    // memory of the graph's own, and fills a table of its own if it is the first call.
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(L->stream, &cs) != cudaSuccess) cudaGetLastError();
+    const bool capturing = cs != cudaStreamCaptureStatusNone;
+    std::vector<SfLattice>& h = L->h_sf;
+    if (h.empty()) {
         h.reserve((size_t)L->B);
         for (const DevCfg& d : L->h_dev)
             for (int r = 0; r < d.n_rep; ++r) h.push_back(SfLattice{d.offset + r * d.N, d.Lx, d.Ly});
-        cudaError_t e0 = reserve_slot(L, xy_lattice::kSfLats, sizeof(SfLattice) * h.size(), &lats);
-        if (e0 == cudaSuccess)
-            e0 = cudaMemcpyAsync(lats, h.data(), sizeof(SfLattice) * h.size(), cudaMemcpyHostToDevice, L->stream);
-        if (e0 != cudaSuccess) {
-            cudaGetLastError();
+    }
+    const size_t lat_bytes = sizeof(SfLattice) * h.size(), part_bytes = sf_scratch_bytes(b_count, max_x, max_y, K);
+    void *lats = L->slot[xy_lattice::kSfLats].p, *scratch = nullptr;
+    const bool fill = !lats;
+    cudaError_t e0 = cudaSuccess;
+    if (fill) {
+        e0 = capturing ? cudaMallocAsync(&lats, lat_bytes, L->stream) : reserve_slot(L, xy_lattice::kSfLats, lat_bytes, &lats);
+        if (e0 == cudaSuccess) e0 = cudaMemcpyAsync(lats, h.data(), lat_bytes, cudaMemcpyHostToDevice, L->stream);
+        if (e0 != cudaSuccess && !capturing) {
             cudaFree(L->slot[xy_lattice::kSfLats].p);
             L->slot[xy_lattice::kSfLats] = {};
-            return fail(XY_ENOMEM, "structure factor tables: %s", cudaGetErrorString(e0));
         }
     }
-    lats = L->slot[xy_lattice::kSfLats].p;
-    {
-        const cudaError_t e0 = reserve_slot(L, xy_lattice::kSfPart, sf_scratch_bytes(b_count, max_x, max_y, K), &scratch);
-        if (e0 != cudaSuccess) {
-            cudaGetLastError();
-            return fail(XY_ENOMEM, "structure factor partial sums: %s", cudaGetErrorString(e0));
-        }
+    if (e0 == cudaSuccess)
+        e0 = capturing ? cudaMallocAsync(&scratch, part_bytes, L->stream)
+                       : reserve_slot(L, xy_lattice::kSfPart, part_bytes, &scratch);
+    if (e0 != cudaSuccess) {
+        cudaGetLastError();
+        return fail(XY_ENOMEM, "structure factor tables and partial sums: %s", cudaGetErrorString(e0));
     }
     const bool dev = is_device_ptr(S_par) && is_device_ptr(S_perp);
     double *dp = S_par, *dq = S_perp;
@@ -2101,6 +2106,10 @@ int xy_structure_factor(xy_lattice* L, int b_first, int b_count, int K, double r
     cudaError_t e = launch_structure_factor(L->thA, static_cast<const SfLattice*>(lats) + b_first, b_count, max_x, max_y, K,
                                             (float)rotor, scratch, dp, dq, &launches, L->stream);
     L->launches += launches;
+    if (capturing) {
+        if (e == cudaSuccess) e = cudaFreeAsync(scratch, L->stream);
+        if (e == cudaSuccess && fill) e = cudaFreeAsync(lats, L->stream);
+    }
     if (e == cudaSuccess && !dev) {
         e = cudaMemcpyAsync(S_par, dp, bytes, cudaMemcpyDeviceToHost, L->stream);
         if (e == cudaSuccess) e = cudaMemcpyAsync(S_perp, dq, bytes, cudaMemcpyDeviceToHost, L->stream);
