@@ -1022,9 +1022,9 @@ int time_window(xy_lattice* L, int64_t n_call)
 }
 
 // First part of every key of the tuner's cache: the GPU and the generation of
-// the kernels.  Raised when a kernel changes enough that choices timed with the
-// old one no longer hold (a cache file outlives the library that wrote it).
-constexpr int kTuneGeneration = 2;
+// the kernels.  Raised when a kernel, or how candidates are timed, changes enough that
+// choices timed before no longer hold (a cache file outlives the library that wrote it).
+constexpr int kTuneGeneration = 3;
 
 std::string gpu_name()
 {
@@ -1059,6 +1059,7 @@ int autotune_lattice(xy_lattice* L)
     CK(cudaEventCreate(&e1));
     int rc = time_window(L, 8);
     const Buffers buf = state_buffers(L);
+    bool warm = false;
     // candidates run sliced the way the captured chunks run them
     const std::vector<int> parts =
         slice_parts(L->strip_groups, (int)L->res_groups.size() + (L->plain_cfgs.empty() ? 0 : 1),
@@ -1067,28 +1068,51 @@ int autotune_lattice(xy_lattice* L)
         if (rc) break;
         if ((int64_t)g.Lx * g.Ly * g.n_lat < ((int64_t)1 << 21)) continue;  // too small to matter
         const int n_parts = parts[&g - L->strip_groups.data()];
-        // milliseconds of one launch per slice: the best of 5 timings, each over
-        // enough launches to span `span` milliseconds, `most` of them (single launches
-        // of a small batch differ by less than their timing noise; and over a few
-        // launches the slices' start and end count as much as what a long run repeats:
-        // 32 lattices of 1024^2 then took 32-row bands, 5 % slower than 64-row ones in
-        // long runs)
-        auto time_it = [&](const std::vector<int>& cuts, float span, int most, auto&& run, float& out) -> int {
-            int reps = 3;
-            out = 1e30f;
-            for (int round = 0; round < 5; ++round) {
-                CK(launch_sliced(L, cuts, 1, run));
+        // Milliseconds of one launch per slice: the mean of 5 timings (how the slices fall
+        // beside each other differs from run to run: 8-row strips of 2 x 2176 x 512 take
+        // 7.1 or 8.5 us), each of a captured run of enough launches to span `span`
+        // milliseconds (256 at most).  Over a few launches the slices' start and end
+        // count as much as what a long run repeats (32 lattices of 1024^2 took 32-row
+        // bands, 5 % slower than 64-row ones in long runs), and short launches made one
+        // by one are timed by the host (chosen so, and captured: 40 x 256^2 8.3 and 7.5 us
+        // a step, 6 x 384 x 1024 7.8 and 7.1, 300 x 100^2 12.0 and 10.7, 2 x 2176 x 512 8.5 or
+        // 9.5 and 8.5).
+        auto time_it = [&](const std::vector<int>& cuts, float span, auto&& run, float& out) -> int {
+            auto elapsed = [&](float& ms, auto&& work) -> int {
                 CK(cudaEventRecord(e0, L->stream));
-                CK(launch_sliced(L, cuts, reps, run));
+                CK(work());
                 CK(cudaEventRecord(e1, L->stream));
                 CK(cudaEventSynchronize(e1));
-                float ms = 0.f;
                 CK(cudaEventElapsedTime(&ms, e0, e1));
-                L->launches += (int64_t)(1 + reps) * ((int)cuts.size() - 1);
-                out = std::min(out, ms / reps);
-                if (round == 0 && ms < span) reps = std::min(most, (int)(span / std::max(ms / reps, 1e-3f)) + 1);
+                return XY_OK;
+            };
+            float ms = 0.f;
+            CK(launch_sliced(L, cuts, 1, run));
+            int rc1 = elapsed(ms, [&] { return launch_sliced(L, cuts, 3, run); });
+            if (rc1) return rc1;
+            const int reps = std::min(256, (int)(3.0f * span / std::max(ms, 1e-3f)) + 1);
+            // the launches go to L->stream and the branch streams forked from it
+            cudaGraph_t graph = nullptr;
+            cudaGraphExec_t exec = nullptr;
+            CK(cudaStreamBeginCapture(L->cap_stream, cudaStreamCaptureModeThreadLocal));
+            std::swap(L->stream, L->cap_stream);
+            const cudaError_t el = launch_sliced(L, cuts, reps, run);
+            std::swap(L->stream, L->cap_stream);
+            cudaError_t e = cudaStreamEndCapture(L->cap_stream, &graph);
+            if (el != cudaSuccess) e = el;
+            if (e == cudaSuccess) e = cudaGraphInstantiate(&exec, graph, 0);
+            if (graph) cudaGraphDestroy(graph);
+            CK(e);
+            out = 0.f;
+            // (the first run uploads the graph; the first candidate's also wake the device)
+            for (int round = warm ? -1 : -10; round < 5 && rc1 == XY_OK; ++round) {
+                rc1 = elapsed(ms, [&] { return cudaGraphLaunch(exec, L->stream); });
+                if (round >= 0) out += ms / (5 * reps);
             }
-            return XY_OK;
+            cudaGraphExecDestroy(exec);
+            warm = true;
+            L->launches += (int64_t)(4 + 6 * reps) * ((int)cuts.size() - 1);
+            return rc1;
         };
         // a cached choice is used only if it satisfies the same constraints
         // as the candidates below (the cache is a plain text file)
@@ -1110,9 +1134,8 @@ int autotune_lattice(xy_lattice* L)
                 const std::vector<int> cuts = cut_tasks(g.tasks, n_parts);
                 for (int v : {2, 3, 4}) {
                     float t = 1e30f;
-                    // (where strips take every step their choice decides: over 64 launches of 8
-                    // us 2 x 2176 x 512 took 8-row strips every other time, 9.5 for 8.5 us a step)
-                    rc = time_it(cuts, g.band_H == 0 ? 3.0f : 0.5f, g.band_H == 0 ? 512 : 64, [&](cudaStream_t st, int t0, int cnt) {
+                    // (where strips take every step their choice decides)
+                    rc = time_it(cuts, g.band_H == 0 ? 3.0f : 0.5f, [&](cudaStream_t st, int t0, int cnt) {
                         return launch_strip_step(L->d_cfg, g.d_tasks + t0, cnt, H, v, 0, group_sched(L, g), false, g.seed, 0,
                                                  buf, L->d_call, L->pa, st);
                     }, t);
@@ -1143,7 +1166,7 @@ int autotune_lattice(xy_lattice* L)
         if (h2 == 0) {
             float t1 = 1e30f, best2 = 1e30f;
             if (g.strip_ok)
-                rc = time_it(cut_tasks(g.tasks, n_parts), 3.0f, 64, [&](cudaStream_t st, int t0, int cnt) {
+                rc = time_it(cut_tasks(g.tasks, n_parts), 3.0f, [&](cudaStream_t st, int t0, int cnt) {
                     return launch_strip_step(L->d_cfg, g.d_tasks + t0, cnt, g.H, g.variant, 0, group_sched(L, g), false,
                                              g.seed, 0, buf, L->d_call, L->pa, st);
                 }, t1);
@@ -1152,7 +1175,7 @@ int autotune_lattice(xy_lattice* L)
                 const int H = even_band(g.Ly, h);
                 if ((rc = build_band_tasks(L, g, H))) break;
                 float t2 = 1e30f;
-                rc = time_it(cut_tasks(g.band_tasks, n_parts), 3.0f, 64, [&](cudaStream_t st, int t0, int cnt) {
+                rc = time_it(cut_tasks(g.band_tasks, n_parts), 3.0f, [&](cudaStream_t st, int t0, int cnt) {
                     return launch_band_step(L->d_cfg, g.d_band_tasks + t0, cnt, g.Lx, H, 0, group_sched(L, g), 2, false,
                                             g.seed, 0, buf, L->d_call, L->pa, false, st);
                 }, t2);
