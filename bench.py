@@ -665,7 +665,7 @@ def profile_case(name):
         lat.label_domains(0, 64)
     elif name in ("strip1024", "band2-1024"):
         # 128 lattices of 1024^2 (1.07 GB of state in both halves of the double
-        # buffer), 32 steps with one or two steps per launch (32-row bands for
+        # buffer), 32 steps with one or two steps per launch (64-row bands for
         # two); four concurrent slices of 32 lattices, each launch several waves
         lat = Lattice([Config(Lx=1024, Ly=1024, n_replicas=128, seed=1, init_mode=1, knots=((0,), (TC,)),
                               n_total=10 ** 6)])

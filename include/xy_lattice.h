@@ -264,6 +264,8 @@ int xy_set_coupling_schedule(xy_lattice* lat, int cfg, const int64_t* step_knots
  *          batches, which it does not time, take two;
  *   kt = 1: one step per launch everywhere;
  *   kt = 2: two steps per launch wherever the shape allows.
+ * Where a call's launches of pairs would be odd in number its last pair goes as
+ * two single steps, which saves copying the state back to the caller's buffers.
  * XY_EINVAL for any other value. */
 int xy_set_temporal_blocking(xy_lattice* lat, int kt);
 

@@ -17,10 +17,10 @@ namespace xy {
 // The four sites of a quad as two pairs (0, 1), (2, 3).  sm_103a issues one
 // FP32 instruction for a pair (fma.rn.f32x2 and its add and mul), each half
 // rounded like the scalar instruction, so a pair costs one issue slot and the
-// bits are those of the scalar code.  The steppers are bound by the issue rate
-// (82 instructions per site-update in the one-step strip kernel, 74 in the
-// two-step band kernel, at 67-71 % of the issue slots), and a third of their
-// instructions were FP32 adds and multiplies of whole quads.
+// bits are those of the scalar code.  The steppers are bound by the issue of
+// instructions, a third of which were FP32 adds and multiplies of whole quads: 82 per
+// site-update in the one-step strip kernel and 70 in the first two-step kernel, 68
+// and 44 now (the band kernel, at 58 % of the issue slots).
 // -------------------------------------------------------------------------
 struct P4 {
     float2 a, b;

@@ -694,16 +694,16 @@ cudaError_t launch_strip_step(const DevCfg* d_cfg, const StripTask* tasks, int n
 // floor(32 / (Lx / 4)) bands, one per lane group, and warps are independent.
 //
 // What bounds it: the issue slots that dependent instructions leave empty.  A
-// site-update takes about 49 instructions (10 of Philox, 5 on the special-function
-// unit), 57 % of the issue slots at 16 warps per SM (128 registers; 20 warps at
-// 96 registers gained 2 %, less than what they spilled), and 8 bytes, 60 % of the
-// copy bandwidth.  So: rows rotate through three register sets (the loop is
+// site-update takes about 44 instructions in bands of 64 rows (10 of Philox, 5 on the
+// special-function unit), 58 % of the issue slots at 16 warps per SM (128 registers;
+// 20 warps at 96 registers gained 2 %, less than what they spilled), and 8 bytes, 60 %
+// of the copy bandwidth.  So: rows rotate through three register sets (the loop is
 // unrolled by three, no copies), each of the two updates has the other one's
 // noise to interleave with, neighbours come from shared memory, and the first
 // iterations, which have no level 1 or 2 row yet, are peeled.  Measured on
 // 3.4e7 sites at 2070 MHz, one step per launch (strip kernel) against two:
 // 256 x 256 4.02e11 -> 5.1e11 site-updates/s, 1024 x 1024 4.13e11 -> 4.8e11,
-// 2048 x 2048 4.13e11 -> 4.8e11.
+// 2048 x 2048 4.13e11 -> 4.7e11.
 namespace {
 
 constexpr int kBStages = 3;
