@@ -1186,7 +1186,11 @@ int autotune_lattice(xy_lattice* L)
                 }
             }
             if (rc) break;
-            pair = best2 / 2 < t1 ? 1 : 0;
+            // single steps must gain 5 %: candidates read the same buffers at every launch,
+            // which flatters short ones, and pairs are also what steps that record take
+            // best (64 x 2048 x 16, 100 steps: singles, chosen by the bare times, 0.78 ms and
+            // 1.46 with a record each; pairs 0.75 and 1.16)
+            pair = best2 / 2 < 1.05f * t1 ? 1 : 0;
             g_tune.put(key2, h2, pair);
         }
         g.kt2_auto = pair != 0;
